@@ -399,7 +399,7 @@ int kscf_selftest_eig_barrier_timeout(void* stream);
  *          Rayleigh-Ritz]; rho; V_H; V_xc; SRE and energies; mixing unless converged.
  * The kscf_scf handle borrows the Hamiltonian (it rewrites its potential) and the
  * caller's X; both must outlive it.  It owns every other buffer (device memory about
- * (14 + 2 history) * n_slots doubles plus the CheFSI work buffers).  All calls are
+ * (15 + 2 history) * n_slots doubles plus the CheFSI work buffers).  All calls are
  * synchronous (they read Ritz values and reductions on the host). */
 typedef struct kscf_scf kscf_scf;
 

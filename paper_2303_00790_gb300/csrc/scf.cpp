@@ -39,8 +39,11 @@ struct kscf_scf {
   double sre_prev = 0.0;      // SRE of the previous step (Ry), 0 before the first
   double* part = nullptr;     // kScfRedBlocks x 44 partial sums
   double* part_bb = nullptr;  // kScfRedBlocks
-  double* part_rr[2] = {nullptr, nullptr};
-  double* part_pq = nullptr;
+  double* part_rr = nullptr;  // kScfRedBlocks
+  double* part_cg = nullptr;  // 2 kScfRedBlocks
+  uint32_t* cg_max = nullptr; // 2 kScfRedBlocks
+  void* cg_rf = nullptr;      // n x 2 int32: the CG residual in fixed point
+  unsigned* cg_sync = nullptr;  // barrier counter and status
   double* small = nullptr;    // 128 doubles of reduction results
   int* d_iters = nullptr;
   double* part_col = nullptr; // kScfRedBlocks x k partial column sums
@@ -69,13 +72,14 @@ namespace {
 constexpr int kMom = 0;      // 10 multipole sums
 constexpr int kRes = 16;     // 5 residual / energy sums
 constexpr int kGram = 32;    // 44 Anderson sums
-constexpr int kCg = 96;      // r.r, b.b
+constexpr int kCg = 96;      // r.r, b.b, beta
+constexpr int kCgLaunchIters = 1024;
 
 void free_scf(kscf_scf* S) {
   void* dev[] = {S->rel,    S->atoms,  S->v_ion,  S->v_start, S->v_in,       S->rho,        S->vh,
                  S->vxc,    S->eps,    S->f,      S->cg_b,    S->cg_r,       S->cg_p,       S->cg_q,
-                 S->v_prev, S->f_prev, S->dv,     S->df,      S->part,       S->part_bb,    S->part_rr[0],
-                 S->part_rr[1], S->part_pq, S->small, S->d_iters, S->P.d_grel, S->P.d_vghost, S->P.d_gptr,
+                 S->v_prev, S->f_prev, S->dv,     S->df,      S->part,       S->part_bb,    S->part_rr,
+                 S->part_cg, S->cg_max, S->cg_rf, S->cg_sync, S->small, S->d_iters, S->P.d_grel, S->P.d_vghost, S->P.d_gptr,
                  S->P.d_gidx, S->P.d_gw, S->work, S->part_col, S->colsq, S->d_occ,
                  S->pf, S->pf_prev, S->dpf, S->ku, S->hx};
   for (void* q : dev)
@@ -160,13 +164,6 @@ int sync_read(kscf_scf* S, const double* src, int count, double* dst) {
   return KSCF_OK;
 }
 
-int read_iters(kscf_scf* S, int* it) {
-  KSCF_CUDA_TRY(cudaMemcpyAsync(S->host, S->d_iters, sizeof(int), cudaMemcpyDeviceToHost, S->st));
-  KSCF_CUDA_TRY(cudaStreamSynchronize(S->st));
-  std::memcpy(it, S->host, sizeof(int));
-  return KSCF_OK;
-}
-
 // CG on (-Lap_h + shift) x = b for the right-hand side already in S->cg_b (its partial
 // squares in S->part_bb), from the guess in x.
 int cg_solve(kscf_scf* S, double shift, double* x, int* iters_out, const char* what) {
@@ -174,11 +171,10 @@ int cg_solve(kscf_scf* S, double shift, double* x, int* iters_out, const char* w
   cudaStream_t st = S->st;
   KSCF_CUDA_TRY(launch_mask_v(H, x, x, st));
   KSCF_CUDA_TRY(cudaMemsetAsync(S->d_iters, 0, sizeof(int), st));
-  int cur = 0;
-  KSCF_CUDA_TRY(launch_cg_init(H, shift, x, S->cg_b, S->cg_r, S->cg_p, S->part_rr[cur], st));
+  KSCF_CUDA_TRY(launch_cg_init(H, shift, x, S->cg_b, S->cg_r, S->cg_p, S->part_rr, st));
   const double rtol = S->p.poisson_rtol;
   double cg[2];
-  KSCF_CUDA_TRY(launch_finalize_partials(S->part_rr[cur], kScfRedBlocks, 1, S->small + kCg, st));
+  KSCF_CUDA_TRY(launch_finalize_partials(S->part_rr, kScfRedBlocks, 1, S->small + kCg, st));
   KSCF_CUDA_TRY(launch_finalize_partials(S->part_bb, kScfRedBlocks, 1, S->small + kCg + 1, st));
   int rc = sync_read(S, S->small + kCg, 2, cg);
   if (rc) return rc;
@@ -191,35 +187,45 @@ int cg_solve(kscf_scf* S, double shift, double* x, int* iters_out, const char* w
     KSCF_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(double) * S->n, st));
     return KSCF_OK;
   }
-  int launched = 0;
-  const int batch = 16;
+  // launches of at most kCgLaunchIters iterations; the cap is poisson_maxiter in whole
+  // batches of 16
+  const CgWork w = {S->cg_r, S->cg_p, S->cg_q, S->cg_rf, S->part_bb, S->part_cg, S->cg_max, S->small + kCg,
+                    S->d_iters, S->cg_sync};
+  const int64_t cap = ((int64_t)S->p.poisson_maxiter + 15) / 16 * 16;
+  const double* rr_in = S->part_rr;
+  int n_rr = kScfRedBlocks, it = 0;
+  int64_t launched = 0;
   while (!(cg[0] < rtol * rtol * cg[1])) {
-    if (launched >= S->p.poisson_maxiter) {
-      int it = 0;
-      rc = read_iters(S, &it);
-      if (rc) return rc;
+    if (launched >= cap) {
       if (iters_out) *iters_out = it;
       set_error("kscf_scf: %s CG not converged after %d iterations (|r|/|b| = %.3e)", what, it,
                 std::sqrt(cg[0] / cg[1]));
       return KSCF_ERR_NO_CONVERGE;
     }
-    for (int i = 0; i < batch; i++) {
-      KSCF_CUDA_TRY(launch_cg_iteration(H, shift, S->part_bb, rtol, x, S->cg_r, S->cg_p, S->cg_q, S->part_rr[cur],
-                                        S->part_pq, S->part_rr[cur ^ 1], S->d_iters, st));
-      cur ^= 1;
-    }
+    const int batch = (int)std::min<int64_t>(cap - launched, kCgLaunchIters);
+    KSCF_CUDA_TRY(launch_cg(H, shift, w, rtol, x, rr_in, n_rr, launched == 0, batch, st));
     launched += batch;
-    KSCF_CUDA_TRY(launch_finalize_partials(S->part_rr[cur], kScfRedBlocks, 1, S->small + kCg, st));
-    rc = sync_read(S, S->small + kCg, 1, cg);
-    if (rc) return rc;
+    // one read: r.r and b.b, the iteration count, the barrier status
+    double* h = S->host;
+    KSCF_CUDA_TRY(cudaMemcpyAsync(h, S->small + kCg, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    KSCF_CUDA_TRY(cudaMemcpyAsync(h + 2, S->d_iters, sizeof(int), cudaMemcpyDeviceToHost, st));
+    KSCF_CUDA_TRY(cudaMemcpyAsync(h + 3, S->cg_sync, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    KSCF_CUDA_TRY(cudaStreamSynchronize(st));
+    unsigned sync[2];
+    std::memcpy(cg, h, sizeof(cg));
+    std::memcpy(&it, h + 2, sizeof(it));
+    std::memcpy(sync, h + 3, sizeof(sync));
+    if (sync[1] != 0) {
+      set_error("kscf_scf: a bounded grid barrier of the %s CG gave up", what);
+      return KSCF_ERR_TIMEOUT;
+    }
     if (!std::isfinite(cg[0])) {
       set_error("kscf_scf: %s CG produced a non-finite residual", what);
       return KSCF_ERR_NONFINITE;
     }
+    rr_in = S->small + kCg;
+    n_rr = 1;
   }
-  int it = 0;
-  rc = read_iters(S, &it);
-  if (rc) return rc;
   if (iters_out) *iters_out = it;
   return KSCF_OK;
 }
@@ -490,9 +496,12 @@ extern "C" int kscf_scf_create(kscf_ham* ham, const kscf_atom* atoms, int n_atom
     if (e == cudaSuccess) e = dalloc(&S->atoms, at.size());
     if (e == cudaSuccess) e = dalloc(&S->part, (size_t)kScfRedBlocks * 48);
     if (e == cudaSuccess) e = dalloc(&S->part_bb, (size_t)kScfRedBlocks);
-    if (e == cudaSuccess) e = dalloc(&S->part_rr[0], (size_t)kScfRedBlocks);
-    if (e == cudaSuccess) e = dalloc(&S->part_rr[1], (size_t)kScfRedBlocks);
-    if (e == cudaSuccess) e = dalloc(&S->part_pq, (size_t)kScfRedBlocks);
+    if (e == cudaSuccess) e = dalloc(&S->part_rr, (size_t)kScfRedBlocks);
+    if (e == cudaSuccess) e = dalloc(&S->part_cg, 2 * (size_t)kScfRedBlocks);
+    if (e == cudaSuccess) e = dalloc(&S->cg_max, 2 * (size_t)kScfRedBlocks);
+    if (e == cudaSuccess) e = dalloc(&S->cg_sync, 2);
+    if (e == cudaSuccess) e = cudaMalloc(&S->cg_rf, 8 * ((size_t)n + kCgZeroSlots));
+    if (e == cudaSuccess) e = cudaMemsetAsync(S->cg_rf, 0, 8 * ((size_t)n + kCgZeroSlots), S->st);
     if (e == cudaSuccess) e = dalloc(&S->small, 128);
     if (e == cudaSuccess) e = dalloc(&S->d_iters, 1);
     if (e == cudaSuccess) e = dalloc(&S->part_col, (size_t)kScfRedBlocks * p.k);

@@ -40,10 +40,25 @@ cudaError_t launch_poisson_rhs(const Ham& H, const double* rho, const PoissonPla
 // CG on A x = b with A = -Lap_h + shift (zero outside the domain)
 cudaError_t launch_cg_init(const Ham& H, double shift, double* x, const double* b, double* r, double* p,
                            double* part_rr, cudaStream_t st);
-// one CG iteration (three kernels); every kernel returns at once when r.r < rtol^2 b.b
-cudaError_t launch_cg_iteration(const Ham& H, double shift, const double* part_bb, double rtol, double* x, double* r,
-                                double* p, double* q, const double* part_rr, double* part_pq, double* part_rr_next,
-                                int* iters, cudaStream_t st);
+// Buffers of the CG: r, p, q (n_slots doubles), r in fixed point (n_slots + kCgZeroSlots x 2
+// int32, zero in padding slots and behind the field), partial sums of b.b, 2 kScfRedBlocks partial sums and maxima, and small
+// words: state (r.r, b.b, beta), the iteration count, sync (barrier counter, timeout status).
+constexpr int kCgZeroSlots = 4096;   // 6 planes of a 16^3 brick each way from the middle
+struct CgWork {
+  double *r, *p, *q;
+  void* rf;
+  const double* part_bb;
+  double* part;
+  uint32_t* hmax;
+  double* state;
+  int* iters;
+  unsigned* sync;
+};
+// up to max_iters CG iterations in one launch, from x, w.r and the partial sums rr_in of r.r
+// (first), or continuing the previous launch (rr_in = w.state, n_rr = 1); ends when r.r < rtol^2 b.b or r.r is not finite.  w.state and *w.iters (added to) and
+// w.sync[1] (1: a bounded grid barrier gave up) are read back by the caller.
+cudaError_t launch_cg(const Ham& H, double shift, const CgWork& w, double rtol, double* x, const double* rr_in,
+                      int n_rr, bool first, int max_iters, cudaStream_t st);
 // b = f on the domain, partial b.b
 cudaError_t launch_rhs_copy(const Ham& H, const double* f, double* b, double* part_bb, cudaStream_t st);
 // out = a + c b on the domain

@@ -11,6 +11,9 @@
 // sum per value, and consumers add the partials in a fixed order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
+#include "fixlap.cuh"
 #include "kscf_internal.h"
 #include "scf_internal.h"
 
@@ -192,18 +195,6 @@ __device__ __forceinline__ double lap_at(const LapArgs& a, const double* __restr
   return acc;
 }
 
-// Convergence state of the CG, read by every kernel from the partial sums:
-// rr = r.r of the current residual, converged when rr < thr2 = rtol^2 b.b.
-struct CgState {
-  const double* part_bb;  // kScfRedBlocks partials of b.b
-  double rtol2;
-};
-
-__device__ __forceinline__ bool cg_done(const CgState& c, double rr) {
-  const double bb = warp_sum_partials(c.part_bb, kScfRedBlocks);
-  return rr < c.rtol2 * bb;
-}
-
 // b = 4 pi rho + sum over the ghost points g of the slot: w_g V_ghost[g]; partial b.b
 __global__ void __launch_bounds__(kScfThreads) poisson_rhs_kernel(const double* __restrict__ rho,
                                                                   const uint8_t* __restrict__ mask,
@@ -241,63 +232,344 @@ __global__ void __launch_bounds__(kScfThreads) cg_init_kernel(LapArgs a, double*
   block_partials<1>(acc, part_rr);
 }
 
-// q = A p, partial p.q   (no-op once converged)
-template <int B>
-__global__ void __launch_bounds__(kScfThreads) cg_apply_kernel(LapArgs a, CgState c, const double* __restrict__ p,
-                                                               double* __restrict__ q,
-                                                               const double* __restrict__ part_rr,
-                                                               double* __restrict__ part_pq) {
-  const double rr = warp_sum_partials(part_rr, kScfRedBlocks);
-  if (cg_done(c, rr)) return;
-  double acc[1] = {0.0};
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.n; s += (int64_t)gridDim.x * blockDim.x) {
-    double qv = 0.0;
-    if (a.mask[s]) {
-      qv = lap_at<B>(a, p, s);
-      acc[0] += p[s] * qv;
+// ---------------------------------------------------------------------------
+// The conjugate gradients in one cooperative launch (one CTA per SM, the domain points in
+// contiguous shares, two bounded grid barriers per iteration):
+//   q = A r + beta q, p = r + beta p, p.q | x += alpha p, r -= alpha q, r.r
+// (q = A p by the recurrence of Chronopoulos & Gear 1989, so that the only neighbour values
+// read are those of r, which are ready at the barrier of r.r.)  A r reads r as 58-bit fixed
+// point (fixlap.cuh), whose exponent comes from max|r| and max|q| of the reductions before.
+// What bounds an iteration: the barriers (~1.5 us each with their skew), the FP64 chains of
+// the two reductions (only one warp of a CTA adds the other CTAs' partial sums) and 10 FP64
+// instructions per point (64 cycles per warp each).  Up to 4 points per thread the vectors
+// stay in registers; larger grids (NPT = 0) keep them in global memory.  Three launches per
+// iteration with the star in FP64 and every warp adding the 304 partials two or three times
+// took 89 us at 234,489 points and 67 us at 45,025; this kernel takes 15.6 us and 9.1 us (Hartree
+// solve of the 2.2 nm cluster, 368 iterations: 32.7 -> 5.75 ms).
+constexpr int kCgThreads = 512;   // most threads of a CTA
+
+struct CgArgs {
+  LapArgs a;
+  const int32_t* live;      // domain slots
+  int64_t n_live;
+  double lap_unit;          // -1 / (831600 h^2)
+  double *x, *r, *p, *q;
+  int2* rf;                 // r in fixed point, zero in padding slots
+  const double* rr_in;      // partial sums of r.r at entry
+  int n_rr;
+  const double* part_bb;
+  int n_bb;
+  double rtol2;
+  double* part;             // 2 x grid partial sums: p.q, r.r
+  uint32_t* hmax;           // 2 x grid maxima of the high words of |q|, |r|
+  double* state;            // out: r.r, b.b, beta (in unless first)
+  int* iters;               // += iterations done
+  unsigned* bar;            // arrival counter, zero at launch
+  int* status;              // 1: a barrier wait gave up
+  long long spin_limit;
+  int max_iters;
+  int first;                // p, q start from zero
+};
+
+// Grid barrier as in the eigensolver's tridiagonalisation: release arrivals on a monotonic
+// counter, acquire polls, bounded by spin_limit clock cycles.
+__device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.bar) : "memory");
+    int ok = 1;
+    const long long t0 = clock64();
+    for (;;) {
+      unsigned n;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(c.bar) : "memory");
+      if (n >= target) break;
+      if (*(volatile int*)c.status != 0 || clock64() - t0 > c.spin_limit) {
+        atomicExch(c.status, 1);
+        ok = 0;
+        break;
+      }
     }
-    q[s] = qv;
+    *s_ok = ok;
   }
-  block_partials<1>(acc, part_pq);
+  __syncthreads();
+  return *s_ok != 0;
 }
 
-// alpha = rr / p.q; x += alpha p; r -= alpha q; partial of the new r.r
-// (once converged: carries the partials of rr forward unchanged)
-__global__ void __launch_bounds__(kScfThreads) cg_update_kernel(CgState c, int64_t n, double* __restrict__ x,
-                                                                double* __restrict__ r, const double* __restrict__ p,
-                                                                const double* __restrict__ q,
-                                                                const double* __restrict__ part_rr,
-                                                                const double* __restrict__ part_pq,
-                                                                double* __restrict__ part_rr_next, int* iters) {
-  const double rr = warp_sum_partials(part_rr, kScfRedBlocks);
-  if (cg_done(c, rr)) {
-    if (threadIdx.x == 0) part_rr_next[blockIdx.x] = part_rr[blockIdx.x];
-    return;
+// CTA sum of v and maximum of m into *sum and *mx (global, thread 0).  The first four warps,
+// one per SM sub-partition, add the other warps' values, so that the FP64 adds (64 cycles
+// per warp) number 9 in a row instead of 5 in every warp and 16 more.  sh: kCgThreads, zero
+// beyond the CTA's threads (at least 128).
+__device__ __forceinline__ void cg_reduce(double v, uint32_t m, double* sh, double* sh4, uint32_t* shm, double* sum,
+                                          uint32_t* mx) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  sh[tid] = v;
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) shm[warp] = m;
+  __syncthreads();
+  if (warp < 4) {
+    double s = (sh[tid] + sh[tid + 128]) + (sh[tid + 256] + sh[tid + 384]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sh4[warp] = s;
   }
-  const double pq = warp_sum_partials(part_pq, kScfRedBlocks);
-  const double alpha = rr / pq;
-  double acc[1] = {0.0};
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    x[s] += alpha * p[s];
-    const double rv = r[s] - alpha * q[s];
-    r[s] = rv;
-    acc[0] += rv * rv;
+  __syncthreads();
+  if (tid == 0) {
+    *sum = (sh4[0] + sh4[1]) + (sh4[2] + sh4[3]);
+    uint32_t t = shm[0];
+    for (int w = 1; w < (int)(blockDim.x >> 5); w++) t = max(t, shm[w]);
+    *mx = t;
   }
-  block_partials<1>(acc, part_rr_next);
-  if (blockIdx.x == 0 && threadIdx.x == 0) iters[0] += 1;
 }
 
-// beta = rr_new / rr; p = r + beta p
-__global__ void __launch_bounds__(kScfThreads) cg_dir_kernel(CgState c, int64_t n, const double* __restrict__ r,
-                                                             double* __restrict__ p,
-                                                             const double* __restrict__ part_rr,
-                                                             const double* __restrict__ part_rr_next) {
-  const double rr = warp_sum_partials(part_rr, kScfRedBlocks);
-  if (cg_done(c, rr)) return;
-  const double rr_new = warp_sum_partials(part_rr_next, kScfRedBlocks);
-  const double beta = rr_new / rr;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
-    p[s] = r[s] + beta * p[s];
+// Sum of part[0..P) and maximum of mx[0..P) in one warp; the loads are issued together.
+__device__ __forceinline__ double cg_collect(const double* part, const uint32_t* mx, int P, uint32_t* m_out) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  uint32_t m = 0;
+  for (int b0 = lane; b0 < P; b0 += 160) {
+    double v[5];
+    uint32_t u[5];
+#pragma unroll
+    for (int q = 0; q < 5; q++) {
+      const int b = b0 + 32 * q;
+      v[q] = b < P ? __ldcg(part + b) : 0.0;
+      u[q] = b < P ? __ldcg(mx + b) : 0u;
+    }
+    s += ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+#pragma unroll
+    for (int q = 0; q < 5; q++) m = max(m, u[q]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  *m_out = __reduce_max_sync(0xffffffffu, m);
+  return s;
+}
+
+// A double at least every double whose high word (sign cleared) is hw
+__device__ __forceinline__ double hw_bound(uint32_t hw) { return __hiloint2double((int)min(hw + 1, 0x7ff00000u), 0); }
+__device__ __forceinline__ uint32_t abs_hw(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
+
+// Byte offsets (in the fixed-point field) of the face neighbours of slot s: nb[2 ax + sg] +-
+// 8 k stride is the slot at distance k beyond the brick's face.  A missing brick points into
+// the zeros behind the field (kCgZeroSlots), so that the star needs no predicates; 32-bit
+// offsets from one base keep the address arithmetic out of the loads.
+template <int B>
+__device__ __forceinline__ void cg_faces(const int32_t* nbr, int s, uint32_t zero, uint32_t* nb) {
+  constexpr int B3 = B * B * B;
+  const int brick = s / B3, li = s - brick * B3;
+  const int stride[3] = {1, B, B * B};
+#pragma unroll
+  for (int f = 0; f < 6; f++) {
+    const int n = __ldg(nbr + brick * 6 + f);
+    nb[f] = n >= 0 ? 8u * (uint32_t)(n * B3 + li + ((f & 1) ? -B : B) * stride[f >> 1]) : zero;
+  }
+}
+
+// 831600 h^2 Lap_h of the fixed-point field f at slot s
+template <int B>
+__device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* nb, int nbs) {
+  const int li = s & (B * B * B - 1);
+  const int l[3] = {li % B, (li / B) % B, li / (B * B)};
+  const int stride[3] = {1, B, B * B};
+  const uint32_t own = 8u * (uint32_t)s;
+  FixAcc acc = {0, 0};
+  fix_mad(acc, FIX_W0, *(const int2*)(f + own));
+  uint32_t face[6];
+#pragma unroll
+  for (int q = 0; q < 6; q++) face[q] = nb[q * nbs];
+#pragma unroll
+  for (int k = 1; k <= 6; k++) {
+    int2 v[6];
+#pragma unroll
+    for (int ax = 0; ax < 3; ax++) {
+      const uint32_t lo = l[ax] >= k ? own : face[2 * ax], hi = l[ax] + k < B ? own : face[2 * ax + 1];
+      v[2 * ax] = *(const int2*)(f + (size_t)lo - 8 * k * stride[ax]);
+      v[2 * ax + 1] = *(const int2*)(f + (size_t)hi + 8 * k * stride[ax]);
+    }
+    fix_mad(acc, FIX_W[k - 1], make_int2((v[0].x + v[1].x + v[2].x) + (v[3].x + v[4].x + v[5].x),
+                                         (v[0].y + v[1].y + v[2].y) + (v[3].y + v[4].y + v[5].y)));
+  }
+  return acc;
+}
+
+template <int B, int NPT>
+__global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
+  extern __shared__ uint32_t s_face[];   // NPT > 0: [6][NPT][threads] face neighbours of the points
+  __shared__ double sh[kCgThreads], sh4[4];
+  __shared__ uint32_t shm[kCgThreads / 32];
+  __shared__ double s_val[2];
+  __shared__ uint32_t s_max;
+  __shared__ int s_ok;
+  const int tid = threadIdx.x, nt = blockDim.x, warp = tid >> 5, lane = tid & 31, P = gridDim.x, cta = blockIdx.x;
+  const int64_t per = (c.n_live + P - 1) / P;
+  const int64_t i0 = cta * per, i1 = min(c.n_live, i0 + per);
+  double* part_pq = c.part;
+  double* part_rr = c.part + P;
+  uint32_t* max_q = c.hmax;
+  uint32_t* max_r = c.hmax + P;
+  unsigned target = 0;
+  for (int t = tid; t < kCgThreads; t += nt) sh[t] = 0.0;
+  const uint32_t zero = 8u * (uint32_t)(c.a.n + kCgZeroSlots / 2);
+  constexpr int NR = NPT > 0 ? NPT : 1;
+  int sv[NR];
+  double xv[NR], rv[NR], pv[NR], qv[NR];
+  // f(point number k of the thread, slot, x, r, p, q) over the thread's points; the vectors
+  // are registers or global memory.  With registers a thread without a k-th point works on a
+  // zero point behind the field (all its values stay zero), so that the points interleave
+  // without branches.
+  auto each = [&](auto f) {
+    if constexpr (NPT > 0) {
+#pragma unroll
+      for (int k = 0; k < NPT; k++) f(k, sv[k], xv[k], rv[k], pv[k], qv[k]);
+    } else {
+      for (int64_t i = i0 + tid; i < i1; i += nt) {
+        const int s = c.live[i];
+        f(0, s, c.x[s], c.r[s], c.p[s], c.q[s]);
+      }
+    }
+  };
+  if constexpr (NPT > 0) {
+#pragma unroll
+    for (int k = 0; k < NPT; k++) {
+      const int64_t i = i0 + tid + (int64_t)k * nt;
+      const bool on = i < i1;
+      sv[k] = on ? c.live[i] : (int)(zero / 8);
+      uint32_t nb[6];
+      if (on) cg_faces<B>(c.a.nbr, sv[k], zero, nb);
+#pragma unroll
+      for (int q = 0; q < 6; q++) s_face[(q * NPT + k) * nt + tid] = on ? nb[q] : zero;
+      xv[k] = on ? c.x[sv[k]] : 0.0;
+      rv[k] = on ? c.r[sv[k]] : 0.0;
+      pv[k] = on && !c.first ? c.p[sv[k]] : 0.0;
+      qv[k] = on && !c.first ? c.q[sv[k]] : 0.0;
+    }
+  } else if (c.first) {
+    each([&](int, int, double&, double&, double& p, double& q) { p = q = 0.0; });
+  }
+  // the largest |r|, r.r and b.b at entry, r in fixed point
+  uint32_t mr = 0;
+  each([&](int, int, double&, double& r, double&, double&) { mr = max(mr, abs_hw(r)); });
+  __syncthreads();
+  cg_reduce(0.0, mr, sh, sh4, shm, part_pq + cta, max_r + cta);
+  if (!cg_barrier(c, target += P, &s_ok)) return;
+  if (warp == 0) {
+    const double rr0 = warp_sum_partials(c.rr_in, c.n_rr), bb0 = warp_sum_partials(c.part_bb, c.n_bb);
+    uint32_t m;
+    cg_collect(part_pq, max_r, P, &m);
+    if (lane == 0) {
+      s_val[0] = rr0;
+      s_val[1] = bb0;
+      s_max = m;
+    }
+  }
+  __syncthreads();
+  double rr = s_val[0], beta = c.first ? 0.0 : c.state[2];
+  const double bb = s_val[1];
+  mr = s_max;
+  int e = fix_exp(mr);
+  each([&](int, int s, double&, double& r, double&, double&) { c.rf[s] = fix_from(r, e); });
+  if (!cg_barrier(c, target += P, &s_ok)) return;
+  int it = 0;
+  for (; it < c.max_iters; it++) {
+    if (rr < c.rtol2 * bb || !(rr <= 1.7976931348623157e308)) break;
+    // q = A r + beta q, p = r + beta p, p.q
+    const double sc = c.lap_unit * FIX_SUM_UNIT * fix_unit(e);
+    double acc = 0.0;
+    uint32_t mq = 0;
+    each([&](int k, int s, double&, double& r, double& p, double& q) {
+      FixAcc t;
+      if constexpr (NPT > 0) {
+        t = cg_star<B>((const char*)c.rf, s, s_face + k * nt + tid, NPT * nt);
+      } else {
+        uint32_t nb[6];
+        cg_faces<B>(c.a.nbr, s, zero, nb);
+        t = cg_star<B>((const char*)c.rf, s, nb, 1);
+      }
+      const double pn = fma(beta, p, r);
+      double qn = fma(sc, fix_value(t), beta * q);
+      if (c.a.shift != 0.0) qn = fma(c.a.shift, r, qn);
+      p = pn;
+      q = qn;
+      acc = fma(pn, qn, acc);
+      mq = max(mq, abs_hw(qn));
+    });
+    cg_reduce(acc, mq, sh, sh4, shm, part_pq + cta, max_q + cta);
+    if (!cg_barrier(c, target += P, &s_ok)) return;
+    if (warp == 0) {
+      uint32_t m;
+      const double pq = cg_collect(part_pq, max_q, P, &m);
+      if (lane == 0) {
+        const double alpha = rr / pq;
+        s_val[0] = alpha;
+        // |r - alpha q| <= max|r| + |alpha| max|q|
+        s_max = abs_hw(fma(fabs(alpha), hw_bound(m), hw_bound(mr)));
+      }
+    }
+    __syncthreads();
+    const double alpha = s_val[0];
+    e = fix_exp(s_max);
+    // x += alpha p, r -= alpha q, r.r
+    acc = 0.0;
+    mr = 0;
+    each([&](int, int s, double& x, double& r, double& p, double& q) {
+      const double rn = fma(-alpha, q, r);
+      x = fma(alpha, p, x);
+      r = rn;
+      c.rf[s] = fix_from(rn, e);
+      acc = fma(rn, rn, acc);
+      mr = max(mr, abs_hw(rn));
+    });
+    cg_reduce(acc, mr, sh, sh4, shm, part_rr + cta, max_r + cta);
+    if (!cg_barrier(c, target += P, &s_ok)) return;
+    if (warp == 0) {
+      uint32_t m;
+      const double t = cg_collect(part_rr, max_r, P, &m);
+      if (lane == 0) {
+        s_val[0] = t;
+        s_val[1] = t / rr;
+        s_max = m;
+      }
+    }
+    __syncthreads();
+    rr = s_val[0];
+    beta = s_val[1];
+    mr = s_max;
+  }
+  if constexpr (NPT > 0) {
+#pragma unroll
+    for (int k = 0; k < NPT; k++) {
+      if (i0 + tid + (int64_t)k * nt >= i1) continue;
+      c.x[sv[k]] = xv[k];
+      c.r[sv[k]] = rv[k];
+      c.p[sv[k]] = pv[k];
+      c.q[sv[k]] = qv[k];
+    }
+  }
+  if (cta == 0 && tid == 0) {
+    c.state[0] = rr;
+    c.state[1] = bb;
+    c.state[2] = beta;
+    c.iters[0] += it;
+  }
+}
+
+template <int B>
+static cudaError_t cg_launch(CgArgs& c, int P, cudaStream_t st) {
+  const int64_t per = (c.n_live + P - 1) / P;
+  const int npt = (int)((per + kCgThreads - 1) / kCgThreads);
+  // the fewest threads that hold the share with npt points each, so that the warps are full
+  int nt = npt <= 4 ? (int)(((per + npt - 1) / npt + 31) / 32 * 32) : kCgThreads;
+  nt = std::max(nt, 128);
+  const int smem = npt <= 4 ? 6 * npt * nt * (int)sizeof(int) : 0;
+  const void* k = npt == 1   ? (const void*)cg_kernel<B, 1>
+                  : npt == 2 ? (const void*)cg_kernel<B, 2>
+                  : npt == 3 ? (const void*)cg_kernel<B, 3>
+                  : npt == 4 ? (const void*)cg_kernel<B, 4>
+                             : (const void*)cg_kernel<B, 0>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&c};
+  return cudaLaunchCooperativeKernel(k, dim3(P), dim3(nt), args, smem, st);
 }
 
 static LapArgs lap_args(const Ham& H, double shift) {
@@ -329,22 +601,42 @@ cudaError_t launch_cg_init(const Ham& H, double shift, double* x, const double* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_cg_iteration(const Ham& H, double shift, const double* part_bb, double rtol, double* x, double* r,
-                                double* p, double* q, const double* part_rr, double* part_pq, double* part_rr_next,
-                                int* iters, cudaStream_t st) {
-  const LapArgs a = lap_args(H, shift);
-  CgState c;
-  c.part_bb = part_bb;
+cudaError_t launch_cg(const Ham& H, double shift, const CgWork& w, double rtol, double* x, const double* rr_in,
+                      int n_rr, bool first, int max_iters, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.sync, 0, 2 * sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  CgArgs c;
+  c.a = lap_args(H, shift);
+  c.live = H.d_live;
+  c.n_live = H.n_live;
+  c.lap_unit = -1.0 / (FIX_DEN * H.grid.h * H.grid.h);
+  c.x = x;
+  c.r = w.r;
+  c.p = w.p;
+  c.q = w.q;
+  c.rf = (int2*)w.rf;
+  c.rr_in = rr_in;
+  c.n_rr = n_rr;
+  c.part_bb = w.part_bb;
+  c.n_bb = kScfRedBlocks;
   c.rtol2 = rtol * rtol;
-  const int64_t n = H.grid.n_slots;
-  if (H.grid.B == 8)
-    cg_apply_kernel<8><<<kScfRedBlocks, kScfThreads, 0, st>>>(a, c, p, q, part_rr, part_pq), count_launch();
-  else
-    cg_apply_kernel<16><<<kScfRedBlocks, kScfThreads, 0, st>>>(a, c, p, q, part_rr, part_pq), count_launch();
-  cg_update_kernel<<<kScfRedBlocks, kScfThreads, 0, st>>>(c, n, x, r, p, q, part_rr, part_pq, part_rr_next, iters),
-      count_launch();
-  cg_dir_kernel<<<kScfRedBlocks, kScfThreads, 0, st>>>(c, n, r, p, part_rr, part_rr_next), count_launch();
-  return cudaGetLastError();
+  c.part = w.part;
+  c.hmax = w.hmax;
+  c.state = w.state;
+  c.iters = w.iters;
+  c.bar = w.sync;
+  c.status = (int*)w.sync + 1;
+  c.spin_limit = 2000000000LL;   // ~1 s
+  c.max_iters = max_iters;
+  c.first = first ? 1 : 0;
+  // one CTA per SM; a CTA takes at least 128 points (small grids: fewer CTAs, cheaper barriers)
+  const int P = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(sms, kScfRedBlocks), (H.n_live + 127) / 128));
+  e = H.grid.B == 8 ? cg_launch<8>(c, P, st) : cg_launch<16>(c, P, st);
+  count_launch();
+  return e;
 }
 
 // b = f on the domain (0 outside); partial b.b
