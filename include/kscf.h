@@ -28,7 +28,8 @@
  *   - Inner products use the grid weight h^3: <u, v> = h^3 sum_s u_s v_s.
  *   - Device work buffers must be at least the size kscf_workspace_size() reports for
  *     the same (op, k, dtype, mode, block); a smaller buffer gives KSCF_ERR_WORKSPACE
- *     before any launch.  Work buffers must be 256-byte aligned.
+ *     before any launch (the part for FP64 products on the tensor cores is optional:
+ *     without it they run on the CUDA cores).  Work buffers must be 256-byte aligned.
  */
 #ifndef KSCF_H
 #define KSCF_H
@@ -57,8 +58,11 @@ extern "C" {
 #define KSCF_F32 1
 
 /* ---- Gram / projection GEMM modes (orthonormalize, rayleigh_ritz) ---- */
-#define KSCF_GEMM_NATIVE 0   /* CUDA-core GEMM in the dtype of X; FP32 X: FP32 products with FP64
-                                sums of partial sums over at most 256 rows */
+#define KSCF_GEMM_NATIVE 0   /* products in the dtype of X.  FP32 X: CUDA cores, FP32 products with
+                                FP64 sums of partial sums over at most 256 rows.  FP64 X: exact sums
+                                of 56-bit integer digits on the tensor cores (every value rounded to
+                                2^-56 of its column's or row's bound, one rounding of the result)
+                                when the work buffer has the reported size, else CUDA-core FP64 */
 #define KSCF_GEMM_TENSOR 1   /* tensor cores (tcgen05), F32 X only: every FP32 operand is split into
                                 three bf16 pieces x = x1 + x2 + x3 and the six products x1y1, x1y2,
                                 x2y1, x1y3, x2y2, x3y1 are accumulated in FP32 over chunks of rows,
@@ -256,8 +260,8 @@ int kscf_orthonormalize(const kscf_ham* ham, void* X, int64_t ld, int k, int dty
                         void* work, size_t work_bytes, void* stream);
 
 /* In place Rayleigh-Ritz (CheFSI paragraph): HX = H X, Hs = h^3 X^T (HX) symmetrised
- * (FP64 k x k; in tensor mode with HX computed in one block, only the upper-triangle
- * tiles are computed and mirrored), Hs = Q Lambda Q^T (FP64 symmetric eigensolver,
+ * (FP64 k x k; with HX computed in one block, only the upper-triangle tiles of the
+ * tensor-core products are computed and mirrored), Hs = Q Lambda Q^T (FP64 symmetric eigensolver,
  * ascending), X <- X Q.  In tensor mode the eigenvector signs are chosen with
  * diag(Q) >= 0 and the rotation is applied as X + X (Q - I).  Requires h^3 X^T X = I on
  * entry.  HX is computed in column blocks as wide as the work buffer allows: all k columns
@@ -310,7 +314,8 @@ int kscf_random_subspace(const kscf_ham* ham, void* X, int64_t ld, int k, int dt
  *   reads bf16 copies of A; minus_identity adds A's own element in the epilogue); in the
  *   native mode out must not overlap A.
  * Work buffers: kscf_gemm_workspace_size(op = 0 gram / 1 rotate, rows, m|kin, n|kout,
- * dtype, mode, &bytes). */
+ * dtype, mode, &bytes).  In the native mode a Gram needs none and a rotation kin * kout
+ * elements; FP64 products use the rest of the reported size for the tensor cores. */
 int kscf_gram(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t rows, int m, int n, int dtype,
               int mode, double scale, double* C, int64_t ldc, void* work, size_t work_bytes, void* stream);
 int kscf_rotate(const void* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin, int kout,

@@ -48,10 +48,11 @@ int eig_info_code(const int* info, const char* who) {
 }
 
 // after a synchronisation: did a tensor-core pipeline wait time out?
-int check_tc(int mode, const char* who) {
-  if (mode != KSCF_GEMM_TENSOR) return KSCF_OK;
+// (f64tc: FP64 products ran on the tensor cores)
+int check_tc(int mode, bool f64tc, const char* who) {
+  if (mode != KSCF_GEMM_TENSOR && !f64tc) return KSCF_OK;
   unsigned int st = 0;
-  cudaError_t e = tc_status(true, &st);
+  cudaError_t e = f64tc ? f64tc_status(true, &st) : tc_status(true, &st);
   if (e != cudaSuccess) {
     set_error("%s: reading the tensor-core status failed: %s", who, cudaGetErrorString(e));
     return KSCF_ERR_CUDA;
@@ -102,8 +103,17 @@ int64_t panel_rows(int64_t n_slots, int k, int dtype) {
   return std::min<int64_t>(r, n_slots);
 }
 
+// Work bytes of the FP64 products on the tensor cores: k columns, row panels of prows in the
+// rotation, a Gram of k x w.  They come last in the work buffer and are optional: a buffer
+// without them runs the CUDA-core products.
+size_t f64tc_bytes(const Ham& H, int k, int w, int64_t prows) {
+  const size_t g = gram_f64tc_wanted(H.n_live) ? gram_f64tc_work_bytes(H.n_live, k, w) : 0;
+  const size_t r = rotate_f64tc_wanted(H.n_live, k, k) ? rotate_f64tc_work_bytes(std::min(prows, H.n_live), k, k) : 0;
+  return kscf_align256(std::max(g, r));
+}
+
 struct OrthoPlan {
-  size_t S, Rinv, info, chol, panel, tc;
+  size_t S, Rinv, info, chol, panel, tc, tc64;
   int64_t prows;
 };
 
@@ -117,16 +127,18 @@ int ortho_plan(const Ham& H, int k, int dtype, int mode, OrthoPlan* p) {
   p->tc = 0;
   if (mode == KSCF_GEMM_TENSOR)
     p->tc = std::max(gram_tc_work_bytes(H.grid.n_slots, k, k), rotate_tc_work_bytes(p->prows, k, k));
+  p->tc64 = dtype == KSCF_F64 ? f64tc_bytes(H, k, k, p->prows) : 0;
   return KSCF_OK;
 }
 
+// without the optional tc64
 size_t ortho_bytes(const OrthoPlan& p) {
   return kscf_align256(p.S) + kscf_align256(p.Rinv) + kscf_align256(p.info) + kscf_align256(p.chol) +
          kscf_align256(p.panel) + kscf_align256(p.tc);
 }
 
 struct RRPlan {
-  size_t hxb, coef, Hs, W, Q, info, lwork_bytes, panel, tc;
+  size_t hxb, coef, Hs, W, Q, info, lwork_bytes, panel, tc, tc64;
   int64_t prows;
   int w;
 };
@@ -149,9 +161,11 @@ int rr_plan(const Ham& H, int k, int dtype, int mode, int block, RRPlan* p) {
   p->tc = 0;
   if (mode == KSCF_GEMM_TENSOR)
     p->tc = std::max(gram_tc_work_bytes(H.grid.n_slots, k, p->w), rotate_tc_work_bytes(p->prows, k, k));
+  p->tc64 = dtype == KSCF_F64 ? f64tc_bytes(H, k, p->w, p->prows) : 0;
   return KSCF_OK;
 }
 
+// without the optional tc64
 size_t rr_bytes(const RRPlan& p) {
   return kscf_align256(p.hxb) + kscf_align256(p.coef) + kscf_align256(p.Hs) + kscf_align256(p.W) +
          kscf_align256(p.Q) + kscf_align256(p.info) + kscf_align256(p.lwork_bytes) + kscf_align256(p.panel) +
@@ -207,45 +221,61 @@ int check_mode(int dtype, int mode, const char* who) {
   return KSCF_OK;
 }
 
+// Work buffer of the products: for the tensor mode or, with gram64 / rot64, for FP64 products
+// on the tensor cores.
+struct GemmWork {
+  void* buf;
+  size_t bytes;
+  bool gram64, rot64;
+};
+GemmWork gemm_work(const Ham& H, int k, void* buf, size_t bytes, bool f64tc) {
+  return {buf, bytes, f64tc && gram_f64tc_wanted(H.n_live), f64tc && rotate_f64tc_wanted(H.n_live, k, k)};
+}
+
 // X <- X Qm (Qm column-major k x k in the dtype of X for the native path, FP64 for the
-// tensor path) in row panels.  The tensor path writes each panel in place (its product
-// reads the panel's bf16 pieces, made before the launch); the native path goes through
-// the panel buffer.
+// tensor path) in row panels.  The tensor paths write each panel in place (their products
+// read the panel's bf16 pieces, made before the launch); the native path goes through
+// the panel buffer.  upper: Qm is upper triangular.  With gw.gram64 gw.buf still holds what the
+// Gram with X as its first operand left there (its column maxima are used).
 int rotate_inplace(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, const void* Qm,
-                   const double* Q64, bool near_identity, void* panel, int64_t prows, void* tcwork, size_t tcbytes,
+                   const double* Q64, bool near_identity, bool upper, void* panel, int64_t prows, const GemmWork& gw,
                    cudaStream_t st) {
   const size_t es = esize(dtype);
-  // the tensor path rotates the domain rows only (through the grid's list of domain slots)
-  const bool live = mode == KSCF_GEMM_TENSOR && H.d_live;
+  // the tensor paths rotate the domain rows only (through the grid's list of domain slots)
+  const bool live = (mode == KSCF_GEMM_TENSOR || gw.rot64) && H.d_live;
   const int64_t rows = live ? H.n_live : H.grid.n_slots;
   for (int64_t r0 = 0; r0 < rows; r0 += prows) {
     const int64_t nr = std::min(prows, rows - r0);
-    char* Xr = (char*)X + (size_t)r0 * ld * es;
+    char* Xr = live ? (char*)X : (char*)X + (size_t)r0 * ld * es;
+    const int32_t* map = live ? H.d_live + r0 : nullptr;
     if (mode == KSCF_GEMM_TENSOR) {
-      if (live)
-        KSCF_CUDA_TRY(launch_rotate_tc((const float*)X, ld, Q64, k, nr, k, k, near_identity, (float*)X, ld, tcwork,
-                                       tcbytes, st, H.d_live + r0));
-      else
-        KSCF_CUDA_TRY(launch_rotate_tc((const float*)Xr, ld, Q64, k, nr, k, k, near_identity, (float*)Xr, ld, tcwork,
-                                       tcbytes, st));
-    } else {
-      KSCF_CUDA_TRY(launch_rotate_native(Xr, ld, Qm, k, nr, k, k, dtype, panel, k, st));
-      KSCF_CUDA_TRY(launch_copy_cols(panel, k, Xr, ld, nr, k, dtype, st));
+      KSCF_CUDA_TRY(launch_rotate_tc((const float*)Xr, ld, Q64, k, nr, k, k, near_identity, (float*)Xr, ld, gw.buf,
+                                     gw.bytes, st, map));
+      continue;
     }
+    const int* only_if = nullptr;
+    if (gw.rot64)
+      KSCF_CUDA_TRY(launch_rotate_f64tc((const double*)Xr, ld, (const double*)Qm, k, nr, k, k, upper, (double*)Xr, ld,
+                                        gw.buf, gw.bytes, map, gw.gram64, r0 > 0, &only_if, st));
+    KSCF_CUDA_TRY(launch_rotate_native(Xr, ld, Qm, k, nr, k, k, dtype, panel, k, st, map, only_if));
+    KSCF_CUDA_TRY(launch_copy_cols(panel, k, Xr, ld, nr, k, dtype, st, map, only_if));
   }
   return KSCF_OK;
 }
 
-// symmetric_result: A^T B is known to be symmetric (m == n), so the tensor path computes
-// the upper-triangle tiles only and mirrors them.
+// symmetric_result: A^T B is known to be symmetric (m == n), so the tensor paths compute
+// the upper-triangle tiles only and mirror them.
 int gram(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t rows, int m, int n, int dtype, int mode,
-         double scale, double* C, int64_t ldc, void* tcwork, size_t tcbytes, cudaStream_t st,
-         bool symmetric_result = false, const int32_t* rowmap = nullptr) {
+         double scale, double* C, int64_t ldc, const GemmWork& gw, cudaStream_t st, bool symmetric_result = false,
+         const int32_t* rowmap = nullptr) {
   if (mode == KSCF_GEMM_TENSOR) {
     KSCF_CUDA_TRY(launch_gram_tc((const float*)A, lda, (const float*)B, ldb, rows, m, n, scale, C, ldc, false,
-                                 tcwork, tcbytes, st, symmetric_result && m == n, rowmap));
+                                 gw.buf, gw.bytes, st, symmetric_result && m == n, rowmap));
+  } else if (gw.gram64) {
+    KSCF_CUDA_TRY(launch_gram_f64tc((const double*)A, lda, (const double*)B, ldb, rows, m, n, scale, C, ldc, gw.buf,
+                                    gw.bytes, symmetric_result, rowmap, st));
   } else {
-    KSCF_CUDA_TRY(launch_gram_native(A, lda, B, ldb, rows, m, n, dtype, scale, C, ldc, false, st));
+    KSCF_CUDA_TRY(launch_gram_native(A, lda, B, ldb, rows, m, n, dtype, scale, C, ldc, false, st, rowmap));
   }
   return KSCF_OK;
 }
@@ -266,7 +296,7 @@ constexpr double kFp32PolarTol = 1e-4;
 // fails on a pivot at the Gram matrix's own rounding level (8 u S_cc), where the plain
 // factor would amplify rounding noise into the basis.
 int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, const OrthoPlan& p, Carver& cv,
-                bool second_pass, cudaStream_t st, bool* shifted = nullptr, double polar_tol = 0.0) {
+                bool f64tc, bool second_pass, cudaStream_t st, bool* shifted = nullptr, double polar_tol = 0.0) {
   Carver c = cv;
   double* S = (double*)c.take(p.S);
   void* Rinv = c.take(p.Rinv);
@@ -274,9 +304,11 @@ int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, c
   void* cwork = c.take(p.chol);
   void* panel = c.take(p.panel);
   void* tcw = c.take(p.tc);
+  if (f64tc) tcw = c.take(p.tc64);
+  const GemmWork gw = gemm_work(H, k, tcw, f64tc ? p.tc64 : p.tc, f64tc);
   const double h3 = H.grid.h * H.grid.h * H.grid.h;
-  // the tensor path sums over the domain rows only (the padding rows are zero)
-  const int32_t* live = mode == KSCF_GEMM_TENSOR ? H.d_live : nullptr;
+  // the tensor paths sum over the domain rows only (the padding rows are zero)
+  const int32_t* live = mode == KSCF_GEMM_TENSOR || gw.gram64 ? H.d_live : nullptr;
   const int64_t rows = live ? H.n_live : H.grid.n_slots;
   const double u = dtype == KSCF_F64 ? 0x1.0p-53 : 0x1.0p-24;
   int hst[3] = {0, 0, 0};
@@ -286,7 +318,7 @@ int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, c
     KSCF_CUDA_TRY(launch_chol_inv(S, k, k, floor_rel, S, k, cwork, status, st));
     KSCF_CUDA_TRY(cudaMemcpyAsync(hst, status, sizeof(hst), cudaMemcpyDeviceToHost, st));
     KSCF_CUDA_TRY(cudaStreamSynchronize(st));
-    int r = check_tc(mode, "Cholesky-QR");
+    int r = check_tc(mode, f64tc, "Cholesky-QR");
     if (r) return r;
     if (hst[1] != 0) {
       set_error("Cholesky-QR: a grid barrier of the factorisation kernel timed out");
@@ -298,7 +330,7 @@ int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, c
     }
     return KSCF_OK;
   };
-  int rc = gram(X, ld, X, ld, rows, k, k, dtype, mode, h3, S, k, tcw, p.tc, st, false, live);
+  int rc = gram(X, ld, X, ld, rows, k, k, dtype, mode, h3, S, k, gw, st, false, live);
   if (rc) return rc;
   if (polar_tol > 0.0) {
     // S = I + E with |E| <= polar_tol: X <- X (I - E/2), no factorisation
@@ -307,23 +339,23 @@ int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, c
     unsigned long long bits = 0;
     KSCF_CUDA_TRY(cudaMemcpyAsync(&bits, dv, sizeof(bits), cudaMemcpyDeviceToHost, st));
     KSCF_CUDA_TRY(cudaStreamSynchronize(st));
-    rc = check_tc(mode, "Cholesky-QR");
+    rc = check_tc(mode, f64tc, "Cholesky-QR");
     if (rc) return rc;
     double dev;
     std::memcpy(&dev, &bits, sizeof(dev));
     if (dev <= polar_tol) {
       KSCF_CUDA_TRY(launch_polar_first_order(S, k, k, st));
       if (mode != KSCF_GEMM_TENSOR) KSCF_CUDA_TRY(launch_f64_to_dtype(S, (int64_t)k * k, dtype, Rinv, st));
-      rc = rotate_inplace(H, X, ld, k, dtype, mode, Rinv, S, true, panel, p.prows, tcw, p.tc, st);
+      rc = rotate_inplace(H, X, ld, k, dtype, mode, Rinv, S, true, false, panel, p.prows, gw, st);
       if (rc) return rc;
       KSCF_CUDA_TRY(cudaStreamSynchronize(st));
-      return check_tc(mode, "Cholesky-QR");
+      return check_tc(mode, f64tc, "Cholesky-QR");
     }
   }
   rc = factor(shifted ? 8.0 * u : 0.0);
   if (rc) return rc;
   if (hst[0] > 0 && shifted) {
-    rc = gram(X, ld, X, ld, rows, k, k, dtype, mode, h3, S, k, tcw, p.tc, st, false, live);
+    rc = gram(X, ld, X, ld, rows, k, k, dtype, mode, h3, S, k, gw, st, false, live);
     if (rc) return rc;
     KSCF_CUDA_TRY(launch_shift_diag(S, k, 16.0 * k * u, st));
     rc = factor(0.0);
@@ -337,10 +369,10 @@ int cholqr_pass(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode, c
   }
   // S now holds R^-1 (upper triangular, zero below); the native path takes it in X's type
   if (mode != KSCF_GEMM_TENSOR) KSCF_CUDA_TRY(launch_upper_to_dtype(S, k, dtype, Rinv, st));
-  rc = rotate_inplace(H, X, ld, k, dtype, mode, Rinv, S, second_pass, panel, p.prows, tcw, p.tc, st);
+  rc = rotate_inplace(H, X, ld, k, dtype, mode, Rinv, S, second_pass, true, panel, p.prows, gw, st);
   if (rc) return rc;
   KSCF_CUDA_TRY(cudaStreamSynchronize(st));
-  return check_tc(mode, "Cholesky-QR");
+  return check_tc(mode, f64tc, "Cholesky-QR");
 }
 
 }  // namespace
@@ -366,7 +398,7 @@ extern "C" int kscf_workspace_size(const kscf_ham* ham, int op, int k, int dtype
       OrthoPlan p;
       rc = ortho_plan(H, k, dtype, mode, &p);
       if (rc) return rc;
-      *bytes = ortho_bytes(p);
+      *bytes = ortho_bytes(p) + p.tc64;
       return KSCF_OK;
     }
     case KSCF_OP_RR: {
@@ -375,7 +407,7 @@ extern "C" int kscf_workspace_size(const kscf_ham* ham, int op, int k, int dtype
       RRPlan p;
       rc = rr_plan(H, k, dtype, mode, block, &p);
       if (rc) return rc;
-      *bytes = rr_bytes(p);
+      *bytes = rr_bytes(p) + p.tc64;
       return KSCF_OK;
     }
   }
@@ -558,16 +590,17 @@ extern "C" int kscf_orthonormalize(const kscf_ham* ham, void* X, int64_t ld, int
   cudaStream_t st = (cudaStream_t)stream;
   KSCF_CUDA_TRY(launch_zero_rows(H, X, ld, k, dtype, st));
   Carver cv(work);
+  const bool f64tc = p.tc64 > 0 && work_bytes >= ortho_bytes(p) + p.tc64;
   bool shifted = false;
-  rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, false, st, allow_shift ? &shifted : nullptr);
+  rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, f64tc, false, st, allow_shift ? &shifted : nullptr);
   if (rc) return rc;
   if (shifted) {
-    rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, false, st);
+    rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, f64tc, false, st);
     if (rc) return rc;
   }
   // FP32: a second pass (its rotation by the first-order inverse square root of its Gram
   // matrix when that is within kFp32PolarTol of I, else by a factorised R^-1)
-  if (dtype == KSCF_F32) rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, true, st, nullptr, kFp32PolarTol);
+  if (dtype == KSCF_F32) rc = cholqr_pass(H, X, ld, k, dtype, mode, p, cv, f64tc, true, st, nullptr, kFp32PolarTol);
   return rc;
 }
 
@@ -607,10 +640,13 @@ extern "C" int kscf_rayleigh_ritz(const kscf_ham* ham, void* X, int64_t ld, int 
   void* lwork = cv.take(p.lwork_bytes);
   void* panel = cv.take(p.panel);
   void* tcw = cv.take(p.tc);
+  const bool f64tc = p.tc64 > 0 && work_bytes >= rr_bytes(p) + p.tc64;
+  if (f64tc) tcw = cv.take(p.tc64);
+  const GemmWork gw = gemm_work(H, k, tcw, f64tc ? p.tc64 : p.tc, f64tc);
   const size_t es = esize(dtype);
   const double h3 = H.grid.h * H.grid.h * H.grid.h;
-  // the tensor path sums over the domain rows only (padding rows of X and H X are zero)
-  const int32_t* live = mode == KSCF_GEMM_TENSOR ? H.d_live : nullptr;
+  // the tensor paths sum over the domain rows only (padding rows of X and H X are zero)
+  const int32_t* live = mode == KSCF_GEMM_TENSOR || gw.gram64 ? H.d_live : nullptr;
   const int64_t rows = live ? H.n_live : H.grid.n_slots;
   KSCF_CUDA_TRY(launch_zero_rows(H, X, ld, k, dtype, st));
   for (int c0 = 0; c0 < k; c0 += p.w) {
@@ -622,7 +658,7 @@ extern "C" int kscf_rayleigh_ritz(const kscf_ham* ham, void* X, int64_t ld, int 
     KSCF_CUDA_TRY(launch_cheb_step(H, Xb, ld, nullptr, 0, hxb, wpad, wb,
                                    (int)std::min<int64_t>(ld - c0, wpad), dtype, 1.0, 0.0, 0.0, coef, wpad, st));
     // Hs[:, c0:c0+wb] = h^3 X^T (H X_b); with a single block the product is symmetric (H is)
-    rc = gram(X, ld, hxb, wpad, rows, k, wb, dtype, mode, h3, Hs + (size_t)c0 * k, k, tcw, p.tc, st, wb == k, live);
+    rc = gram(X, ld, hxb, wpad, rows, k, wb, dtype, mode, h3, Hs + (size_t)c0 * k, k, gw, st, wb == k, live);
     if (rc) return rc;
   }
   KSCF_CUDA_TRY(launch_sym_eig(Hs, k, k, W, lwork, p.lwork_bytes, info, st));
@@ -635,7 +671,7 @@ extern "C" int kscf_rayleigh_ritz(const kscf_ham* ham, void* X, int64_t ld, int 
   KSCF_CUDA_TRY(cudaMemcpyAsync(hinfo, info, sizeof(hinfo), cudaMemcpyDeviceToHost, st));
   KSCF_CUDA_TRY(cudaMemcpyAsync(eigvals_host, W, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
   KSCF_CUDA_TRY(cudaStreamSynchronize(st));
-  rc = check_tc(mode, "kscf_rayleigh_ritz");
+  rc = check_tc(mode, f64tc, "kscf_rayleigh_ritz");
   if (rc) return rc;
   rc = eig_info_code(hinfo, "kscf_rayleigh_ritz");
   if (rc) return rc;
@@ -644,7 +680,7 @@ extern "C" int kscf_rayleigh_ritz(const kscf_ham* ham, void* X, int64_t ld, int 
       set_error("kscf_rayleigh_ritz: non-finite Ritz value");
       return KSCF_ERR_NONFINITE;
     }
-  return rotate_inplace(H, X, ld, k, dtype, mode, Qm, Hs, mode == KSCF_GEMM_TENSOR, panel, p.prows, tcw, p.tc, st);
+  return rotate_inplace(H, X, ld, k, dtype, mode, Qm, Hs, mode == KSCF_GEMM_TENSOR, false, panel, p.prows, gw, st);
 }
 
 extern "C" int kscf_sym_eig_work_bytes(int n, size_t* bytes) {
@@ -730,7 +766,12 @@ extern "C" int kscf_gram(const void* A, int64_t lda, const void* B, int64_t ldb,
   const size_t need = mode == KSCF_GEMM_TENSOR ? gram_tc_work_bytes(rows, m, n) : 0;
   rc = check_work(work, work_bytes, need, "kscf_gram");
   if (rc) return rc;
-  return gram(A, lda, B, ldb, rows, m, n, dtype, mode, scale, C, ldc, work, work_bytes, (cudaStream_t)stream);
+  // FP64: on the tensor cores when the sizes are worth it and the (optional) buffer holds a chunk
+  const bool same = A == B && lda == ldb && m == n;
+  const bool f64tc = dtype == KSCF_F64 && mode == KSCF_GEMM_NATIVE && work && ((uintptr_t)work & 255) == 0 &&
+                     gram_f64tc_wanted(rows) && gram_f64tc_fits(rows, m, n, same, work_bytes);
+  return gram(A, lda, B, ldb, rows, m, n, dtype, mode, scale, C, ldc, {work, work_bytes, f64tc, false},
+              (cudaStream_t)stream);
 }
 
 extern "C" int kscf_rotate(const void* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin,
@@ -761,7 +802,11 @@ extern "C" int kscf_rotate(const void* A, int64_t lda, const double* Q, int64_t 
   // native: convert Q into the work buffer (column-major, ld = kin), then rotate
   double* Qc = (double*)work;
   if (dtype == KSCF_F64 && ldq == kin) {
-    KSCF_CUDA_TRY(launch_rotate_native(A, lda, Q, ldq, rows, kin, kout, dtype, out, ldo, st));
+    const int* only_if = nullptr;
+    if (rotate_f64tc_wanted(rows, kin, kout) && work_bytes >= rotate_f64tc_work_bytes(rows, kin, kout))
+      KSCF_CUDA_TRY(launch_rotate_f64tc((const double*)A, lda, Q, ldq, rows, kin, kout, false, (double*)out, ldo, work,
+                                        work_bytes, nullptr, false, false, &only_if, st));
+    KSCF_CUDA_TRY(launch_rotate_native(A, lda, Q, ldq, rows, kin, kout, dtype, out, ldo, st, nullptr, only_if));
     return KSCF_OK;
   }
   (void)Qc;
@@ -783,6 +828,10 @@ extern "C" int kscf_gemm_workspace_size(int op, int64_t rows, int m, int n, int 
     *bytes = op == 0 ? gram_tc_work_bytes(rows, m, n) : rotate_tc_work_bytes(rows, m, n);
   else
     *bytes = op == 0 ? 256 : kscf_align256((size_t)m * n * esize(dtype));
+  if (mode == KSCF_GEMM_NATIVE && dtype == KSCF_F64) {
+    if (op == 0 && gram_f64tc_wanted(rows)) *bytes = std::max(*bytes, gram_f64tc_work_bytes(rows, m, n));
+    if (op != 0 && rotate_f64tc_wanted(rows, m, n)) *bytes = std::max(*bytes, rotate_f64tc_work_bytes(rows, m, n));
+  }
   return KSCF_OK;
 }
 
@@ -846,8 +895,10 @@ extern "C" int kscf_selftest_eig_barrier_timeout(void* stream) {
 }
 
 extern "C" int kscf_check_status(void) {
-  unsigned int st = 0, fs = 0, cs = 0, nf = 0;
+  unsigned int st = 0, f64 = 0, fs = 0, cs = 0, nf = 0;
   cudaError_t e = tc_status(true, &st);
+  if (e == cudaSuccess) e = f64tc_status(true, &f64);
+  st |= f64;
   if (e == cudaSuccess) e = filter_status(true, &fs);
   if (e == cudaSuccess) e = cm_status(true, &cs, &nf);
   st |= (fs | cs) << 1;

@@ -801,11 +801,13 @@ __global__ void zero_rows_kernel(T* X, int64_t ld, int k, const int64_t* pad, in
 }
 
 template <typename T>
-__global__ void copy_cols_kernel(const T* src, int64_t ld_src, T* dst, int64_t ld_dst, int64_t rows, int w) {
+__global__ void copy_cols_kernel(const T* src, int64_t ld_src, T* dst, int64_t ld_dst, int64_t rows, int w,
+                                 const int32_t* rowmap, const int* only_if) {
+  if (only_if && *only_if == 0) return;
   const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (r >= rows) return;
   const T* s = src + r * ld_src;
-  T* d = dst + r * ld_dst;
+  T* d = dst + (rowmap ? (int64_t)rowmap[r] : r) * ld_dst;
   for (int j = threadIdx.x & 31; j < w; j += 32) d[j] = s[j];
 }
 
@@ -995,15 +997,15 @@ cudaError_t launch_cheb_step(const Ham& H, const void* in, int64_t ld_in, const 
 }
 
 cudaError_t launch_copy_cols(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t rows, int w,
-                             int dtype, cudaStream_t st) {
+                             int dtype, cudaStream_t st, const int32_t* rowmap, const int* only_if) {
   if (rows == 0 || w == 0) return cudaSuccess;
   const int64_t n = rows * 32;
   if (dtype == KSCF_F64)
     copy_cols_kernel<double><<<blocks_for(n, 256), 256, 0, st>>>((const double*)src, ld_src, (double*)dst,
-                                                                 ld_dst, rows, w), count_launch();
+                                                                 ld_dst, rows, w, rowmap, only_if), count_launch();
   else
     copy_cols_kernel<float><<<blocks_for(n, 256), 256, 0, st>>>((const float*)src, ld_src, (float*)dst,
-                                                                ld_dst, rows, w), count_launch();
+                                                                ld_dst, rows, w, rowmap, only_if), count_launch();
   return cudaGetLastError();
 }
 

@@ -14,12 +14,16 @@ namespace kscf {
 
 static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// With a row map, row r of the operands is row rowmap[r] of the stored matrix; with only_if the
+// kernel does nothing unless *only_if is set (the general path behind gemm_f64.cu's checks).
 // 64x64 tile of C per CTA, 256 threads with 4x4 outputs each; rows split over
 // gridDim.z; partial sums in T over at most 256 rows, then FP64; FP64 atomics into C.
 template <typename T>
 __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B,
                                                     int64_t ldb, int64_t rows, int m, int n, double scale,
-                                                    double* __restrict__ C, int64_t ldc, int64_t rows_per_split) {
+                                                    double* __restrict__ C, int64_t ldc, int64_t rows_per_split,
+                                                    const int32_t* __restrict__ rowmap, const int* only_if) {
+  if (only_if && *only_if == 0) return;
   __shared__ T As[16][64 + 1];
   __shared__ T Bs[16][64 + 1];
   const int i0 = blockIdx.x * 64, j0 = blockIdx.y * 64;
@@ -40,9 +44,10 @@ __global__ void __launch_bounds__(256) gram_kernel(const T* __restrict__ A, int6
     // load 16 rows x 64 columns of A and B
     for (int q = threadIdx.x; q < 16 * 64; q += 256) {
       const int rr = q >> 6, cc = q & 63;
-      const int64_t r = r0 + rr;
-      As[rr][cc] = (r < r_end && i0 + cc < m) ? A[r * lda + i0 + cc] : T(0);
-      Bs[rr][cc] = (r < r_end && j0 + cc < n) ? B[r * ldb + j0 + cc] : T(0);
+      const int64_t q0 = r0 + rr;
+      const int64_t r = rowmap && q0 < r_end ? rowmap[q0] : q0;
+      As[rr][cc] = (q0 < r_end && i0 + cc < m) ? A[r * lda + i0 + cc] : T(0);
+      Bs[rr][cc] = (q0 < r_end && j0 + cc < n) ? B[r * ldb + j0 + cc] : T(0);
     }
     __syncthreads();
 #pragma unroll
@@ -87,7 +92,8 @@ __global__ void zero_matrix_kernel(double* C, int m, int n, int64_t ldc) {
 }
 
 cudaError_t launch_gram_native(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t rows, int m, int n,
-                               int dtype, double scale, double* C, int64_t ldc, bool accumulate, cudaStream_t st) {
+                               int dtype, double scale, double* C, int64_t ldc, bool accumulate, cudaStream_t st,
+                               const int32_t* rowmap, const int* only_if) {
   if (!accumulate) {
     zero_matrix_kernel<<<blocks_for((int64_t)m * n, 256), 256, 0, st>>>(C, m, n, ldc), count_launch();
   }
@@ -102,10 +108,10 @@ cudaError_t launch_gram_native(const void* A, int64_t lda, const void* B, int64_
   dim3 grid(gx, gy, (unsigned)splits);
   if (dtype == KSCF_F64)
     gram_kernel<double><<<grid, 256, 0, st>>>((const double*)A, lda, (const double*)B, ldb, rows, m, n, scale, C,
-                                               ldc, per), count_launch();
+                                               ldc, per, rowmap, only_if), count_launch();
   else
     gram_kernel<float><<<grid, 256, 0, st>>>((const float*)A, lda, (const float*)B, ldb, rows, m, n, scale, C, ldc,
-                                              per), count_launch();
+                                              per, rowmap, only_if), count_launch();
   return cudaGetLastError();
 }
 
@@ -113,7 +119,9 @@ cudaError_t launch_gram_native(const void* A, int64_t lda, const void* B, int64_
 template <typename T>
 __global__ void __launch_bounds__(256) rotate_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ Q,
                                                       int64_t ldq, int64_t rows, int kin, int kout, T* __restrict__ out,
-                                                      int64_t ldo) {
+                                                      int64_t ldo, const int32_t* __restrict__ rowmap,
+                                                      const int* only_if) {
+  if (only_if && *only_if == 0) return;
   __shared__ T As[64][16 + 1];
   __shared__ T Qs[16][64 + 1];
   const int64_t r0 = (int64_t)blockIdx.x * 64;
@@ -128,7 +136,7 @@ __global__ void __launch_bounds__(256) rotate_kernel(const T* __restrict__ A, in
     for (int q = threadIdx.x; q < 64 * 16; q += 256) {
       const int rr = q >> 4, ii = q & 15;
       const int64_t r = r0 + rr;
-      As[rr][ii] = (r < rows && i0 + ii < kin) ? A[r * lda + i0 + ii] : T(0);
+      As[rr][ii] = (r < rows && i0 + ii < kin) ? A[(rowmap ? (int64_t)rowmap[r] : r) * lda + i0 + ii] : T(0);
       const int jj = q >> 4, i2 = q & 15;
       Qs[i2][jj] = (i0 + i2 < kin && j0 + jj < kout) ? Q[(i0 + i2) + (int64_t)(j0 + jj) * ldq] : T(0);
     }
@@ -158,15 +166,16 @@ __global__ void __launch_bounds__(256) rotate_kernel(const T* __restrict__ A, in
 }
 
 cudaError_t launch_rotate_native(const void* A, int64_t lda, const void* Q, int64_t ldq, int64_t rows, int kin,
-                                 int kout, int dtype, void* out, int64_t ldo, cudaStream_t st) {
+                                 int kout, int dtype, void* out, int64_t ldo, cudaStream_t st, const int32_t* rowmap,
+                                 const int* only_if) {
   if (rows == 0 || kout == 0) return cudaSuccess;
   dim3 grid((unsigned)((rows + 63) / 64), (kout + 63) / 64);
   if (dtype == KSCF_F64)
     rotate_kernel<double><<<grid, 256, 0, st>>>((const double*)A, lda, (const double*)Q, ldq, rows, kin, kout,
-                                                 (double*)out, ldo), count_launch();
+                                                 (double*)out, ldo, rowmap, only_if), count_launch();
   else
     rotate_kernel<float><<<grid, 256, 0, st>>>((const float*)A, lda, (const float*)Q, ldq, rows, kin, kout,
-                                                (float*)out, ldo), count_launch();
+                                                (float*)out, ldo, rowmap, only_if), count_launch();
   return cudaGetLastError();
 }
 

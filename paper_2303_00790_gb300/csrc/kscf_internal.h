@@ -155,7 +155,8 @@ cudaError_t launch_polar_first_order(double* S, int k, int64_t lds, cudaStream_t
 // device status words of the chunk-major path: a timed-out wait, non-finite output
 cudaError_t cm_status(bool reset, unsigned int* timeout, unsigned int* nonfinite);
 cudaError_t launch_copy_cols(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t rows,
-                             int w, int dtype, cudaStream_t st);
+                             int w, int dtype, cudaStream_t st, const int32_t* rowmap = nullptr,
+                             const int* only_if = nullptr);
 
 // ---- launchers (setup.cu) ----
 cudaError_t launch_vloc(const Ham& H, const double* d_xyz /*n_slots*3*/, const double* d_atoms /*n*8*/,
@@ -173,13 +174,39 @@ cudaError_t launch_minmax_v(const Ham& H, double* d_out2, cudaStream_t st);
 cudaError_t launch_mask_v(const Ham& H, const double* src, double* dst, cudaStream_t st);
 
 // ---- launchers (gemm.cu) ----
+// rowmap (device, may be null): row r of A and B is row rowmap[r] of the stored matrices;
+// only_if (device, may be null): the kernel does nothing while *only_if is 0.
 // C[i + j*ldc] (+)= scale * sum_r A[r*lda + i] * B[r*ldb + j], i < m, j < n, r < rows.
 cudaError_t launch_gram_native(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t rows,
                                int m, int n, int dtype, double scale, double* C, int64_t ldc,
-                               bool accumulate, cudaStream_t st);
+                               bool accumulate, cudaStream_t st, const int32_t* rowmap = nullptr,
+                               const int* only_if = nullptr);
 // out[r*ldo + j] = sum_i A[r*lda + i] * Q[i + j*ldq]  (Q column-major, dtype of A)
 cudaError_t launch_rotate_native(const void* A, int64_t lda, const void* Q, int64_t ldq, int64_t rows,
-                                 int kin, int kout, int dtype, void* out, int64_t ldo, cudaStream_t st);
+                                 int kin, int kout, int dtype, void* out, int64_t ldo, cudaStream_t st,
+                                 const int32_t* rowmap = nullptr, const int* only_if = nullptr);
+// ---- FP64 products on the tensor cores (gemm_f64.cu) ----
+// Whether the sizes are worth it (smaller products stay on the CUDA-core kernels)
+bool gram_f64tc_wanted(int64_t rows);
+bool rotate_f64tc_wanted(int64_t rows, int kin, int kout);
+// work buffer sizes; a Gram also runs (in more launches) with any buffer gram_f64tc_fits accepts
+size_t gram_f64tc_work_bytes(int64_t rows, int m, int n);
+bool gram_f64tc_fits(int64_t rows, int m, int n, bool same, size_t bytes);
+size_t rotate_f64tc_work_bytes(int64_t rows, int kin, int kout);
+// C (zeroed here) = scale * A^T B over the (mapped) rows; symmetric: A^T B is known to be symmetric (upper tiles,
+// mirrored).  Operands that hold a NaN, an Inf or extreme magnitudes go through launch_gram_native.
+cudaError_t launch_gram_f64tc(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t rows, int m, int n,
+                              double scale, double* C, int64_t ldc, void* work, size_t work_bytes, bool symmetric,
+                              const int32_t* rowmap, cudaStream_t st);
+// out = A Q (out may be A; rows of both through rowmap).  *flag_out: device word set when Q or A hold a NaN, an
+// Inf or extreme magnitudes; out is then untouched and the caller's general path runs behind only_if.
+// upper: Q is upper triangular.  reuse_max: the work buffer still holds the column maxima that a Gram with the same
+// A (all rows) left there; reuse_q: and Q's digits from the previous row panel.
+cudaError_t launch_rotate_f64tc(const double* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin,
+                                int kout, bool upper, double* out, int64_t ldo, void* work, size_t work_bytes,
+                                const int32_t* rowmap, bool reuse_max, bool reuse_q, const int** flag_out,
+                                cudaStream_t st);
+cudaError_t f64tc_status(bool reset, unsigned int* status);
 cudaError_t launch_symmetrize(double* C, int k, int64_t ldc, cudaStream_t st);
 // S[i][i] += rel * max_i S[i][i]
 cudaError_t launch_shift_diag(double* S, int k, double rel, cudaStream_t st);
