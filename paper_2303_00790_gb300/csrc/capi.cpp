@@ -197,6 +197,24 @@ size_t apply_bytes(const Ham& H, int k, int dtype) {
   return kscf_align256((size_t)std::max(H.n_kb, 1) * 4 * coef_ld(k) * esize(dtype));
 }
 
+// Exponent table of one application of H with the FP64 step in fixed point, optional at the end
+// of the work buffer (a buffer without it runs the generic FP64 kernel)
+size_t emax_bytes(const Ham& H, int w, int dtype) {
+  return dtype == KSCF_F64 && step64_wanted(H, w) ? step64_emax_bytes(H, w) : 0;
+}
+
+// One application of H to w columns in `in` (padding rows zero): the FP64 step in fixed point
+// with its exponents in `emax` when given, else launch_cheb_step
+cudaError_t apply_step(const Ham& H, const void* in, int64_t ld_in, void* out, int64_t ld_out, int w, int wavail,
+                       int dtype, const void* coef, int64_t cld, int* emax, cudaStream_t st) {
+  if (!emax)
+    return launch_cheb_step(H, in, ld_in, nullptr, 0, out, ld_out, w, wavail, dtype, 1.0, 0.0, 0.0, coef, cld, st);
+  cudaError_t e = launch_emax64(H, (const double*)in, ld_in, w, emax, st);
+  if (e != cudaSuccess) return e;
+  return launch_step64(H, (const double*)in, ld_in, nullptr, 0, (double*)out, ld_out, w, 1.0, 0.0, 0.0,
+                       (const double*)coef, cld, emax, nullptr, st);
+}
+
 int check_work(void* work, size_t have, size_t need, const char* who) {
   if (have < need || (need > 0 && !work)) {
     set_error("%s: work buffer of %zu bytes, need %zu", who, have, need);
@@ -387,7 +405,7 @@ extern "C" int kscf_workspace_size(const kscf_ham* ham, int op, int k, int dtype
   const Ham& H = ham->h;
   switch (op) {
     case KSCF_OP_APPLY:
-      *bytes = apply_bytes(H, k, dtype);
+      *bytes = apply_bytes(H, k, dtype) + emax_bytes(H, k, dtype);
       return KSCF_OK;
     case KSCF_OP_FILTER:
       *bytes = filter_bytes(H, k, dtype, block);
@@ -430,8 +448,11 @@ extern "C" int kscf_hamiltonian_apply(const kscf_ham* ham, void* Y, int64_t ld_y
   KSCF_CUDA_TRY(launch_zero_rows(H, Y, ld_y, k, dtype, st));
   KSCF_CUDA_TRY(launch_zero_rows(H, HY, ld_hy, k, dtype, st));
   KSCF_CUDA_TRY(launch_kb_gather(H, Y, ld_y, k, dtype, work, coef_ld(k), st));
-  KSCF_CUDA_TRY(launch_cheb_step(H, Y, ld_y, nullptr, 0, HY, ld_hy, k, (int)std::min<int64_t>(ld_y, ld_hy), dtype,
-                                 1.0, 0.0, 0.0, work, coef_ld(k), st));
+  const size_t opt = emax_bytes(H, k, dtype);
+  int* emax = opt > 0 && work_bytes >= apply_bytes(H, k, dtype) + opt ? (int*)((char*)work + apply_bytes(H, k, dtype))
+                                                                     : nullptr;
+  KSCF_CUDA_TRY(apply_step(H, Y, ld_y, HY, ld_hy, k, (int)std::min<int64_t>(ld_y, ld_hy), dtype, work, coef_ld(k), emax,
+                           st));
   // a NaN or Inf in Y or in the potential shows up in HY: flag it for kscf_check_status
   unsigned int* flag = nonfinite_flag();
   if (!flag) {
@@ -542,6 +563,44 @@ extern "C" int kscf_chebyshev_filter(const kscf_ham* ham, void* X, int64_t ld, i
   void* buf = cv.take((size_t)H.grid.n_slots * wpad * es);
   void* coef = cv.take((size_t)std::max(H.n_kb, 1) * 4 * wpad * es);
   KSCF_CUDA_TRY(launch_zero_rows(H, X, ld, k, dtype, st));
+  if (dtype == KSCF_F64 && step64_available(H)) {
+    // the buffer of one slot-major copy holds two chunk-major copies of about half the columns
+    // and their exponents; the last step writes into the caller's block
+    const int half = (int)(wpad / 2);
+    const size_t room = (size_t)H.grid.n_slots * wpad * 8;
+    auto need = [&](int n) {
+      const int n4 = (n + 3) / 4 * 4;
+      return 2 * kscf_align256((size_t)H.grid.n_slots * n4 * 8) + 2 * step64_emax_bytes(H, n4);
+    };
+    int ws = half;
+    while (ws > 4 && need(ws) > room) ws -= 4;
+    const int parts = (w + ws - 1) / ws;
+    ws = ((w + parts - 1) / parts + 3) / 4 * 4;   // even parts
+    Carver cb(buf);
+    double* A = (double*)cb.take((size_t)H.grid.n_slots * ws * 8);
+    double* B = (double*)cb.take((size_t)H.grid.n_slots * ws * 8);
+    int* emax[2] = {(int*)cb.take(step64_emax_bytes(H, ws)), (int*)cb.take(step64_emax_bytes(H, ws))};
+    double* cf = (double*)coef;
+    for (int c0 = 0; c0 < k; c0 += ws) {
+      const int wb = std::min(ws, k - c0);
+      double* Xb = (double*)X + c0;
+      KSCF_CUDA_TRY(launch_to_cm64(H, Xb, ld, wb, A, B, emax[0], st));
+      double *cur = A, *other = B, sigma = sigma1;
+      for (int j = 1; j <= degree; j++) {
+        const bool last = j == degree;
+        const double sigma_new = j == 1 ? sigma1 : 1.0 / (tau - sigma);
+        KSCF_CUDA_TRY(launch_gather_cm64(H, cur, wb, cf, wpad, st));
+        // Y_1 = (sigma_1/e)(H X - c X); later Y_j overwrites Y_{j-2} in place
+        KSCF_CUDA_TRY(launch_step64(H, cur, -1, j == 1 ? nullptr : other, -1, last ? Xb : other, last ? ld : -1, wb,
+                                    j == 1 ? sigma1 / e : 2.0 * sigma_new / e, j == 1 ? 0.0 : -sigma * sigma_new, c, cf,
+                                    wpad, emax[0], last ? nullptr : emax[1], st));
+        std::swap(cur, other);
+        std::swap(emax[0], emax[1]);
+        sigma = sigma_new;
+      }
+    }
+    return KSCF_OK;
+  }
   for (int c0 = 0; c0 < k; c0 += w) {
     const int wb = std::min(w, k - c0);
     char* Xb = (char*)X + (size_t)c0 * es;
@@ -655,8 +714,11 @@ extern "C" int kscf_rayleigh_ritz(const kscf_ham* ham, void* X, int64_t ld, int 
     const int64_t wpad = coef_ld(wb);
     KSCF_CUDA_TRY(launch_zero_rows(H, hxb, wpad, wb, dtype, st));
     KSCF_CUDA_TRY(launch_kb_gather(H, Xb, ld, wb, dtype, coef, wpad, st));
-    KSCF_CUDA_TRY(launch_cheb_step(H, Xb, ld, nullptr, 0, hxb, wpad, wb,
-                                   (int)std::min<int64_t>(ld - c0, wpad), dtype, 1.0, 0.0, 0.0, coef, wpad, st));
+    // (the exponents borrow the products' work space, which the Gram fills afterwards)
+    const size_t opt = emax_bytes(H, wb, dtype);
+    int* emax = opt > 0 && f64tc && p.tc64 >= opt ? (int*)tcw : nullptr;
+    KSCF_CUDA_TRY(apply_step(H, Xb, ld, hxb, wpad, wb, (int)std::min<int64_t>(ld - c0, wpad), dtype, coef, wpad, emax,
+                             st));
     // Hs[:, c0:c0+wb] = h^3 X^T (H X_b); with a single block the product is symmetric (H is)
     rc = gram(X, ld, hxb, wpad, rows, k, wb, dtype, mode, h3, Hs + (size_t)c0 * k, k, gw, st, wb == k, live);
     if (rc) return rc;

@@ -122,6 +122,23 @@ cudaError_t launch_cheb_step(const Ham& H, const void* in, int64_t ld_in, const 
                              int64_t ld_prev, void* out, int64_t ld_out, int w, int wavail, int dtype,
                              double alpha, double beta, double c, const void* coef, int64_t cld,
                              cudaStream_t st);
+// ---- FP64 step on 8^3 bricks in fixed point (filter_f64.cu) ----
+bool step64_available(const Ham& H);
+bool step64_wanted(const Ham& H, int w);   // for a single application to w columns
+// emax tables (exponents per brick and vector) of w columns
+size_t step64_emax_bytes(const Ham& H, int w);
+cudaError_t launch_emax64(const Ham& H, const double* X, int64_t ld, int w, int* emax, cudaStream_t st);
+// A = chunk-major copy (4 columns per chunk, round4(w) columns of n_slots rows) of w columns of X, padding rows of A
+// and B zero, emax of X
+cudaError_t launch_to_cm64(const Ham& H, const double* X, int64_t ld, int w, double* A, double* B, int* emax,
+                           cudaStream_t st);
+cudaError_t launch_gather_cm64(const Ham& H, const double* Y, int w, double* coef, int64_t cld, cudaStream_t st);
+// Blocks with a row stride ld < 0 are chunk-major.
+// The step of launch_cheb_step with emax_in the exponents of `in`; emax_out (may be null) receives those of
+// `out`.  Padding rows of `in` must be zero; those of `out` are not written.
+cudaError_t launch_step64(const Ham& H, const double* in, int64_t ld_in, const double* prev, int64_t ld_prev, double* out,
+                          int64_t ld_out, int w, double alpha, double beta, double c, const double* coef, int64_t cld,
+                          const int* emax_in, int* emax_out, cudaStream_t st);
 inline int64_t coef_ld(int w) { return (int64_t)(w + 31) / 32 * 32; }
 
 // ---- chunk-major filter path (filter_cm.cu, FP32, 8^3 and 16^3 bricks) ----
