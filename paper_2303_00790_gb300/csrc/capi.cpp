@@ -204,15 +204,18 @@ size_t emax_bytes(const Ham& H, int w, int dtype) {
 }
 
 // One application of H to w columns in `in` (padding rows zero): the FP64 step in fixed point
-// with its exponents in `emax` when given, else launch_cheb_step
+// with its exponents in `emax` when given, else launch_cheb_step.  FP64 with flag64: the kernel
+// zeroes the padding rows of `out` and reports a NaN or Inf in *flag64.
 cudaError_t apply_step(const Ham& H, const void* in, int64_t ld_in, void* out, int64_t ld_out, int w, int wavail,
-                       int dtype, const void* coef, int64_t cld, int* emax, cudaStream_t st) {
+                       int dtype, const void* coef, int64_t cld, int* emax, cudaStream_t st,
+                       unsigned int* flag64 = nullptr) {
   if (!emax)
-    return launch_cheb_step(H, in, ld_in, nullptr, 0, out, ld_out, w, wavail, dtype, 1.0, 0.0, 0.0, coef, cld, st);
+    return launch_cheb_step(H, in, ld_in, nullptr, 0, out, ld_out, w, wavail, dtype, 1.0, 0.0, 0.0, coef, cld, st,
+                            flag64);
   cudaError_t e = launch_emax64(H, (const double*)in, ld_in, w, emax, st);
   if (e != cudaSuccess) return e;
   return launch_step64(H, (const double*)in, ld_in, nullptr, 0, (double*)out, ld_out, w, 1.0, 0.0, 0.0,
-                       (const double*)coef, cld, emax, nullptr, st);
+                       (const double*)coef, cld, emax, nullptr, st, flag64);
 }
 
 int check_work(void* work, size_t have, size_t need, const char* who) {
@@ -445,21 +448,22 @@ extern "C" int kscf_hamiltonian_apply(const kscf_ham* ham, void* Y, int64_t ld_y
   rc = check_work(work, work_bytes, apply_bytes(H, k, dtype), "kscf_hamiltonian_apply");
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
-  KSCF_CUDA_TRY(launch_zero_rows(H, Y, ld_y, k, dtype, st));
-  KSCF_CUDA_TRY(launch_zero_rows(H, HY, ld_hy, k, dtype, st));
-  KSCF_CUDA_TRY(launch_kb_gather(H, Y, ld_y, k, dtype, work, coef_ld(k), st));
-  const size_t opt = emax_bytes(H, k, dtype);
-  int* emax = opt > 0 && work_bytes >= apply_bytes(H, k, dtype) + opt ? (int*)((char*)work + apply_bytes(H, k, dtype))
-                                                                     : nullptr;
-  KSCF_CUDA_TRY(apply_step(H, Y, ld_y, HY, ld_hy, k, (int)std::min<int64_t>(ld_y, ld_hy), dtype, work, coef_ld(k), emax,
-                           st));
   // a NaN or Inf in Y or in the potential shows up in HY: flag it for kscf_check_status
   unsigned int* flag = nonfinite_flag();
   if (!flag) {
     set_error("kscf_hamiltonian_apply: status word lookup failed");
     return KSCF_ERR_CUDA;
   }
-  KSCF_CUDA_TRY(launch_finite_rows(H, HY, ld_hy, k, dtype, flag, st));
+  const bool f64 = dtype == KSCF_F64;   // its kernels zero the padding rows and check themselves
+  KSCF_CUDA_TRY(launch_zero_rows(H, Y, ld_y, k, dtype, st));
+  if (!f64) KSCF_CUDA_TRY(launch_zero_rows(H, HY, ld_hy, k, dtype, st));
+  KSCF_CUDA_TRY(launch_kb_gather(H, Y, ld_y, k, dtype, work, coef_ld(k), st));
+  const size_t opt = emax_bytes(H, k, dtype);
+  int* emax = opt > 0 && work_bytes >= apply_bytes(H, k, dtype) + opt ? (int*)((char*)work + apply_bytes(H, k, dtype))
+                                                                     : nullptr;
+  KSCF_CUDA_TRY(apply_step(H, Y, ld_y, HY, ld_hy, k, (int)std::min<int64_t>(ld_y, ld_hy), dtype, work, coef_ld(k), emax,
+                           st, f64 ? flag : nullptr));
+  if (!f64) KSCF_CUDA_TRY(launch_finite_rows(H, HY, ld_hy, k, dtype, flag, st));
   return KSCF_OK;
 }
 

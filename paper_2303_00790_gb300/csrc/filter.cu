@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "gather.cuh"
 #include "kscf_internal.h"
 
 namespace kscf {
@@ -39,10 +40,11 @@ struct StepArgs {
   const T* kb_chi;
   T st[7];
   int64_t n_slots;
+  unsigned int* flag;   // generic kernel: set when a domain row gets a NaN or Inf (may be null)
 };
 
 // ---------------------------------------------------------------------------
-// Reference-shaped kernel: one thread per (slot, vector).
+// Reference-shaped kernel: one thread per (slot, vector); padding rows of out are zeroed.
 template <typename T, int B>
 __global__ void __launch_bounds__(256) cheb_step_generic(StepArgs<T> a) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -87,6 +89,7 @@ __global__ void __launch_bounds__(256) cheb_step_generic(StepArgs<T> a) {
     }
     res = a.alpha * (acc - a.c * y);
     if (a.prev) res += a.beta * a.prev[s * a.ld_prev + v];
+    if (a.flag && !(fabs((double)res) <= 1.7976931348623157e308)) atomicOr(a.flag, 1u);
   }
   a.out[s * a.ld_out + v] = res;
 }
@@ -760,37 +763,6 @@ cudaError_t filter_status(bool reset, unsigned int* status) {
   return e;
 }
 
-// coef[(a*4+l)*w + v] = E_l h^3 sum_{entries e of atom a} chi_l(e) Y[slot_e][v]
-template <typename T>
-__global__ void __launch_bounds__(256) kb_gather_kernel(const T* __restrict__ Y, int64_t ld, int w, int64_t cld,
-                                                         const int64_t* __restrict__ aptr,
-                                                         const int64_t* __restrict__ aslot,
-                                                         const T* __restrict__ achi,
-                                                         const double* __restrict__ energy,
-                                                         T* __restrict__ coef) {
-  const int at = blockIdx.x;
-  const int v = blockIdx.y * 32 + threadIdx.x;
-  T acc[4] = {T(0), T(0), T(0), T(0)};
-  if (v < w) {
-    for (int64_t e = aptr[at] + threadIdx.y; e < aptr[at + 1]; e += 8) {
-      const T y = Y[aslot[e] * ld + v];
-#pragma unroll
-      for (int l = 0; l < 4; l++) acc[l] += achi[4 * e + l] * y;
-    }
-  }
-  __shared__ T red[8][4][32];
-#pragma unroll
-  for (int l = 0; l < 4; l++) red[threadIdx.y][l][threadIdx.x] = acc[l];
-  __syncthreads();
-  if (threadIdx.y < 4 && v < w) {
-    const int l = threadIdx.y;
-    T sum = T(0);
-#pragma unroll
-    for (int q = 0; q < 8; q++) sum += red[q][l][threadIdx.x];
-    coef[((int64_t)at * 4 + l) * cld + v] = (T)energy[4 * at + l] * sum;
-  }
-}
-
 // one warp per row: coalesced 128-byte stores, no per-element division
 template <typename T>
 __global__ void zero_rows_kernel(T* X, int64_t ld, int k, const int64_t* pad, int64_t n_pad) {
@@ -851,16 +823,14 @@ cudaError_t launch_zero_rows(const Ham& H, void* X, int64_t ld, int k, int dtype
 cudaError_t launch_kb_gather(const Ham& H, const void* Y, int64_t ld, int w, int dtype, void* coef, int64_t cld,
                              cudaStream_t st) {
   if (H.n_kb == 0 || w == 0) return cudaSuccess;
-  dim3 grid(H.n_kb, (w + 31) / 32), block(32, 8);
+  count_launch();
   if (dtype == KSCF_F64)
-    kb_gather_kernel<double><<<grid, block, 0, st>>>((const double*)Y, ld, w, cld, H.d_kb_atom_ptr,
-                                                     H.d_kb_atom_slot, H.d_kb_atom_chi64,
-                                                     H.d_kb_energy, (double*)coef), count_launch();
-  else
-    kb_gather_kernel<float><<<grid, block, 0, st>>>((const float*)Y, ld, w, cld, H.d_kb_atom_ptr,
-                                                    H.d_kb_atom_slot, H.d_kb_atom_chi32,
-                                                    H.d_kb_energy, (float*)coef), count_launch();
-  return cudaGetLastError();
+    return launch_gather<double, 1>({(const double*)Y, 0, ld, 30, w, 0, cld, H.d_kb_atom_ptr, H.d_kb_atom_slot,
+                                     H.d_kb_atom_chi64, H.d_kb_energy, (double*)coef},
+                                    H.n_kb, st);
+  return launch_gather<float, 1>({(const float*)Y, 0, ld, 30, w, 0, cld, H.d_kb_atom_ptr, H.d_kb_atom_slot,
+                                  H.d_kb_atom_chi32, H.d_kb_energy, (float*)coef},
+                                 H.n_kb, st);
 }
 
 
@@ -870,8 +840,9 @@ static bool g_brick32_attr[64] = {false};
 template <typename T>
 static cudaError_t step_t(const Ham& H, const void* in, int64_t ld_in, const void* prev, int64_t ld_prev,
                           void* out, int64_t ld_out, int w, int wavail, double alpha, double beta, double c,
-                          const void* coef, int64_t cld, const T* V, const T* chi, cudaStream_t st) {
+                          const void* coef, int64_t cld, const T* V, const T* chi, unsigned int* flag, cudaStream_t st) {
   StepArgs<T> a;
+  a.flag = flag;
   a.in = (const T*)in;
   a.ld_in = ld_in;
   a.prev = (const T*)prev;
@@ -988,12 +959,12 @@ static cudaError_t step_t(const Ham& H, const void* in, int64_t ld_in, const voi
 
 cudaError_t launch_cheb_step(const Ham& H, const void* in, int64_t ld_in, const void* prev, int64_t ld_prev,
                              void* out, int64_t ld_out, int w, int wavail, int dtype, double alpha, double beta,
-                             double c, const void* coef, int64_t cld, cudaStream_t st) {
+                             double c, const void* coef, int64_t cld, cudaStream_t st, unsigned int* flag64) {
   if (dtype == KSCF_F64)
     return step_t<double>(H, in, ld_in, prev, ld_prev, out, ld_out, w, wavail, alpha, beta, c, coef, cld,
-                          H.d_v64, H.d_kb_slot_chi64, st);
+                          H.d_v64, H.d_kb_slot_chi64, flag64, st);
   return step_t<float>(H, in, ld_in, prev, ld_prev, out, ld_out, w, wavail, alpha, beta, c, coef, cld, H.d_v32,
-                       H.d_kb_slot_chi32, st);
+                       H.d_kb_slot_chi32, nullptr, st);
 }
 
 cudaError_t launch_copy_cols(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int64_t rows, int w,

@@ -15,7 +15,7 @@
 // One step computes, for every slot s and vector v,
 //   out = alpha (H in - c in) + beta prev,
 //   H in = -1/2 Lap_h in + V in + sum_i chi_i (E_i h^3 <chi_i, in>),
-// the nonlocal projections <chi_i, in> coming from kb_gather_cm launched just before.
+// the nonlocal projections <chi_i, in> coming from kb_gather_kernel launched just before.
 // cm_step_ldg16 does it for one cell and 16 vectors per CTA: the cell core is copied
 // into shared memory, the halo rows of each line come from the neighbour cells in L2
 // into registers, lines that hold no domain point are skipped, and the nonlocal term of a
@@ -28,6 +28,7 @@
 #include <cstdlib>
 #include <mutex>
 
+#include "gather.cuh"
 #include "kscf_internal.h"
 
 namespace kscf {
@@ -366,61 +367,6 @@ __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t*
 }
 
 // ---------------------------------------------------------------------------
-// coef[(a*4+l)*cld + v] = E_l h^3 sum_{entries e of atom a} chi_l(e) Y(slot_e, v) for
-// v < w, and 0 for w <= v < cld (the padded columns of the last chunk then stay zero
-// through the recurrence).  Y chunk-major with chunks of 16 columns.  A CTA takes one atom
-// and 128 columns (8 chunks); its 8 warps stride over the atom's entries, lane (chunk
-// lane / 4, quad lane % 4) reading its 4 columns of the entry's row as one float4; the
-// warps' sums meet in shared memory.
-__global__ void __launch_bounds__(256) kb_gather_cm(const float* __restrict__ Y, int64_t n_slots, int w, int nchunk,
-                                                    int64_t cld, const int64_t* __restrict__ aptr,
-                                                    const int64_t* __restrict__ aslot,
-                                                    const float* __restrict__ achi,
-                                                    const double* __restrict__ energy, float* __restrict__ coef) {
-  const int at = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.y * 8 + (lane >> 2);
-  float acc[16];   // [l * 4 + column of the quad]
-#pragma unroll
-  for (int i = 0; i < 16; i++) acc[i] = 0.f;
-  if (chunk < nchunk) {
-    const float* base = Y + (int64_t)chunk * n_slots * 16 + (lane & 3) * 4;
-    const int64_t e1 = __ldg(aptr + at + 1);
-    int64_t e = __ldg(aptr + at) + warp;
-    auto add = [&](float4 c, float4 y) {
-      const float cl[4] = {c.x, c.y, c.z, c.w}, yv[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-      for (int l = 0; l < 4; l++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[l * 4 + q] = fmaf(cl[l], yv[q], acc[l * 4 + q]);
-    };
-    for (; e + 8 < e1; e += 16) {
-      const int64_t s0 = __ldg(aslot + e), s1 = __ldg(aslot + e + 8);
-      const float4 c0 = __ldg((const float4*)(achi + 4 * e)), c1 = __ldg((const float4*)(achi + 4 * (e + 8)));
-      const float4 y0 = __ldg((const float4*)(base + s0 * 16)), y1 = __ldg((const float4*)(base + s1 * 16));
-      add(c0, y0);
-      add(c1, y1);
-    }
-    if (e < e1) add(__ldg((const float4*)(achi + 4 * e)), __ldg((const float4*)(base + __ldg(aslot + e) * 16)));
-  }
-  __shared__ float red[8][16][33];
-#pragma unroll
-  for (int i = 0; i < 16; i++) red[warp][i][lane] = acc[i];
-  __syncthreads();
-  // output element o = l * 128 + vv (vv: column inside the CTA's 128): contiguous stores
-  for (int o = threadIdx.x; o < 512; o += 256) {
-    const int l = o >> 7, vv = o & 127;
-    const int ln = (vv >> 4) * 4 + ((vv >> 2) & 3), i = l * 4 + (vv & 3);
-    const int64_t v = (int64_t)blockIdx.y * 128 + vv;
-    if (v < cld) {
-      float sum = 0.f;
-#pragma unroll
-      for (int q = 0; q < 8; q++) sum += red[q][i][ln];
-      coef[((int64_t)at * 4 + l) * cld + v] = v < w ? (float)energy[4 * at + l] * sum : 0.f;
-    }
-  }
-}
-
 // chunk-major copy (chunks of 16 columns) of w columns of a slot-major block (row stride
 // ld), padded columns and padding rows zero (padding rows are not read); the padding rows
 // of the second working buffer are zeroed too (the step kernels never write padding rows,
@@ -462,11 +408,11 @@ cudaError_t launch_kb_gather_cm(const Ham& H, const float* Y, int cw, int w, flo
                                 cudaStream_t st) {
   if (H.n_kb == 0 || w == 0) return cudaSuccess;
   if (cw != 16) return cudaErrorInvalidValue;
-  dim3 grid(H.n_kb, (unsigned)((cld + 127) / 128));
-  kb_gather_cm<<<grid, 256, 0, st>>>(Y, H.grid.n_slots, w, (w + 15) / 16, cld, H.d_kb_atom_ptr, H.d_kb_atom_slot,
-                                     H.d_kb_atom_chi32, H.d_kb_energy, coef),
-      count_launch();
-  return cudaGetLastError();
+  count_launch();
+  // the padded columns of the last chunk get zero coefficients and stay zero in the recurrence
+  return launch_gather<float, 4>({Y, H.grid.n_slots * 16, 16, 4, w, (int)cld, cld, H.d_kb_atom_ptr, H.d_kb_atom_slot,
+                                  H.d_kb_atom_chi32, H.d_kb_energy, coef},
+                                 H.n_kb, st);
 }
 
 // One degree step: in chunk-major (chunk width cm_chunk_width()); prev chunk-major or

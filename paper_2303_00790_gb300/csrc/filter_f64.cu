@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "fixlap.cuh"
+#include "gather.cuh"
 #include "kscf_internal.h"
 
 namespace kscf {
@@ -75,6 +76,7 @@ struct Step64 {
   const int32_t *batoms, *bnat;
   const int *emax_in;
   int* emax_out;
+  unsigned int* flag;   // with it, padding rows of out are zeroed and NaN or Inf in domain rows reported
   double st[7];
 };
 
@@ -242,7 +244,10 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
   constexpr int PL = P_PLANE * S_NV * 8;   // bytes of a plane
 #pragma unroll
   for (int z = 0; z < 8; z++) {
-    if (!((live >> z) & 1u)) continue;
+    if (!((live >> z) & 1u)) {
+      if (a.flag && on) outc[z * 64 * a.ld_out] = 0.0;
+      continue;
+    }
     const int r = z * 64 + p;
     double t;
     if (slow) {
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
     outc[z * 64 * a.ld_out] = t;
     mx = max(mx, abs_hw(t));
   }
+  if (a.flag && mx >= 0x7ff00000u) atomicOr(a.flag, 1u);
   if (a.emax_out) {
     // lanes of the same vector are 4 apart
 #pragma unroll
@@ -360,52 +366,6 @@ __global__ void __launch_bounds__(256) to_cm64_kernel(const double* __restrict__
   }
 }
 
-// coef[(a*4+l)*cld + v] = E_l h^3 sum over the atom's entries of chi_l Y(slot, v), Y chunk-major.
-// One CTA per atom and 32 columns; its 8 warps stride over the entries, four in flight.
-__global__ void __launch_bounds__(256) gather_cm64_kernel(const double* __restrict__ Y, int64_t n_slots, int w,
-                                                          int64_t cld, const int64_t* __restrict__ aptr,
-                                                          const int64_t* __restrict__ aslot,
-                                                          const double* __restrict__ achi,
-                                                          const double* __restrict__ energy, double* __restrict__ coef) {
-  const int at = blockIdx.x, lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
-  const int v = blockIdx.y * 32 + lane;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  if (v < w) {
-    const double* y0 = Y + (int64_t)(v / S_NV) * n_slots * S_NV + (v & (S_NV - 1));
-    const int64_t e1 = __ldg(aptr + at + 1);
-    int64_t e = __ldg(aptr + at) + wy;
-    for (; e + 24 < e1; e += 32) {
-      double y[4];
-#pragma unroll
-      for (int u = 0; u < 4; u++) y[u] = __ldg(y0 + __ldg(aslot + e + 8 * u) * S_NV);
-#pragma unroll
-      for (int u = 0; u < 4; u++) {
-        const double2 c0 = __ldg((const double2*)(achi + 4 * (e + 8 * u))),
-                      c1 = __ldg((const double2*)(achi + 4 * (e + 8 * u)) + 1);
-        acc[0] = fma(c0.x, y[u], acc[0]);
-        acc[1] = fma(c0.y, y[u], acc[1]);
-        acc[2] = fma(c1.x, y[u], acc[2]);
-        acc[3] = fma(c1.y, y[u], acc[3]);
-      }
-    }
-    for (; e < e1; e += 8) {
-      const double y = __ldg(y0 + __ldg(aslot + e) * S_NV);
-#pragma unroll
-      for (int l = 0; l < 4; l++) acc[l] = fma(__ldg(achi + 4 * e + l), y, acc[l]);
-    }
-  }
-  __shared__ double red[8][4][32];
-#pragma unroll
-  for (int l = 0; l < 4; l++) red[wy][l][lane] = acc[l];
-  __syncthreads();
-  if (wy < 4 && v < w) {
-    double sum = 0.0;
-#pragma unroll
-    for (int q = 0; q < 8; q++) sum += red[q][wy][lane];
-    coef[((int64_t)at * 4 + wy) * cld + v] = energy[4 * at + wy] * sum;
-  }
-}
-
 int emax_ld(int w) { return (w + 3) / 4 * 4; }
 
 constexpr int kFixW[6] = {1425600, -222750, 44000, -7425, 864, -50};
@@ -456,18 +416,18 @@ cudaError_t launch_to_cm64(const Ham& H, const double* X, int64_t ld, int w, dou
 
 cudaError_t launch_gather_cm64(const Ham& H, const double* Y, int w, double* coef, int64_t cld, cudaStream_t st) {
   if (H.n_kb == 0 || w == 0) return cudaSuccess;
-  gather_cm64_kernel<<<dim3(H.n_kb, (w + 31) / 32), 256, 0, st>>>(Y, H.grid.n_slots, w, cld, H.d_kb_atom_ptr,
-                                                                 H.d_kb_atom_slot, H.d_kb_atom_chi64, H.d_kb_energy,
-                                                                 coef),
-      count_launch();
-  return cudaGetLastError();
+  count_launch();
+  return launch_gather<double, 2>({Y, H.grid.n_slots * S_NV, S_NV, 2, w, 0, cld, H.d_kb_atom_ptr, H.d_kb_atom_slot,
+                                   H.d_kb_atom_chi64, H.d_kb_energy, coef},
+                                  H.n_kb, st);
 }
 
 // ld < 0: chunk-major
 cudaError_t launch_step64(const Ham& H, const double* in, int64_t ld_in, const double* prev, int64_t ld_prev, double* out,
                           int64_t ld_out, int w, double alpha, double beta, double c, const double* coef, int64_t cld,
-                          const int* emax_in, int* emax_out, cudaStream_t st) {
+                          const int* emax_in, int* emax_out, cudaStream_t st, unsigned int* flag) {
   Step64 a;
+  a.flag = flag;
   const bool cm = ld_in < 0;
   auto place = [&](int64_t ld, int64_t* cs, int64_t* l) {
     *cs = ld < 0 ? H.grid.n_slots * S_NV : S_NV;

@@ -115,13 +115,14 @@ cudaError_t launch_kb_gather(const Ham& H, const void* Y, int64_t ld, int w, int
                              int64_t cld, cudaStream_t st);
 // The FP32 brick kernels do not write padding rows of `out`: callers keep padding rows
 // zero in every buffer they pass (launch_zero_rows once per buffer).
+// FP64: padding rows of `out` are zeroed, and *flag64 (may be null) is set when a domain row gets a NaN or Inf.
 // wavail: columns readable and writable from in/prev/out in every row (>= w); the FP32
 // brick kernel is used when wavail and cld cover round_up8(w) (32-vector CTAs when they
 // cover round_up32(w))
 cudaError_t launch_cheb_step(const Ham& H, const void* in, int64_t ld_in, const void* prev,
                              int64_t ld_prev, void* out, int64_t ld_out, int w, int wavail, int dtype,
                              double alpha, double beta, double c, const void* coef, int64_t cld,
-                             cudaStream_t st);
+                             cudaStream_t st, unsigned int* flag64 = nullptr);
 // ---- FP64 step on 8^3 bricks in fixed point (filter_f64.cu) ----
 bool step64_available(const Ham& H);
 bool step64_wanted(const Ham& H, int w);   // for a single application to w columns
@@ -135,10 +136,11 @@ cudaError_t launch_to_cm64(const Ham& H, const double* X, int64_t ld, int w, dou
 cudaError_t launch_gather_cm64(const Ham& H, const double* Y, int w, double* coef, int64_t cld, cudaStream_t st);
 // Blocks with a row stride ld < 0 are chunk-major.
 // The step of launch_cheb_step with emax_in the exponents of `in`; emax_out (may be null) receives those of
-// `out`.  Padding rows of `in` must be zero; those of `out` are not written.
+// `out`.  Padding rows of `in` must be zero; those of `out` are zeroed with flag (may be null), which is also
+// set when a domain row gets a NaN or Inf, and else not written.
 cudaError_t launch_step64(const Ham& H, const double* in, int64_t ld_in, const double* prev, int64_t ld_prev, double* out,
                           int64_t ld_out, int w, double alpha, double beta, double c, const double* coef, int64_t cld,
-                          const int* emax_in, int* emax_out, cudaStream_t st);
+                          const int* emax_in, int* emax_out, cudaStream_t st, unsigned int* flag = nullptr);
 inline int64_t coef_ld(int w) { return (int64_t)(w + 31) / 32 * 32; }
 
 // ---- chunk-major filter path (filter_cm.cu, FP32, 8^3 and 16^3 bricks) ----

@@ -79,3 +79,19 @@ def test_values_outside_the_fixed_point(kscf, systems, bad):
     fine = torch.isfinite(ref)
     top = torch.where(fine, ref.abs(), 0.0).amax(0)
     assert torch.all(torch.where(fine, (got - ref).abs(), 0.0).amax(0) <= 1e-12 * top)
+
+
+@pytest.mark.parametrize("dtype,tol", [(torch.float64, 1e-13), (torch.float32, 2e-5)])
+def test_projections_of_wide_blocks(kscf, systems, dtype, tol):
+    """The projections' kernel for many columns gives the columns what the one for few gives them
+    (the same sums in another order; the apply tests' tolerances)."""
+    grid, ham = systems[8]
+    k = 35 * 220 if dtype == torch.float32 else 35 * 110     # above the wide variant's CTA count
+    P = block(grid.info["n_points"], 40, "normal").to(dtype)
+    few = torch.zeros((ham.n_slots, 64), dtype=dtype, device="cuda")[:, :40]
+    kscf.kscf_points_to_slots(ham, P, few)
+    many = torch.zeros((ham.n_slots, (k + 31) // 32 * 32), dtype=dtype, device="cuda")[:, :k]
+    many[:, k - 40:] = few
+    a = kscf.kscf_hamiltonian_apply(ham, few, torch.empty_like(few))
+    b = kscf.kscf_hamiltonian_apply(ham, many, torch.empty_like(many))[:, k - 40:]
+    assert (a - b).abs().max() <= tol * a.abs().max()
