@@ -18,7 +18,8 @@ cudaError_t launch_gram_tc(const float* A, int64_t lda, const float* B, int64_t 
                            cudaStream_t st, bool symmetric_result = false, const int32_t* rowmap = nullptr);
 cudaError_t launch_rotate_tc(const float* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin,
                              int kout, bool add_identity_input, float* out, int64_t ldo, void* work,
-                             size_t work_bytes, cudaStream_t st, const int32_t* rowmap = nullptr);
+                             size_t work_bytes, cudaStream_t st, const int32_t* rowmap = nullptr,
+                             bool upper = false);
 size_t gram_tc_work_bytes(int64_t rows, int m, int n);
 size_t rotate_tc_work_bytes(int64_t rows, int kin, int kout);
 bool tc_available();
@@ -271,7 +272,7 @@ int rotate_inplace(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode
     const int32_t* map = live ? H.d_live + r0 : nullptr;
     if (mode == KSCF_GEMM_TENSOR) {
       KSCF_CUDA_TRY(launch_rotate_tc((const float*)Xr, ld, Q64, k, nr, k, k, near_identity, (float*)Xr, ld, gw.buf,
-                                     gw.bytes, st, map));
+                                     gw.bytes, st, map, upper));
       continue;
     }
     const int* only_if = nullptr;

@@ -61,6 +61,7 @@ struct TcArgs {
   const float* addsrc;             // if non-null: out = A Q + addsrc (same shape as out)
   int64_t ldadd;
   const int32_t* rowmap;           // if non-null: row r of out and addsrc is row rowmap[r]
+  int upper;                       // Q upper triangular: N tile nt needs K < (nt + 1) TN only
 };
 
 // products (A piece, B piece) kept: orders 2^0, 2^-8 (two), 2^-16 (three)
@@ -72,7 +73,8 @@ __constant__ int kProdB[6] = {0, 1, 0, 2, 1, 0};
 // K blocks of consecutive tiles through one STAGES-deep ring; the MMA thread alternates
 // between two 256-column TMEM accumulators, so the four epilogue warps drain tile i
 // (TMEM -> registers -> shared-memory transpose -> coalesced row stores) while tile i+1
-// is being multiplied.
+// is being multiplied.  With an upper triangular Q the K blocks below a tile's last column
+// are zero and left out.
 __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -85,7 +87,12 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntiles = p.m_tiles * p.n_tiles;
-  const int nk = p.kb_total;
+  // N tile of tile t: rotated by one for each round of the grid, so that a CTA meets every N
+  // tile (with a grid that is a multiple of n_tiles it would keep one, and an upper
+  // triangular Q would leave the CTAs of the first N tiles idle)
+  const int group_span = max(1, (int)gridDim.x / p.n_tiles);
+  auto n_tile = [&](int t) { return (t + (t / p.n_tiles) / group_span) % p.n_tiles; };
+  auto k_blocks = [&](int nt) { return p.upper ? min(p.kb_total, (nt + 1) * (TN / TK)) : p.kb_total; };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; s++) {
@@ -114,7 +121,7 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
       int g = 0;  // global stage counter
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const int nt = t % p.n_tiles, mt = t / p.n_tiles;
+        const int nt = n_tile(t), mt = t / p.n_tiles, nk = k_blocks(nt);
         for (int kb = 0; kb < nk; kb++, g++) {
           const int s = g % STAGES;
           if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1)) {
@@ -146,7 +153,8 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
         tc_fence_after();
         const uint32_t acc = tmem + b * TN;
         // the last column tile multiplies only its valid columns (rounded up to 16)
-        const uint32_t idesc = idesc_n(tile_n(p.n - (t % p.n_tiles) * TN, TN));
+        const int nt = n_tile(t), nk = k_blocks(nt);
+        const uint32_t idesc = idesc_n(tile_n(p.n - nt * TN, TN));
         for (int kb = 0; kb < nk; kb++, g++) {
           const int s = g % STAGES;
           ok = mbar_wait(&full[s], (g / STAGES) & 1);
@@ -178,7 +186,7 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
     float* tr = trbuf + q * 32 * 17;
     int it = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, it++) {
-      const int nt = t % p.n_tiles, mt = t / p.n_tiles;
+      const int nt = n_tile(t), mt = t / p.n_tiles;
       const int b = it & 1;
       // warp-uniform decision: tcgen05.ld below is executed by all lanes or none
       const bool ok = __all_sync(0xffffffffu, mbar_wait(&tfull[b], (it >> 1) & 1));
@@ -682,7 +690,7 @@ cudaError_t launch_gram_tc(const float* A, int64_t lda, const float* B, int64_t 
 
 cudaError_t launch_rotate_tc(const float* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin,
                              int kout, bool add_identity_input, float* out, int64_t ldo, void* work,
-                             size_t work_bytes, cudaStream_t st, const int32_t* rowmap) {
+                             size_t work_bytes, cudaStream_t st, const int32_t* rowmap, bool upper) {
   if (work_bytes < rotate_tc_work_bytes(rows, kin, kout)) return cudaErrorInvalidValue;
   if (add_identity_input && kin != kout) return cudaErrorInvalidValue;
   cudaError_t e = prepare_kernel();
@@ -732,6 +740,7 @@ cudaError_t launch_rotate_tc(const float* A, int64_t lda, const double* Q, int64
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
   const int ntiles = a.m_tiles * a.n_tiles;
+  a.upper = upper ? 1 : 0;
   tc_gemm_kernel<<<std::min(ntiles, sms), 192, SMEM_BYTES, st>>>(a), count_launch();
   return cudaGetLastError();
 }
