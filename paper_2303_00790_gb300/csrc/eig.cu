@@ -21,10 +21,11 @@
 //  3. Back-transformation Z = Q_H Z_T, column-parallel: each CTA holds a few columns of
 //     Z_T in shared memory and applies the reflectors from the last to the first.
 //
-// On this part FP64 issues one warp instruction per 64 cycles per SM sub-partition, so
-// every stage is written to keep all four FP64 pipes busy and to keep the dependent
-// chains (reductions, square roots, reciprocals) short: reciprocals and reciprocal square
-// roots start from an FP32 seed and take two Newton-Raphson steps in FP64.  All waits
+// On this part FP64 issues one warp instruction per 64 cycles per SM sub-partition (65 from one
+// dependent operation to the next, 111 with a shuffle between them), so every stage is written
+// to keep all four FP64 pipes busy and to keep the dependent chains (reductions, square roots,
+// reciprocals) short: reciprocals and reciprocal square roots start from an FP32 seed, and sums
+// over a warp are formed in integers.  All waits
 // are bounded; a wait that gives up sets a status word that the host reports.
 #include <cuda_runtime.h>
 
@@ -40,13 +41,42 @@ namespace {
 constexpr double EPS = 2.220446049250313e-16;   // 2^-52
 constexpr int NT = 256;                           // threads per CTA
 constexpr int NW = NT / 32;
+constexpr int MAX_P = 256;                        // CTAs of the tridiagonalisation
 
 // ---------------------------------------------------------------- FP64 helpers ----
 
+// A tree of five shuffles and additions costs ~560 cycles, all of it on the FP64 pipe's time for
+// 320.  The sum is therefore formed in integers: every value is aligned to the largest
+// exponent of the warp as a 58-bit integer (cut below 2^-57 of the largest value, where each
+// addition of the tree rounds at 2^-53), the integers are summed exactly as three 26-bit parts
+// by integer reductions, and the total is rounded to a double once.  Values near or beyond the
+// end of the range (Inf and NaN among them) take the tree.  Subnormal values count as zero.
 __device__ __forceinline__ double warp_sum(double v) {
+  const long long b = __double_as_longlong(v);
+  const int e = (int)(b >> 52) & 0x7ff;
+  const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  if (em >= 0x7f8) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  }
+  if (em == 0) return 0.0;
+  long long m = e ? ((b & 0xfffffffffffffLL) | (1LL << 52)) << 5 : 0;
+  m >>= min(em - e, 63);
+  if (b < 0) m = -m;
+  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x3ffffffu);
+  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 26) & 0x3ffffffu);
+  const int s2 = __reduce_add_sync(0xffffffffu, (int)(m >> 52));
+  const long long s = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+  if (s == 0) return 0.0;
+  // |s| = u 2^-z with bit 63 of u set; the leading 53 bits, rounded, and the exponent
+  unsigned long long u = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
+  const int z = __clzll((long long)u);
+  u <<= z;
+  const int ex = em + 6 - z;
+  if (ex <= 0) return 0.0;
+  const long long mag = ((long long)(ex - 1) << 52) + (long long)((u >> 11) + (u >> 10 & 1));
+  return __longlong_as_double(mag | (s & (1LL << 63)));
 }
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
@@ -188,13 +218,12 @@ struct TriArgs {
 };
 
 // Grid-wide barrier of the tridiagonalisation: arrival by a release reduction on a
-// monotonic counter, then acquire loads until all P arrivals of this step are seen (the
-// bar.sync before and after orders the other threads of the CTA).  Bounded: after
+// monotonic counter, then acquire loads until all P arrivals of this step are seen (a
+// bar.sync of the caller before and the one here after order the other threads of the CTA).  Bounded: after
 // spin_limit clock cycles, or when another CTA gave up, the status word is set and
 // false returned.
 __device__ bool tri_barrier(const TriArgs& a, unsigned target, int* s_ok) {
   if ((int)blockIdx.x == a.leave_cta) return false;
-  __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
     int ok = 1;
@@ -221,23 +250,54 @@ __device__ bool tri_barrier(const TriArgs& a, unsigned target, int* s_ok) {
 // v = x - beta e_1 (so v_0 = alpha - beta = sign(alpha)(|alpha| + |x|), v_l = x_l after it)
 // and tau = 2 / v^T v = 1 / (|x|^2 + |alpha| |x|), (I - tau v v^T) x = beta e_1.  A tail
 // negligible against max|A| = 1 (sigma <= eps^2) gives tau = 0, beta = alpha.
-// Returns tau, beta, v_0 in sc[0..2].  One thread.
+// Returns tau, beta, v_0 in sc[0..2].  One thread, on the critical path of every step: the FP32
+// seeds of |x| and tau (relative error < 2^-20) are made and widened by integer instructions,
+// off the FP64 chain, and one cubic step each (error e -> e^3) takes them to FP64: eight
+// dependent FP64 operations (two quadratic steps each made it thirteen).  Below |x|^2 = 2^100
+// (max|A| = 1, so always for finite A) everything is in the range of FP32.
+__device__ __forceinline__ float narrow(double x) {   // x >= 0: cut to FP32, below 2^-120: 0
+  const long long b = __double_as_longlong(x) >> 29;
+  return b < ((long long)(1023 - 120) << 23) ? 0.0f : __int_as_float((int)(b - ((long long)896 << 23)));
+}
+__device__ __forceinline__ double widen(float x) {    // x > 0, normal
+  return __longlong_as_double(((long long)__float_as_int(x) << 29) + ((long long)896 << 52));
+}
 __device__ __forceinline__ void reflector_scalars(double alpha, double sigma, double* sc) {
-  if (sigma <= EPS * EPS) {
+  if (__double_as_longlong(sigma) <= __double_as_longlong(EPS * EPS)) {   // sigma >= 0
     sc[0] = 0.0;
     sc[1] = alpha;
     sc[2] = 1.0;
     return;
   }
   const double x2 = fma(alpha, alpha, sigma);
-  const double y = rsqrt_pos(x2);
-  const double nrm = x2 * y;
   const double aa = fabs(alpha);
-  sc[0] = recip(fma(aa, nrm, x2));
-  sc[1] = alpha >= 0.0 ? -nrm : nrm;
-  sc[2] = alpha >= 0.0 ? aa + nrm : -(aa + nrm);
+  double nrm, tau;
+  if (__double_as_longlong(x2) < (1123LL << 52)) {
+    const float xf = narrow(x2);
+    float rf, zf;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(xf));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(zf) : "f"(fmaf(narrow(aa), xf * rf, xf)));
+    const double r0 = widen(rf), r1 = widen(zf);
+    const double t = x2 * r0, e = fma(-t, r0, 1.0);
+    nrm = fma(t * e, fma(e, 0.375, 0.5), t);
+    const double e1 = fma(-fma(aa, nrm, x2), r1, 1.0);
+    tau = fma(r1, fma(e1, e1, e1), r1);
+  } else {
+    nrm = x2 * rsqrt_pos(x2);
+    tau = recip(fma(aa, nrm, x2));
+  }
+  const bool neg = __double_as_longlong(alpha) < 0;
+  sc[0] = tau;
+  sc[1] = neg ? nrm : -nrm;
+  sc[2] = neg ? -(aa + nrm) : aa + nrm;
 }
 
+// A step is bound by latency: at n = 100 9,400 cycles, of which the grid barrier 2,400, p and the
+// row from L2 1,500, the sums' and scalars' chains the rest; at n = 850 11,600, with the passes
+// over the rows.  Sums in integers, the row formed before K, whole-warp branches and cubic steps
+// took it from 10,700 and 14,800 (564 -> 483 us and 6.6 -> 5.8 ms in all).  Sending p and the row
+// as tagged 16-byte words that every CTA polls, without a barrier, was slower (152 CTAs read
+// 27 KB a step from lines being written: 13.0 ms instead of 11.2 for the whole solver at 850).
 template <bool SMEM>
 __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
   extern __shared__ __align__(16) double smd[];
@@ -279,10 +339,7 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
   if (lane == 0) red[warp] = sg;
   __syncthreads();
   if (warp == 0) {
-    double t = lane < NW ? red[lane] : 0.0;
-    t += __shfl_xor_sync(0xffffffffu, t, 4);
-    t += __shfl_xor_sync(0xffffffffu, t, 2);
-    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    const double t = warp_sum(lane < NW ? red[lane] : 0.0);
     if (lane == 0) reflector_scalars(vc[1], t, sc);
   }
   __syncthreads();
@@ -313,22 +370,31 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       const double vpi = upd ? vp[i] : 0.0, wpi = upd ? wp[i] : 0.0;
       const bool pub = i == j + 1;
       double acc0 = 0.0, acc1 = 0.0;
-      for (int l = j + 1 + lane; l < n; l += 8 * 32) {
-        double x[8];
-#pragma unroll
-        for (int q = 0; q < 8; q++) x[q] = l + 32 * q < n ? row[l + 32 * q] : 0.0;
+      // whole warps branch, lanes beyond n multiply zeros: a branch that splits a warp costs
+      // ~50 cycles, nearly one FP64 operation
+      for (int lb = j + 1; lb < n; lb += 8 * 32) {
+        const int l = lb + lane;
+        double x[8], v[8];
 #pragma unroll
         for (int q = 0; q < 8; q++) {
-          const int ll = l + 32 * q;
-          if (ll < n) {
+          x[q] = v[q] = 0.0;
+          if (l + 32 * q < n) {
+            x[q] = row[l + 32 * q];
+            v[q] = vc[l + 32 * q];
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          if (lb + 32 * q < n) {
+            const int ll = l + 32 * q;
             double y = x[q];
-            if (upd) {
+            if (upd && ll < n) {
               y = fma(-vpi, wp[ll], fma(-wpi, vp[ll], y));
               row[ll] = y;
             }
-            if (pub) rb[ll] = y;
-            if (q & 1) acc1 = fma(y, vc[ll], acc1);
-            else acc0 = fma(y, vc[ll], acc0);
+            if (pub && ll < n) rb[ll] = y;
+            if (q & 1) acc1 = fma(y, v[q], acc1);
+            else acc0 = fma(y, v[q], acc0);
           }
         }
       }
@@ -340,54 +406,66 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     }
     if (lane == 0) red[warp] = dotp;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < NW; w++) s += red[w];
-      a.dotbuf[par * P + cta] = s;
+    if (warp == 0) {
+      const double s = warp_sum(lane < NW ? red[lane] : 0.0);
+      if (lane == 0) a.dotbuf[par * P + cta] = s;
     }
     if (!tri_barrier(a, (unsigned)P * (unsigned)(j + 1), &s_ok)) return;
     // every CTA: K = tau/2 p.v, w_j = p - K v_j, row j+1 of A^(j+1), next reflector.
-    // The first 4 NT elements of p and of the published row are loaded before the
-    // reduction of K so that the two L2 round trips overlap.
+    // The row r + 2 K v_1 v - v_1 p - p_1 v is K's multiple of v added to what is known
+    // before K, which is formed while K's sum is; the first 4 NT elements stay in registers.
     const int l0 = j + 1 + threadIdx.x;
-    double pv[4], rv[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-      const int ll = l0 + q * NT;
-      pv[q] = ll < n ? __ldcg(pb + ll) : 0.0;
-      rv[q] = ll < n ? __ldcg(rb + ll) : 0.0;
-    }
-    const double p1 = __ldcg(pb + j + 1);
-    if (warp == 0) {
-      double s = 0.0;
-      for (int c = lane; c < P; c += 32) s += __ldcg(a.dotbuf + par * P + c);
-      s = warp_sum(s);
-      if (lane == 0) sc[3] = 0.5 * tj * s;
-    }
-    __syncthreads();
-    const double K = sc[3];
-    const double v1 = vc[j + 1];
-    const double w1 = fma(-K, v1, p1);   // w_j[j+1]
-    double sig = 0.0;
-    for (int l = l0; l < n; l += 4 * NT) {
-      if (l > l0) {
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-          const int ll = l + q * NT;
-          pv[q] = ll < n ? __ldcg(pb + ll) : 0.0;
-          rv[q] = ll < n ? __ldcg(rb + ll) : 0.0;
-        }
-      }
+    const double v1 = vc[j + 1], p1 = __ldcg(pb + j + 1);
+    double pv[4], yv[4], vv[4];
+    auto load = [&](int l) {
 #pragma unroll
       for (int q = 0; q < 4; q++) {
         const int ll = l + q * NT;
+        pv[q] = yv[q] = vv[q] = 0.0;
         if (ll < n) {
-          const double vl = vc[ll];
-          const double wl = fma(-K, vl, pv[q]);
-          const double x = fma(-w1, vl, fma(-v1, wl, rv[q]));
-          wp[ll] = wl;
-          rw[ll] = x;
-          if (ll >= j + 3) sig = fma(x, x, sig);
+          pv[q] = __ldcg(pb + ll);
+          yv[q] = __ldcg(rb + ll);
+          vv[q] = vc[ll];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (l - lane + q * NT < n) yv[q] = fma(-p1, vv[q], fma(-v1, pv[q], yv[q]));
+    };
+    double part[MAX_P / 32];
+    if (warp == 0) {
+#pragma unroll
+      for (int c = 0; c < MAX_P / 32; c++) {
+        part[c] = 0.0;
+        if (c * 32 < P && c * 32 + lane < P) part[c] = __ldcg(a.dotbuf + par * P + c * 32 + lane);
+      }
+    }
+    load(l0);
+    if (warp == 0) {
+      double s = part[0];
+      if (P > 32) s += part[1];
+      if (P > 64) s += part[2] + part[3];
+      if (P > 128) s += (part[4] + part[5]) + (part[6] + part[7]);
+      s = warp_sum(s);
+      if (lane == 0) sc[3] = s;
+    }
+    const double ht = 0.5 * tj, tv = tj * v1;
+    __syncthreads();
+    const double K = ht * sc[3], c2 = tv * sc[3];
+    double sig = 0.0;
+    for (int l = l0; l < n; l += 4 * NT) {
+      if (l > l0) load(l);
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        const int ll = l + q * NT;
+        if (ll - lane < n) {   // warp-uniform; beyond n all is zero
+          const double x = fma(c2, vv[q], yv[q]), xs = ll >= j + 3 ? x : 0.0;
+          sig = fma(xs, xs, sig);
+          const double w = fma(-K, vv[q], pv[q]);
+          if (ll < n) {
+            rw[ll] = x;
+            wp[ll] = w;
+          }
         }
       }
     }
@@ -396,15 +474,14 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     __syncthreads();
     if (j <= n - 3) {
       if (warp == 0) {
-        double t = lane < NW ? red[lane] : 0.0;
-        t += __shfl_xor_sync(0xffffffffu, t, 4);
-        t += __shfl_xor_sync(0xffffffffu, t, 2);
-        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        const double t = warp_sum(lane < NW ? red[lane] : 0.0);
+        double h[3];
+        reflector_scalars(rw[j + 2], t, h);
         if (lane == 0) {
-          const double dj = rw[j + 1];
-          reflector_scalars(rw[j + 2], t, sc);
-          rw[j + 2] = sc[2];        // v_{j+1} = rw with its first element replaced
-          sc[3] = dj;
+          sc[0] = h[0];
+          sc[1] = h[1];
+          sc[3] = rw[j + 1];
+          rw[j + 2] = h[2];        // v_{j+1} = rw with its first element replaced
         }
       } else if (SMEM && (warp & 3) != 0) {
         // meanwhile the warps of the other three SM sub-partitions (whose FP64 pipes the
@@ -419,14 +496,17 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
           const int i = cta + r * P;
           double* row = rows + (int64_t)r * n;
           const double vi = vc[i], wi = wp[i];
-          const int lb = j + 2 + (it % nch) * 256 + lane;
+          const int lb = j + 2 + (it % nch) * 256;
           double x[8];
 #pragma unroll
-          for (int q = 0; q < 8; q++) x[q] = lb + 32 * q < n ? row[lb + 32 * q] : 0.0;
+          for (int q = 0; q < 8; q++) x[q] = lb + lane + 32 * q < n ? row[lb + lane + 32 * q] : 0.0;
 #pragma unroll
           for (int q = 0; q < 8; q++) {
-            const int ll = lb + 32 * q;
-            if (ll < n) row[ll] = fma(-vi, wp[ll], fma(-wi, vc[ll], x[q]));
+            if (lb + 32 * q < n) {   // warp-uniform
+              const int ll = lb + 32 * q + lane, lc = min(ll, n - 1);
+              const double y = fma(-vi, wp[lc], fma(-wi, vc[lc], x[q]));
+              if (ll < n) row[ll] = y;
+            }
           }
         }
       }
@@ -450,7 +530,6 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       a.e[n - 1] = 0.0;
       a.tau[n - 1] = 0.0;
     }
-    __syncthreads();
   }
 }
 
@@ -1268,8 +1347,6 @@ enum {
   L_TAUK, L_LAMK, L_ZH, L_INVN, L_RC, L_RS, L_IDX, L_STAT, L_NTP, L_KIDX, L_ORIG, L_COLREF, L_RP, L_RT, L_KOF,
   L_NROT, L_CAND, L_AMAX, L_TSCALE, L_BAR, L_COUNT
 };
-
-constexpr int MAX_P = 256;
 
 EigLayout eig_layout(int n) {
   EigLayout L;
