@@ -78,60 +78,70 @@ __device__ __forceinline__ double warp_sum(double v) {
   const long long mag = ((long long)(ex - 1) << 52) + (long long)((u >> 11) + (u >> 10 & 1));
   return __longlong_as_double(mag | (s & (1LL << 63)));
 }
-__device__ __forceinline__ double warp_max(double v) {
+// Sum and product over groups of G lanes (every lane of the group gets it; all lanes of the
+// warp take part).  Below a whole warp the few FP64 steps are cheaper than warp_sum's integers.
+template <int G>
+__device__ __forceinline__ double group_sum(double v) {
+  if constexpr (G == 32) return warp_sum(v);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_prod(double v) {
+template <int G>
+__device__ __forceinline__ double group_prod(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = G / 2; o > 0; o >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// 1/x.  For 2^-1000 < |x| < 2^1000: the reciprocal of the leading mantissa in FP32
-// (relative error < 2^-22) scaled by the exponent, then two Newton-Raphson steps
-// r <- r + r (1 - |x| r), each squaring the relative error.  Other x: IEEE division.
+// 1/x.  For 2^-1000 <= |x| < 2^1000: the reciprocal of the leading mantissa bits in FP32
+// (relative error < 2^-21) with the exponent put in by integer instructions, then one cubic
+// step r <- r + r (e + e^2), e = 1 - x r, which leaves e^3 < 2^-63: three FP64 operations.
+// Comparing and converting in FP64 and two Newton-Raphson steps took eight.  Other x: IEEE
+// division.
 __device__ __forceinline__ double recip(double x) {
-  const double ax = fabs(x);
-  if (!(ax > 0x1p-1000 && ax < 0x1p+1000)) return 1.0 / x;
-  const long long bits = __double_as_longlong(ax);
-  const int e = (int)((bits >> 52) & 0x7ff) - 1023;
-  const float m = __int_as_float(0x3f800000 | (int)((bits >> 29) & 0x7fffff));   // [1, 2)
-  double r = (double)__frcp_rn(m) * __longlong_as_double((long long)(1023 - e) << 52);
-  r = fma(r, fma(-ax, r, 1.0), r);
-  r = fma(r, fma(-ax, r, 1.0), r);
-  return copysign(r, x);
+  const long long b = __double_as_longlong(x);
+  const int e = (int)(b >> 52) & 0x7ff;
+  if ((unsigned)(e - 23) >= 2000u) return 1.0 / x;
+  float f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__int_as_float(0x3f800000 | ((int)(b >> 29) & 0x7fffff))));
+  const double r = __longlong_as_double(((long long)__float_as_int(f) << 29) + ((long long)(896 + 1023 - e) << 52) |
+                                        (b & (1LL << 63)));
+  const double q = fma(-x, r, 1.0);
+  return fma(r, fma(q, q, q), r);
 }
 
-// 1/sqrt(x) for 2^-1000 < x < 2^1000: FP32 seed of the even-exponent mantissa in [1, 4),
-// then two Newton-Raphson steps r <- r + r (1 - x r^2) / 2.  Other x: IEEE sqrt.
+// 1/sqrt(x) for 2^-1000 <= x < 2^1000: FP32 seed of the mantissa in [1, 4) with an even
+// exponent, then one cubic step r <- r + r (e/2 + 3 e^2/8), e = 1 - x r^2.  Other x: IEEE sqrt.
 __device__ __forceinline__ double rsqrt_pos(double x) {
-  if (!(x > 0x1p-1000 && x < 0x1p+1000)) return 1.0 / sqrt(x);
-  const long long bits = __double_as_longlong(x);
-  int e = (int)((bits >> 52) & 0x7ff) - 1023;
-  float m = __int_as_float(0x3f800000 | (int)((bits >> 29) & 0x7fffff));
-  if (e & 1) {   // odd exponent: mantissa in [2, 4), even exponent
-    m *= 2.0f;
-    e -= 1;
-  }
-  double r = (double)rsqrtf(m) * __longlong_as_double((long long)(1023 - e / 2) << 52);
-  double t = x * r;
-  r = fma(0.5 * r, fma(-t, r, 1.0), r);
-  t = x * r;
-  r = fma(0.5 * r, fma(-t, r, 1.0), r);
-  return r;
+  const long long b = __double_as_longlong(x);
+  const int e = (int)(b >> 52);   // sign included
+  if ((unsigned)(e - 23) >= 2000u) return 1.0 / sqrt(x);
+  const int odd = (e & 1) ^ 1;    // biased by 1023: an even e is an odd exponent
+  float f;
+  asm("rsqrt.approx.ftz.f32 %0, %1;"
+      : "=f"(f)
+      : "f"(__int_as_float((0x3f800000 + (odd << 23)) | ((int)(b >> 29) & 0x7fffff))));
+  const double r = __longlong_as_double(((long long)__float_as_int(f) << 29) +
+                                        ((long long)(896 - ((e - 1023 - odd) >> 1)) << 52));
+  const double t = x * r, q = fma(-t, r, 1.0);
+  return fma(r * q, fma(q, 0.375, 0.5), r);
 }
+__device__ __forceinline__ double sqrt_nonneg(double x) { return x > 0.0 ? x * rsqrt_pos(x) : 0.0; }
 
+// Largest of the CTA's values, all >= 0 (ordered like their bits; FP64 comparisons would take
+// the FP64 pipe's time)
 __device__ __forceinline__ double block_max(double v, double* red) {
-  v = warp_max(v);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = red[0];
+  long long m = __double_as_longlong(v);
 #pragma unroll
-  for (int w = 1; w < NW; w++) t = fmax(t, red[w]);
-  return t;
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = __longlong_as_double(m);
+  __syncthreads();
+  m = __double_as_longlong(red[0]);
+#pragma unroll
+  for (int w = 1; w < NW; w++) m = max(m, __double_as_longlong(red[w]));
+  return __longlong_as_double(m);
 }
 
 // exclusive prefix sum of per-thread counts over the CTA; returns the thread's offset and
@@ -718,51 +728,43 @@ __global__ void __launch_bounds__(NT) dc_deflate_kernel(DcArgs a, int depth) {
   if (C0 - A0 >= 2) dc_deflate_node(a, A0, B0, C0);
 }
 
-// Secular equation 1 + rho sum_i z_i^2 / (d_i - lambda) = 0, one warp per root j of the K
+// Secular equation 1 + rho sum_i z_i^2 / (d_i - lambda) = 0, G lanes per root j of the K
 // kept poles d_0 < ... < d_{K-1}.  Root j lies in (d_j, d_{j+1}) (j < K-1) or in
-// (d_{K-1}, d_{K-1} + rho |z|^2].  The origin is the nearer pole (sign of the secular
-// function at the midpoint); lambda = d_o + tau with tau bracketed in (lo, hi).  Each
-// iteration evaluates psi (poles i <= j) and phi (poles i > j) with their derivatives,
-// replaces each by a + b / (d_pole - tau) through the current point (pole d_j for psi,
-// d_{j+1} for phi; one pole for the last root) and takes the root of that model inside
-// the bracket, else bisects.  Stops when |g| is below its rounding bound or the bracket
-// has collapsed.
+// (d_{K-1}, d_{K-1} + rho |z|^2].  The first evaluation, at the midpoint, also decides the
+// origin, the nearer pole (sign of the secular function); lambda = d_o + tau with tau
+// bracketed in (lo, hi).  Each iteration evaluates psi (poles i <= j) and phi (poles i > j)
+// with their derivatives, replaces each by a + b / (d_pole - tau) through the current point
+// (pole d_j for psi, d_{j+1} for phi; the last root has no phi) and takes the root of that
+// model inside the bracket, else bisects.  Stops when |g| is below its rounding bound or the
+// bracket has collapsed.  Called by whole warps; lanes with j >= K work on the last root and
+// write nothing.
+//
+// Bound by the FP64 pipe: ten operations per pole and ~50 for the model, which every lane of a
+// root repeats.  So a root of a large merge has a warp, but a merge of at most 32 rows gives
+// each root four lanes (eight poles each): the model's operations then serve eight roots at
+// once (25 rows: 143 -> 60 us for the merge).  With an evaluation less (the midpoint's is used
+// by the model) and cheap reciprocals, 100 rows: 86 -> 44 us.
+template <int G>
 __device__ void dc_secular_root(const DcArgs& a, int A0, int B0, int K, int j) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (G - 1);
+  const bool live = j < K;
+  j = min(j, K - 1);
   const double rho = 2.0 * fabs(a.es[B0 - 1]);
   const double* dk = a.dk + A0;
   const double* zz = a.zz + A0;
-  int o;
-  double lo, hi;
-  if (j < K - 1) {
-    const double mid = 0.5 * (dk[j + 1] - dk[j]);
-    double f = 0.0;
-    for (int i = lane; i < K; i += 32) f += zz[i] * recip((dk[i] - dk[j]) - mid);
-    f = 1.0 + rho * warp_sum(f);
-    if (f >= 0.0) {
-      o = j;
-      lo = 0.0;
-      hi = mid;
-    } else {
-      o = j + 1;
-      lo = -mid;
-      hi = 0.0;
-    }
-  } else {
-    double s = 0.0;
-    for (int i = lane; i < K; i += 32) s += zz[i];
-    o = K - 1;
-    lo = 0.0;
-    hi = rho * warp_sum(s);
-  }
-  const double dorg = dk[o];
-  const double dl = dk[j] - dorg;
-  const double dr = j < K - 1 ? dk[j + 1] - dorg : 0.0;
-  double tau = 0.5 * (lo + hi);
+  const bool inner = j < K - 1;
+  double zs = 0.0;
+  for (int i = lane; i < K; i += G) zs += zz[i];
+  zs = rho * group_sum<G>(zs);
+  const double gap = inner ? dk[j + 1] - dk[j] : 0.0;
+  int o = j;
+  double lo = 0.0, hi = inner ? gap : zs, dl = 0.0, dr = gap;
+  double dorg = dk[j], tau = 0.5 * hi;
   bool conv = false;
+  const double Kd = (double)K;
   for (int it = 0; it < 64; it++) {
     double ps = 0.0, dps = 0.0, ph = 0.0, dph = 0.0;
-    for (int i = lane; i < K; i += 32) {
+    for (int i = lane; i < K; i += G) {
       const double r = recip((dk[i] - dorg) - tau);
       const double t1 = zz[i] * r;
       if (i <= j) {
@@ -773,49 +775,54 @@ __device__ void dc_secular_root(const DcArgs& a, int A0, int B0, int K, int j) {
         dph = fma(t1, r, dph);
       }
     }
-    ps = rho * warp_sum(ps);
-    dps = rho * warp_sum(dps);
-    ph = rho * warp_sum(ph);
-    dph = rho * warp_sum(dph);
+    ps = rho * group_sum<G>(ps);
+    dps = rho * group_sum<G>(dps);
+    ph = rho * group_sum<G>(ph);
+    dph = rho * group_sum<G>(dph);
     const double g = 1.0 + ps + ph;
-    if (g < 0.0) lo = tau;
-    else hi = tau;
-    const double bound = 8.0 * EPS * (K * (fabs(ps) + fabs(ph)) + 1.0);
-    if (fabs(g) <= bound || hi - lo <= 2.0 * EPS * fmax(fabs(lo), fabs(hi))) {
-      conv = true;
-      break;
-    }
-    double nt = lo - 1.0;   // outside the bracket: bisect unless the model gives a root
-    if (j < K - 1) {
-      const double el = dl - tau, er = dr - tau;
-      const double B1 = dps * el * el, A1 = ps - dps * el;
-      const double B2 = dph * er * er, A2 = ph - dph * er;
-      const double c = 1.0 + A1 + A2;
-      const double bq = c * (dl + dr) + B1 + B2;
-      const double cq = c * dl * dr + B1 * dr + B2 * dl;
-      const double disc = bq * bq - 4.0 * c * cq;
-      if (disc >= 0.0) {
-        const double sq = sqrt(disc);
-        if (c != 0.0) {
-          const double x1 = (bq + copysign(sq, bq)) * 0.5 * recip(c);
-          if (x1 > lo && x1 < hi) nt = x1;
-          if (x1 != 0.0) {
-            const double x2 = cq * recip(c * x1);
-            if (x2 > lo && x2 < hi) nt = x2;
-          }
-        } else if (bq != 0.0) {
-          nt = cq * recip(bq);
+    // a converged root keeps its values while others of the warp go on
+    if (!conv) {
+      const bool neg = __double_as_longlong(g) < 0;
+      if (it == 0 && inner) {
+        hi = tau;
+        if (neg) {   // nearer to d_{j+1}
+          o = j + 1;
+          dorg = dk[j + 1];
+          dl = -gap;
+          dr = 0.0;
+          tau = -tau;
+          lo = tau;
+          hi = 0.0;
         }
+      } else if (neg) {
+        lo = tau;
+      } else {
+        hi = tau;
       }
-    } else {
-      const double el = dl - tau;
-      const double B1 = dps * el * el;
-      const double c = g - B1 * recip(el);
-      if (c != 0.0) nt = dl + B1 * recip(c);
+      const double bound = fma(8.0 * EPS * Kd, fabs(ps) + fabs(ph), 8.0 * EPS);
+      conv = fabs(g) <= bound || hi - lo <= 2.0 * EPS * fmax(fabs(lo), fabs(hi));
+      if (!conv) {
+        // c + B1 / (dl - x) + B2 / (dr - x) = 0; one of dl, dr is 0
+        const double el = dl - tau, er = dr - tau;
+        const double s1 = dps * el, s2 = dph * er;
+        const double B1 = s1 * el, B2 = s2 * er;
+        const double c = (g - s1) - s2;
+        const double bq = fma(c, dl + dr, B1 + B2);
+        const double cq = fma(B1, dr, B2 * dl);
+        const double disc = fma(bq, bq, -4.0 * c * cq);
+        double nt = lo - 1.0;   // outside the bracket: bisect unless the model gives a root
+        if (disc >= 0.0) {
+          const double h = 0.5 * (bq + copysign(sqrt_nonneg(disc), bq));
+          const double x1 = h * recip(c), x2 = cq * recip(h);
+          if (x1 > lo && x1 < hi) nt = x1;
+          if (x2 > lo && x2 < hi) nt = x2;
+        }
+        tau = nt > lo && nt < hi ? nt : 0.5 * (lo + hi);
+      }
     }
-    tau = nt > lo && nt < hi ? nt : 0.5 * (lo + hi);
+    if (__all_sync(0xffffffffu, conv)) break;
   }
-  if (lane == 0) {
+  if (lane == 0 && live) {
     a.orig[A0 + j] = o;
     a.tauk[A0 + j] = tau;
     a.lamk[A0 + j] = dorg + tau;
@@ -823,29 +830,35 @@ __device__ void dc_secular_root(const DcArgs& a, int A0, int B0, int K, int j) {
   }
 }
 
-__global__ void __launch_bounds__(NT) dc_secular_kernel(DcArgs a, int depth) {
+// one warp per SM sub-partition
+constexpr int SEC_NT = 128;
+__global__ void __launch_bounds__(SEC_NT) dc_secular_kernel(DcArgs a, int depth) {
   int A0, B0, C0;
   node_range(a.n, depth, blockIdx.y, &A0, &B0, &C0);
   if (C0 - A0 < 2) return;
   const int K = a.Kof[A0];
-  const int j = blockIdx.x * NW + (threadIdx.x >> 5);
-  if (j < K) dc_secular_root(a, A0, B0, K, j);
+  const int j = blockIdx.x * (SEC_NT / 32) + (threadIdx.x >> 5);
+  if (j < K) dc_secular_root<32>(a, A0, B0, K, j);
 }
 
 // Gu-Eisenstat: zh_i^2 = prod_j (lambda_j - d_i) / (rho prod_{j != i} (d_j - d_i)), the
-// sign of z_i; lambda_j - d_i = (d_{o_j} - d_i) + tau_j.  One warp per kept pole.
+// sign of z_i; lambda_j - d_i = (d_{o_j} - d_i) + tau_j.  G lanes per kept pole; called by
+// whole warps.
+template <int G>
 __device__ void dc_zhat_one(const DcArgs& a, int A0, int B0, int K, int i) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (G - 1);
+  const bool live = i < K;
+  i = min(i, K - 1);
   const double rho = 2.0 * fabs(a.es[B0 - 1]);
   const double* dk = a.dk + A0;
   const double di = dk[i];
   double p = 1.0;
-  for (int jj = lane; jj < K; jj += 32) {
+  for (int jj = lane; jj < K; jj += G) {
     const double num = (dk[min(max(a.orig[A0 + jj], 0), K - 1)] - di) + a.tauk[A0 + jj];
     p *= jj == i ? num : num * recip(dk[jj] - di);
   }
-  p = warp_prod(p);
-  if (lane == 0) a.zh[A0 + i] = copysign(sqrt(fabs(p) * recip(rho)), a.zk[A0 + i]);
+  p = group_prod<G>(p);
+  if (lane == 0 && live) a.zh[A0 + i] = copysign(sqrt(fabs(p) * recip(rho)), a.zk[A0 + i]);
 }
 
 __global__ void __launch_bounds__(NT) dc_zhat_kernel(DcArgs a, int depth) {
@@ -854,21 +867,24 @@ __global__ void __launch_bounds__(NT) dc_zhat_kernel(DcArgs a, int depth) {
   if (C0 - A0 < 2) return;
   const int K = a.Kof[A0];
   const int i = blockIdx.x * NW + (threadIdx.x >> 5);
-  if (i < K) dc_zhat_one(a, A0, B0, K, i);
+  if (i < K) dc_zhat_one<32>(a, A0, B0, K, i);
 }
 
-// 1 / |u_j|, u_j[i] = zh_i / (d_i - lambda_j).  One warp per root.
+// 1 / |u_j|, u_j[i] = zh_i / (d_i - lambda_j).  G lanes per root; called by whole warps.
+template <int G>
 __device__ void dc_colnorm_one(const DcArgs& a, int A0, int K, int j) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & (G - 1);
+  const bool live = j < K;
+  j = min(j, K - 1);
   const double* dk = a.dk + A0;
   const double dorg = dk[min(max(a.orig[A0 + j], 0), K - 1)], tau = a.tauk[A0 + j];
   double s = 0.0;
-  for (int i = lane; i < K; i += 32) {
+  for (int i = lane; i < K; i += G) {
     const double u = a.zh[A0 + i] * recip((dk[i] - dorg) - tau);
     s = fma(u, u, s);
   }
-  s = warp_sum(s);
-  if (lane == 0) a.invn[A0 + j] = rsqrt_pos(s);
+  s = group_sum<G>(s);
+  if (lane == 0 && live) a.invn[A0 + j] = rsqrt_pos(s);
 }
 
 __global__ void __launch_bounds__(NT) dc_colnorm_kernel(DcArgs a, int depth) {
@@ -877,7 +893,7 @@ __global__ void __launch_bounds__(NT) dc_colnorm_kernel(DcArgs a, int depth) {
   if (C0 - A0 < 2) return;
   const int K = a.Kof[A0];
   const int j = blockIdx.x * NW + (threadIdx.x >> 5);
-  if (j < K) dc_colnorm_one(a, A0, K, j);
+  if (j < K) dc_colnorm_one<32>(a, A0, K, j);
 }
 
 // order-preserving integer key of a double
@@ -1034,66 +1050,94 @@ __global__ void __launch_bounds__(NT) dc_rotperm_kernel(DcArgs a, int depth) {
 }
 
 // Merges of at most 32 rows (the lowest depths, many small merges): one CTA per merge runs
-// every phase above in one launch, the phases separated by __syncthreads (the per-merge
-// arrays live in global memory and stay in L1/L2), the two block products element-wise.
-constexpr int DC_SMALL = 32;
+// every phase above in one launch, the phases separated by __syncthreads, the two block
+// products element-wise.  The block of Z, the merge matrices and the per-merge arrays are in
+// shared memory (a phase that reads what the last one stored would wait for L2 otherwise).
+constexpr int DC_SMALL = 32, DC_SLD = DC_SMALL + 1;
 __global__ void __launch_bounds__(NT) dc_small_kernel(DcArgs a, int depth) {
   __shared__ unsigned long long key[DC_SMALL];
   __shared__ int ref[DC_SMALL];
+  __shared__ double mat[3][DC_SMALL * DC_SLD];
+  __shared__ double vec[12][DC_SMALL];
+  __shared__ int ivec[9][DC_SMALL];
+  __shared__ int one[2];
   int A0, B0, C0;
   node_range(a.n, depth, blockIdx.x, &A0, &B0, &C0);
   const int N = C0 - A0, n1 = B0 - A0;
   if (N < 2) return;
-  const int warp = threadIdx.x >> 5;
-  const int64_t ld = a.ldz;
-  dc_deflate_node(a, A0, B0, C0);
+  const int tid = threadIdx.x;
+  // the merge as a problem of its own: rows 0 .. N-1, split at n1
+  DcArgs b = a;
+  b.ldz = DC_SLD;
+  b.es = a.es + A0;
+  b.Z = mat[0];
+  b.Zt = mat[1];
+  b.M = mat[2];
+  double** const dv[12] = {&b.lam, &b.Ds, &b.zs, &b.dk, &b.zk, &b.zz, &b.tauk, &b.lamk, &b.zh, &b.invn, &b.rc, &b.rsn};
+#pragma unroll
+  for (int q = 0; q < 12; q++) *dv[q] = vec[q];
+  int** const iv[9] = {&b.idx, &b.stat, &b.ntp, &b.kidx, &b.orig, &b.colref, &b.rp, &b.rt, &b.cand};
+#pragma unroll
+  for (int q = 0; q < 9; q++) *iv[q] = ivec[q];
+  b.Kof = &one[0];
+  b.nrot = &one[1];
+  for (int q = tid; q < N * N; q += NT) {
+    const int col = q / N, r = q - col * N;
+    mat[0][r + col * DC_SLD] = a.Z[(int64_t)(A0 + r) + (int64_t)(A0 + col) * a.ldz];
+  }
+  if (tid < N) b.lam[tid] = a.lam[A0 + tid];
   __syncthreads();
-  const int K = a.Kof[A0];
-  for (int j = warp; j < K; j += NW) dc_secular_root(a, A0, B0, K, j);
+  dc_deflate_node(b, 0, n1, N);
   __syncthreads();
-  for (int i = warp; i < K; i += NW) dc_zhat_one(a, A0, B0, K, i);
+  const int K = one[0];
+  // four lanes per root or pole: 128 threads for the 32 rows
+  if (K > 0 && tid < 4 * DC_SMALL && (tid & ~31) < 4 * K) dc_secular_root<4>(b, 0, n1, K, tid >> 2);
   __syncthreads();
-  for (int j = warp; j < K; j += NW) dc_colnorm_one(a, A0, K, j);
+  if (K > 0 && tid < 4 * DC_SMALL && (tid & ~31) < 4 * K) dc_zhat_one<4>(b, 0, n1, K, tid >> 2);
   __syncthreads();
-  dc_order_node(a, A0, N, key, ref);
+  if (K > 0 && tid < 4 * DC_SMALL && (tid & ~31) < 4 * K) dc_colnorm_one<4>(b, 0, K, tid >> 2);
   __syncthreads();
-  const bool rot = a.nrot[A0] > 0;
-  for (int q = threadIdx.x; q < N * N; q += NT) {
+  dc_order_node(b, 0, N, key, ref);
+  __syncthreads();
+  const bool rot = one[1] > 0;
+  for (int q = tid; q < N * N; q += NT) {
     const int t = q / N, col = q - t * N;
     double dorg, tau, inv;
-    const int r = dc_col_ref(a, A0, N, K, col, &dorg, &tau, &inv);
-    const double v = dc_m_value(a, A0, K, t, r, dorg, tau, inv);
-    if (rot) a.Zt[(int64_t)(A0 + t) * ld + A0 + col] = v;
-    else a.M[(int64_t)(A0 + min(max(a.idx[A0 + t], 0), N - 1)) * ld + A0 + col] = v;
+    const int r = dc_col_ref(b, 0, N, K, col, &dorg, &tau, &inv);
+    const double v = dc_m_value(b, 0, K, t, r, dorg, tau, inv);
+    if (rot) b.Zt[t * DC_SLD + col] = v;
+    else b.M[min(max(b.idx[t], 0), N - 1) * DC_SLD + col] = v;
   }
   __syncthreads();
   if (rot)
-    for (int col = threadIdx.x; col < N; col += NT) dc_rotperm_col(a, A0, N, col);
+    for (int col = tid; col < N; col += NT) dc_rotperm_col(b, 0, N, col);
   __syncthreads();
-  // Zt[r, col] = sum_k Z[r, k] M[k, col] over the block of row r
-  for (int q = threadIdx.x; q < N * N; q += NT) {
+  // Z[r, col] = sum_k Z[r, k] M[k, col] over the block of row r
+  for (int q = tid; q < N * N; q += NT) {
     const int col = q / N, r = q - col * N;
     const int k0 = r < n1 ? 0 : n1, k1 = r < n1 ? n1 : N;
-    double acc = 0.0;
-    for (int k = k0; k < k1; k++)
-      acc = fma(a.Z[(int64_t)(A0 + r) + (int64_t)(A0 + k) * ld], a.M[(int64_t)(A0 + k) * ld + A0 + col], acc);
-    a.Zt[(int64_t)(A0 + r) + (int64_t)(A0 + col) * ld] = acc;
+    double acc0 = 0.0, acc1 = 0.0;
+    for (int k = k0; k + 1 < k1; k += 2) {
+      acc0 = fma(b.Z[r + k * DC_SLD], b.M[k * DC_SLD + col], acc0);
+      acc1 = fma(b.Z[r + (k + 1) * DC_SLD], b.M[(k + 1) * DC_SLD + col], acc1);
+    }
+    if ((k1 - k0) & 1) acc0 = fma(b.Z[r + (k1 - 1) * DC_SLD], b.M[(k1 - 1) * DC_SLD + col], acc0);
+    a.Z[(int64_t)(A0 + r) + (int64_t)(A0 + col) * a.ldz] = acc0 + acc1;
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < N * N; q += NT) {
-    const int col = q / N, r = q - col * N;
-    a.Z[(int64_t)(A0 + r) + (int64_t)(A0 + col) * ld] = a.Zt[(int64_t)(A0 + r) + (int64_t)(A0 + col) * ld];
-  }
+  if (tid < N) a.lam[A0 + tid] = b.lam[tid];
 }
 
 // Batched FP64 GEMM of the merge: Zt[a:b, a:c] = Z[a:b, a:b] M[a:b, a:c] and
-// Zt[b:c, a:c] = Z[b:c, b:c] M[b:c, a:c] (Z, Zt column-major, M row-major).  32 x 64
-// output tile per CTA (small tiles: the top merges have only a few hundred tiles for 152
-// SMs), 2 x 4 per thread, k-steps of 16 through shared memory.  blockIdx.x: column tile;
+// Zt[b:c, a:c] = Z[b:c, b:c] M[b:c, a:c] (Z, Zt column-major, M row-major).  TM x TN output
+// tile per CTA, TM / 16 x TN / 16 per thread, k-steps of 16 through shared memory: 32 x 64
+// (the top merges have only a few hundred such tiles), or 16 x 16 where 32 x 64 tiles would
+// leave SMs idle (n = 100: 47 -> 10 us for the top merge).  blockIdx.x: column tile;
 // blockIdx.y: row tile (first the rt1 tiles of block 1, then those of block 2);
 // blockIdx.z: node.
-constexpr int GTM = 32, GTN = 64, GTK = 16;
+constexpr int GTK = 16;
+template <int GTM, int GTN>
 __global__ void __launch_bounds__(NT) dc_gemm_kernel(DcArgs a, int depth, int rt1) {
+  constexpr int RM = GTM / 16, RN = GTN / 16;
   __shared__ __align__(16) double As[GTK][GTM];
   __shared__ __align__(16) double Bs[GTK][GTN];
   int A0, B0, C0;
@@ -1113,11 +1157,11 @@ __global__ void __launch_bounds__(NT) dc_gemm_kernel(DcArgs a, int depth, int rt
   if (row0 >= kd || col0 >= N) return;
   const int64_t ld = a.ldz;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[2][4];
+  double acc[RM][RN];
 #pragma unroll
-  for (int i = 0; i < 2; i++)
+  for (int i = 0; i < RM; i++)
 #pragma unroll
-    for (int jj = 0; jj < 4; jj++) acc[i][jj] = 0.0;
+    for (int jj = 0; jj < RN; jj++) acc[i][jj] = 0.0;
   for (int k0 = 0; k0 < kd; k0 += GTK) {
     for (int q = threadIdx.x; q < GTK * GTM; q += NT) {
       const int kk = q / GTM, rr = q % GTM;
@@ -1137,24 +1181,24 @@ __global__ void __launch_bounds__(NT) dc_gemm_kernel(DcArgs a, int depth, int rt
     if (!__syncthreads_or(nz)) continue;
 #pragma unroll
     for (int kk = 0; kk < GTK; kk++) {
-      const double a0 = As[kk][ty * 2], a1 = As[kk][ty * 2 + 1];
-      double bv[4];
+      double av[RM], bv[RN];
 #pragma unroll
-      for (int jj = 0; jj < 4; jj++) bv[jj] = Bs[kk][tx + 16 * jj];
+      for (int i = 0; i < RM; i++) av[i] = As[kk][ty * RM + i];
 #pragma unroll
-      for (int jj = 0; jj < 4; jj++) {
-        acc[0][jj] = fma(a0, bv[jj], acc[0][jj]);
-        acc[1][jj] = fma(a1, bv[jj], acc[1][jj]);
-      }
+      for (int jj = 0; jj < RN; jj++) bv[jj] = Bs[kk][tx + 16 * jj];
+#pragma unroll
+      for (int jj = 0; jj < RN; jj++)
+#pragma unroll
+        for (int i = 0; i < RM; i++) acc[i][jj] = fma(av[i], bv[jj], acc[i][jj]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 2; i++) {
-    const int gr = row0 + ty * 2 + i;
+  for (int i = 0; i < RM; i++) {
+    const int gr = row0 + ty * RM + i;
     if (gr >= kd) continue;
 #pragma unroll
-    for (int jj = 0; jj < 4; jj++) {
+    for (int jj = 0; jj < RN; jj++) {
       const int gc = col0 + tx + 16 * jj;
       if (gc < N) a.Zt[(int64_t)(r0 + gr) + (int64_t)(A0 + gc) * ld] = acc[i][jj];
     }
@@ -1505,14 +1549,17 @@ cudaError_t launch_sym_eig(double* A, int64_t lda, int n, double* w, void* work,
     while (p2 < Nmax) p2 <<= 1;
     const int rw = (Nmax + NW - 1) / NW;
     dc_deflate_kernel<<<nodes, NT, 0, st>>>(a, d), count_launch();
-    dc_secular_kernel<<<dim3(rw, nodes), NT, 0, st>>>(a, d), count_launch();
+    dc_secular_kernel<<<dim3((Nmax + SEC_NT / 32 - 1) / (SEC_NT / 32), nodes), SEC_NT, 0, st>>>(a, d), count_launch();
     dc_zhat_kernel<<<dim3(rw, nodes), NT, 0, st>>>(a, d), count_launch();
     dc_colnorm_kernel<<<dim3(rw, nodes), NT, 0, st>>>(a, d), count_launch();
     dc_order_kernel<<<nodes, NT, (size_t)p2 * 12, st>>>(a, d, p2), count_launch();
     dc_build_m_kernel<<<dim3((Nmax + 31) / 32, (Nmax + 63) / 64, nodes), NT, 0, st>>>(a, d), count_launch();
     dc_rotperm_kernel<<<dim3((Nmax + NT - 1) / NT, nodes), NT, 0, st>>>(a, d), count_launch();
-    const int rt = (Nmax / 2 + 1 + GTM - 1) / GTM;
-    dc_gemm_kernel<<<dim3((Nmax + GTN - 1) / GTN, 2 * rt, nodes), NT, 0, st>>>(a, d, rt), count_launch();
+    const int rt = (Nmax / 2 + 1 + 31) / 32, ct = (Nmax + 63) / 64, rt16 = (Nmax / 2 + 1 + 15) / 16;
+    if (2 * rt * ct * nodes < nsm)
+      dc_gemm_kernel<16, 16><<<dim3((Nmax + 15) / 16, 2 * rt16, nodes), NT, 0, st>>>(a, d, rt16), count_launch();
+    else
+      dc_gemm_kernel<32, 64><<<dim3(ct, 2 * rt, nodes), NT, 0, st>>>(a, d, rt), count_launch();
     const int cb = (int)std::min<int64_t>(256, ((int64_t)Nmax * Nmax + NT - 1) / NT);
     dc_copy_kernel<<<dim3(cb, nodes), NT, 0, st>>>(a, d), count_launch();
   }
