@@ -33,6 +33,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "fp64.cuh"
 #include "kscf_internal.h"
 
 namespace kscf {
@@ -45,39 +46,6 @@ constexpr int MAX_P = 256;                        // CTAs of the tridiagonalisat
 
 // ---------------------------------------------------------------- FP64 helpers ----
 
-// A tree of five shuffles and additions costs ~560 cycles, all of it on the FP64 pipe's time for
-// 320.  The sum is therefore formed in integers: every value is aligned to the largest
-// exponent of the warp as a 58-bit integer (cut below 2^-57 of the largest value, where each
-// addition of the tree rounds at 2^-53), the integers are summed exactly as three 26-bit parts
-// by integer reductions, and the total is rounded to a double once.  Values near or beyond the
-// end of the range (Inf and NaN among them) take the tree.  Subnormal values count as zero.
-__device__ __forceinline__ double warp_sum(double v) {
-  const long long b = __double_as_longlong(v);
-  const int e = (int)(b >> 52) & 0x7ff;
-  const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if (em >= 0x7f8) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-  }
-  if (em == 0) return 0.0;
-  long long m = e ? ((b & 0xfffffffffffffLL) | (1LL << 52)) << 5 : 0;
-  m >>= min(em - e, 63);
-  if (b < 0) m = -m;
-  const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x3ffffffu);
-  const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 26) & 0x3ffffffu);
-  const int s2 = __reduce_add_sync(0xffffffffu, (int)(m >> 52));
-  const long long s = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
-  if (s == 0) return 0.0;
-  // |s| = u 2^-z with bit 63 of u set; the leading 53 bits, rounded, and the exponent
-  unsigned long long u = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
-  const int z = __clzll((long long)u);
-  u <<= z;
-  const int ex = em + 6 - z;
-  if (ex <= 0) return 0.0;
-  const long long mag = ((long long)(ex - 1) << 52) + (long long)((u >> 11) + (u >> 10 & 1));
-  return __longlong_as_double(mag | (s & (1LL << 63)));
-}
 // Sum and product over groups of G lanes (every lane of the group gets it; all lanes of the
 // warp take part).  Below a whole warp the few FP64 steps are cheaper than warp_sum's integers.
 template <int G>
@@ -94,39 +62,6 @@ __device__ __forceinline__ double group_prod(double v) {
   return v;
 }
 
-// 1/x.  For 2^-1000 <= |x| < 2^1000: the reciprocal of the leading mantissa bits in FP32
-// (relative error < 2^-21) with the exponent put in by integer instructions, then one cubic
-// step r <- r + r (e + e^2), e = 1 - x r, which leaves e^3 < 2^-63: three FP64 operations.
-// Comparing and converting in FP64 and two Newton-Raphson steps took eight.  Other x: IEEE
-// division.
-__device__ __forceinline__ double recip(double x) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)(b >> 52) & 0x7ff;
-  if ((unsigned)(e - 23) >= 2000u) return 1.0 / x;
-  float f;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__int_as_float(0x3f800000 | ((int)(b >> 29) & 0x7fffff))));
-  const double r = __longlong_as_double(((long long)__float_as_int(f) << 29) + ((long long)(896 + 1023 - e) << 52) |
-                                        (b & (1LL << 63)));
-  const double q = fma(-x, r, 1.0);
-  return fma(r, fma(q, q, q), r);
-}
-
-// 1/sqrt(x) for 2^-1000 <= x < 2^1000: FP32 seed of the mantissa in [1, 4) with an even
-// exponent, then one cubic step r <- r + r (e/2 + 3 e^2/8), e = 1 - x r^2.  Other x: IEEE sqrt.
-__device__ __forceinline__ double rsqrt_pos(double x) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)(b >> 52);   // sign included
-  if ((unsigned)(e - 23) >= 2000u) return 1.0 / sqrt(x);
-  const int odd = (e & 1) ^ 1;    // biased by 1023: an even e is an odd exponent
-  float f;
-  asm("rsqrt.approx.ftz.f32 %0, %1;"
-      : "=f"(f)
-      : "f"(__int_as_float((0x3f800000 + (odd << 23)) | ((int)(b >> 29) & 0x7fffff))));
-  const double r = __longlong_as_double(((long long)__float_as_int(f) << 29) +
-                                        ((long long)(896 - ((e - 1023 - odd) >> 1)) << 52));
-  const double t = x * r, q = fma(-t, r, 1.0);
-  return fma(r * q, fma(q, 0.375, 0.5), r);
-}
 __device__ __forceinline__ double sqrt_nonneg(double x) { return x > 0.0 ? x * rsqrt_pos(x) : 0.0; }
 
 // Largest of the CTA's values, all >= 0 (ordered like their bits; FP64 comparisons would take
@@ -239,11 +174,12 @@ __device__ bool tri_barrier(const TriArgs& a, unsigned target, int* s_ok) {
     int ok = 1;
     volatile int* to = a.status;
     const long long t0 = clock64();
-    for (;;) {
+    for (unsigned tries = 1;; tries++) {
       unsigned c;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(a.bar) : "memory");
       if (c >= target) break;
-      if (*to != 0 || clock64() - t0 > a.spin_limit) {
+      // (the status word is another trip to L2: not between every two looks at the counter)
+      if (tries % 32 == 0 && (*to != 0 || clock64() - t0 > a.spin_limit)) {
         atomicExch(a.status, 1);
         ok = 0;
         break;
@@ -302,17 +238,20 @@ __device__ __forceinline__ void reflector_scalars(double alpha, double sigma, do
   sc[2] = neg ? -(aa + nrm) : aa + nrm;
 }
 
-// A step is bound by latency: at n = 100 9,400 cycles, of which the grid barrier 2,400, p and the
-// row from L2 1,500, the sums' and scalars' chains the rest; at n = 850 11,600, with the passes
-// over the rows.  Sums in integers, the row formed before K, whole-warp branches and cubic steps
-// took it from 10,700 and 14,800 (564 -> 483 us and 6.6 -> 5.8 ms in all).  Sending p and the row
-// as tagged 16-byte words that every CTA polls, without a barrier, was slower (152 CTAs read
-// 27 KB a step from lines being written: 13.0 ms instead of 11.2 for the whole solver at 850).
+// A step is bound by latency: at n = 100 8,500 cycles, of which the grid barrier 2,200, p and the
+// row from L2 1,600, the reflector's scalars 1,700, the row's two sums 900, p.v and its sum over
+// the CTA 1,200.  Sums in integers, the row formed before K, warp 0 left to the scalars while the
+// others hold the vectors, whole-warp branches and cubic steps took it there from 10,700 cycles,
+// and from 14,800 to 10,500 at n = 850 (564 -> 430 us and 6.6 -> 5.2 ms for all steps).  Sending
+// p and the row as tagged 16-byte words that every CTA polls, without a barrier, was slower (152
+// CTAs read 27 KB a step from lines being written: 13.0 ms instead of 11.2 for the whole solver
+// at 850).
 template <bool SMEM>
 __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
+  constexpr int VT = NT - 32, VE = 4;
   extern __shared__ __align__(16) double smd[];
   __shared__ double red[NW];
-  __shared__ double sc[4];
+  __shared__ double sc[4], s_k[2];
   __shared__ int s_ok;
   const int n = a.n, P = a.P, cta = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -321,8 +260,8 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
   double* vc = smd;
   double* vp = smd + n;
   double* wp = smd + 2 * n;
-  double* rw = a.rwg ? a.rwg + (int64_t)cta * n : smd + 3 * n;
-  double* rows = smd + (a.rwg ? 3 : 4) * n;
+  double* rw = !SMEM && a.rwg ? a.rwg + (int64_t)cta * n : smd + 3 * n;
+  double* rows = smd + 4 * n;   // SMEM only (then rw is in shared memory as well)
   const int nown = cta < n ? (n - cta + P - 1) / P : 0;
   if (n == 1) {
     if (cta == 0 && threadIdx.x == 0) {
@@ -366,13 +305,15 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       a.tau[0] = tj;
     }
   }
+  int r0 = 0, wcta = 0;   // first owned row > j, the CTA of row j + 1
   for (int j = 0; j <= n - 2; j++) {
+    if (r0 < nown && cta + r0 * P <= j) r0++;
+    if (++wcta == P) wcta = 0;
     const int par = j & 1;
     double* pb = a.pbuf + (int64_t)par * n;
     double* rb = a.rowbuf + (int64_t)par * n;
     // pass over the owned rows i > j: A^(j) = A^(j-1) - v w^T - w v^T, p_i = tau_j A^(j)_i. v_j
     double dotp = 0.0;
-    const int r0 = j + 1 > cta ? (j + 1 - cta + P - 1) / P : 0;
     const bool upd = !SMEM && j >= 1;   // shared-memory rows were updated in the last step
     for (int r = r0 + warp; r < nown; r += NW) {
       const int i = cta + r * P;
@@ -423,14 +364,15 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     if (!tri_barrier(a, (unsigned)P * (unsigned)(j + 1), &s_ok)) return;
     // every CTA: K = tau/2 p.v, w_j = p - K v_j, row j+1 of A^(j+1), next reflector.
     // The row r + 2 K v_1 v - v_1 p - p_1 v is K's multiple of v added to what is known
-    // before K, which is formed while K's sum is; the first 4 NT elements stay in registers.
-    const int l0 = j + 1 + threadIdx.x;
-    const double v1 = vc[j + 1], p1 = __ldcg(pb + j + 1);
-    double pv[4], yv[4], vv[4];
+    // before K.  Warp 0 sums K, the others have the vectors (the first VE VT elements in
+    // registers) and form the known part meanwhile.
+    const int l0 = j + 1 + (int)threadIdx.x - 32;
+    double pv[VE], yv[VE], vv[VE];
     auto load = [&](int l) {
+      const double v1 = vc[j + 1], p1 = __ldcg(pb + j + 1);
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int ll = l + q * NT;
+      for (int q = 0; q < VE; q++) {
+        const int ll = l + q * VT;
         pv[q] = yv[q] = vv[q] = 0.0;
         if (ll < n) {
           pv[q] = __ldcg(pb + ll);
@@ -439,52 +381,75 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; q++)
-        if (l - lane + q * NT < n) yv[q] = fma(-p1, vv[q], fma(-v1, pv[q], yv[q]));
+      for (int q = 0; q < VE; q++) {
+        if (l - lane + q * VT < n) yv[q] = fma(-p1, vv[q], fma(-v1, pv[q], yv[q]));
+        asm volatile("" : "+d"(yv[q]));   // formed here, not after the barrier
+      }
     };
-    double part[MAX_P / 32];
     if (warp == 0) {
+      double part[MAX_P / 32];
 #pragma unroll
       for (int c = 0; c < MAX_P / 32; c++) {
         part[c] = 0.0;
         if (c * 32 < P && c * 32 + lane < P) part[c] = __ldcg(a.dotbuf + par * P + c * 32 + lane);
       }
-    }
-    load(l0);
-    if (warp == 0) {
+      const double ht = 0.5 * tj, tv = tj * vc[j + 1];
       double s = part[0];
       if (P > 32) s += part[1];
       if (P > 64) s += part[2] + part[3];
       if (P > 128) s += (part[4] + part[5]) + (part[6] + part[7]);
       s = warp_sum(s);
-      if (lane == 0) sc[3] = s;
+      const double K = ht * s, c2 = tv * s;
+      if (lane == 0) {
+        s_k[0] = K;
+        s_k[1] = c2;
+      }
+    } else {
+      load(l0);
     }
-    const double ht = 0.5 * tj, tv = tj * v1;
     __syncthreads();
-    const double K = ht * sc[3], c2 = tv * sc[3];
-    double sig = 0.0;
-    for (int l = l0; l < n; l += 4 * NT) {
-      if (l > l0) load(l);
+    const double K = s_k[0];
+    if (warp != 0) {
+      const double c2 = s_k[1];
+      double sig = 0.0;
+      auto row = [&](int l) {
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        const int ll = l + q * NT;
-        if (ll - lane < n) {   // warp-uniform; beyond n all is zero
-          const double x = fma(c2, vv[q], yv[q]), xs = ll >= j + 3 ? x : 0.0;
-          sig = fma(xs, xs, sig);
-          const double w = fma(-K, vv[q], pv[q]);
-          if (ll < n) {
-            rw[ll] = x;
-            wp[ll] = w;
+        for (int q = 0; q < VE; q++) {
+          const int ll = l + q * VT;
+          if (ll - lane < n) {   // warp-uniform; beyond n all is zero
+            const double x = fma(c2, vv[q], yv[q]), xs = ll >= j + 3 ? x : 0.0;
+            sig = fma(xs, xs, sig);
+            if (ll < n) rw[ll] = x;
           }
         }
+      };
+      for (int l = l0 + VE * VT; l - lane < n; l += VE * VT) {   // beyond the registers
+        load(l);
+        row(l);
+#pragma unroll
+        for (int q = 0; q < VE; q++)
+          if (l + q * VT < n) wp[l + q * VT] = fma(-K, vv[q], pv[q]);
       }
+      if (l0 + VE * VT - lane < n) load(l0);
+      row(l0);
+      sig = warp_sum(sig);
+      if (lane == 0) red[warp] = sig;
     }
-    sig = warp_sum(sig);
-    if (lane == 0) red[warp] = sig;
     __syncthreads();
+    if (warp != 0) {   // w, which the scalars do not need
+#pragma unroll
+      for (int q = 0; q < VE; q++) {
+        const int ll = l0 + q * VT;
+        if (ll - lane < n) {
+          const double w = fma(-K, vv[q], pv[q]);
+          if (ll < n) wp[ll] = w;
+        }
+      }
+      asm volatile("bar.sync 1, %0;" ::"r"(VT) : "memory");
+    }
     if (j <= n - 3) {
       if (warp == 0) {
-        const double t = warp_sum(lane < NW ? red[lane] : 0.0);
+        const double t = warp_sum(lane > 0 && lane < NW ? red[lane] : 0.0);
         double h[3];
         reflector_scalars(rw[j + 2], t, h);
         if (lane == 0) {
@@ -498,7 +463,7 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
         // scalar chain does not use) update the owned rows i >= j+2 to A^(j+1) over the
         // columns l >= j+2, in items of one row x 256 columns
         const int u = (warp >> 2) * 3 + (warp & 3) - 1;
-        const int rs = j + 2 > cta ? (j + 2 - cta + P - 1) / P : 0;
+        const int rs = r0 < nown && cta + r0 * P == j + 1 ? r0 + 1 : r0;
         const int nch = (n - (j + 2) + 255) / 256;
         const int items = (nown - rs) * nch;
         for (int it = u; it < items; it += NW - NW / 4) {
@@ -522,7 +487,6 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       }
       __syncthreads();
       tj = sc[0];
-      const int wcta = (j + 1) % P;
       if (cta == wcta) {
         for (int l = j + 2 + threadIdx.x; l < n; l += NT) a.V[l + (int64_t)(j + 1) * n] = rw[l];
         if (threadIdx.x == 0) {
