@@ -279,11 +279,12 @@ __device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.bar) : "memory");
     int ok = 1;
     const long long t0 = clock64();
-    for (;;) {
+    for (unsigned tries = 1;; tries++) {
       unsigned n;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(c.bar) : "memory");
       if (n >= target) break;
-      if (*(volatile int*)c.status != 0 || clock64() - t0 > c.spin_limit) {
+      // (the status word is another trip to L2: not between every two looks at the counter)
+      if (tries % 32 == 0 && (*(volatile int*)c.status != 0 || clock64() - t0 > c.spin_limit)) {
         atomicExch(c.status, 1);
         ok = 0;
         break;
