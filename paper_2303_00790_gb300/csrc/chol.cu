@@ -17,7 +17,10 @@
 // tile in phase B, in every CTA).  The two triangular recurrences are those of
 // the textbook blocked Cholesky and triangular inversion (Golub & Van Loan, Matrix
 // Computations, Sec. 4.2 and 3.1); every tile product is FP64 FMA.  On this part FP64
-// runs at ~1 TFLOP/s, so the kernel is FP64-ALU bound: 2 k^3 / 3 flop in total.
+// runs at ~1 TFLOP/s (2 k^3 / 3 flop in total: 0.41 ms at k = 850), but the chain through the
+// block rows is longer: 5,400 cycles to load the tiles, 19,000 for the triangular solve, 12,000
+// for the next diagonal tile's update, 49,000 for its 32 pivots and 2,200 per grid barrier (it
+// was 110,000 together with 61,000 for the pivots and 5,400 per barrier: k = 850 1.42 -> 1.11 ms).
 //
 // A pivot counts as failed when it is not above tau_c = S_cc * max((c + 8) u64, floor_rel)
 // (or is not finite): (c + 8) u64 S_cc is the rounding level of a Cholesky pivot, so an
@@ -29,6 +32,7 @@
 
 #include <algorithm>
 
+#include "fp64.cuh"
 #include "kscf_internal.h"
 
 namespace kscf {
@@ -48,7 +52,7 @@ struct CholArgs {
   double* RC;     // kp: 1 / R_cc of the diagonal tiles factored ahead by CTA 0
   double* out;    // k x k output (may alias S): R^-1 upper, zero below
   int64_t ldo;
-  unsigned* bar;  // [0] arrival count, [1] generation, [2] failed pivot of a tile factored ahead (1-based) or 0
+  unsigned* bar;  // [0] arrival count, [2] failed pivot of a tile factored ahead (1-based) or 0
   int* status;    // [0] first failed pivot (1-based column) or 0, [1] barrier timeout
   double floor_rel;
   long long spin_limit;
@@ -57,34 +61,31 @@ struct CholArgs {
 
 __device__ __forceinline__ double ld(const double* p) { return __ldcg(p); }
 
-// Grid-wide barrier for a cooperative launch; false when a wait gave up (or another CTA
-// reported that it did).
-__device__ bool grid_sync(const CholArgs& a) {
+// Grid-wide barrier for a cooperative launch: release arrivals on a monotonic counter (zero at
+// launch; *target is the arrivals this barrier waits for), acquire polls.  False when a wait
+// gave up (or another CTA reported that it did).  A counter that the last CTA resets, with a
+// generation word, cost three trips to L2 in a row (5,400 cycles a barrier).
+__device__ bool grid_sync(const CholArgs& a, unsigned* target) {
   __shared__ int s_ok;
   if ((int)blockIdx.x == a.leave_cta) return false;
+  *target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = a.bar + 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
     volatile int* timeout = a.status + 1;
-    const unsigned g = *gen;
-    __threadfence();
     int ok = 1;
-    if (atomicAdd(a.bar, 1u) == gridDim.x - 1) {
-      atomicExch(a.bar, 0u);
-      __threadfence();
-      atomicAdd(a.bar + 1, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*gen == g) {
-        if (*timeout != 0 || clock64() - t0 > a.spin_limit) {
-          atomicExch(a.status + 1, 1);
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
+    const long long t0 = clock64();
+    for (unsigned tries = 1;; tries++) {
+      unsigned c;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(a.bar) : "memory");
+      if (c >= *target) break;
+      // (the status word is another trip to L2: not between every two looks)
+      if (tries % 32 == 0 && (*timeout != 0 || clock64() - t0 > a.spin_limit)) {
+        atomicExch(a.status + 1, 1);
+        ok = 0;
+        break;
       }
     }
-    __threadfence();
     s_ok = ok;
   }
   __syncthreads();
@@ -105,66 +106,75 @@ struct TileSmem {
   int fail;
 };
 
-// 1/d for a normal d in (2^-1000, 2^1000): an FP32 seed from the leading 23 mantissa bits
-// (relative error < 2^-22), then two Newton-Raphson steps r <- r + r (1 - d r) in FP64,
-// each of which squares the relative error (2^-44, then below the FP64 rounding).
-__device__ __forceinline__ double recip_pos(double d) {
-  const long long bits = __double_as_longlong(d);
-  const int e = (int)((bits >> 52) & 0x7ff) - 1023;
-  const float mf = __int_as_float(0x3f800000 | (int)((bits >> 29) & 0x7fffff));
-  const int fb = __float_as_int(__frcp_rn(mf));          // 1/mf in (0.5, 1]
-  const long long fe = ((fb >> 23) & 0xff) - 127;
-  double r = __longlong_as_double(((fe - e + 1023) << 52) | ((long long)(fb & 0x7fffff) << 29));
-  r = fma(r, fma(-d, r, 1.0), r);
-  r = fma(r, fma(-d, r, 1.0), r);
-  return r;
-}
-
 __device__ __forceinline__ void bar_factor() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-// Warps 0-3 (one per SM sub-partition, each FP64 pipe busy): factor the diagonal tile in
-// sm.T.  Lane p holds row p; warp w owns columns m = w + 4i.  Square-root-free elimination
-// (pivot c: T_pm -= (T_cp / d_c) T_cm for c < p <= m, d_c = T_cc), so that only a
-// reciprocal lies on the pivot-to-pivot chain; then R_pm = T_pm / sqrt(d_p).  A failed
-// pivot is left in sm.fail.
-__device__ void factor_diag4(const CholArgs& a, int j, TileSmem& sm) {
-  const int w = threadIdx.x >> 5, p = threadIdx.x & 31;
+// The CTA's eight warps (two per SM sub-partition) factor the diagonal tile in sm.T.  Lane p
+// holds row p; warp w owns columns m = w + 8i.  Square-root-free elimination (pivot c:
+// T_pm -= (T_cp / d_c) T_cm for c < p <= m, d_c = T_cc), so that only a reciprocal lies on the
+// pivot-to-pivot chain; then R_pm = T_pm / sqrt(d_p).  A failed pivot is left in sm.fail.
+//
+// Bound by that chain.  So the warp of the next pivot updates its column first and takes the
+// reciprocal and the check (against a threshold made beforehand, by integer comparisons: FP64
+// ones take the pipe's time) while the other warp of its sub-partition updates the rest; with
+// four warps of eight columns each did both in turn (1,950 cycles a pivot).  The loop is
+// rolled, t[0] always the leftmost column left: 32 unrolled pivots are code that is fetched
+// once per tile and run once.
+__device__ void factor_diag(const CholArgs& a, int j, TileSmem& sm) {
+  const int w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), p = threadIdx.x & 31;
   volatile int* fail = &sm.fail;
-  double t[8];
+  double t[4];
 #pragma unroll
-  for (int i = 0; i < 8; i++) t[i] = sm.T[p + (w + 4 * i) * LDT];
-#pragma unroll
+  for (int i = 0; i < 4; i++) t[i] = sm.T[p + (w + 8 * i) * LDT];
+  // pivot p must be above tau: bits compare like the values (tau > 0; a negative or zero pivot
+  // and NaN fail as well)
+  const double tau = fmax(sm.dg[p] * fmax((double)(j * TB + p + 8) * 0x1.0p-53, a.floor_rel), 0x1.0p-1000);
+  const long long tau_bits = __double_as_longlong(tau), top_bits = __double_as_longlong(0x1.0p+1000);
+  // d: the pivot in lane c; all lanes of the warp compute, lane c writes
+  auto pivot = [&](int c, double d) {
+    const double r = recip(d);
+    if (p == c) {
+      const long long b = __double_as_longlong(d);
+      const bool ok = b > tau_bits && b < top_bits;
+      if (!ok) *fail = c;
+      sm.dinv[c] = ok ? r : 0.0;
+      sm.piv[c] = d;
+    }
+  };
+  if (w == 0) pivot(0, t[0]);
+#pragma unroll 1
   for (int c = 0; c < TB; c++) {
     double* buf = sm.xb[c & 1];
+    const int cc = c & 7, m0 = w + (c & ~7);   // t[i] is column m0 + 8 i
     if (p == c) {
 #pragma unroll
-      for (int i = 0; i < 8; i++)
-        if (w + 4 * i >= c) buf[w + 4 * i] = t[i];
-      if (w == (c & 3)) {
-        const double d = t[c >> 2];
-        const int gc = j * TB + c;
-        const double tau = fmax(sm.dg[c] * fmax((double)(gc + 8) * 0x1.0p-53, a.floor_rel), 0x1.0p-1000);
-        if (!(d > tau) || !(d < 0x1.0p+1000)) {
-          *fail = c;
-          sm.dinv[c] = 0.0;
-        } else {
-          sm.dinv[c] = recip_pos(d);
-        }
-        sm.piv[c] = d;
-      }
+      for (int i = 0; i < 4; i++)
+        if (m0 + 8 * i < TB) buf[m0 + 8 * i] = t[i];   // (columns left of c are not read)
     }
-    bar_factor();
-    if (*fail >= 0) return;
-    if (p > c) {
-      const double g = buf[p] * sm.dinv[c];
+    __syncthreads();
+    const double bp = buf[p], dv = sm.dinv[c];
+    double x[4];
 #pragma unroll
-      for (int i = 0; i < 8; i++)
-        if (w + 4 * i > c && p <= w + 4 * i) t[i] = fma(-g, buf[w + 4 * i], t[i]);
+    for (int i = 0; i < 4; i++) x[i] = m0 + 8 * i < TB ? buf[m0 + 8 * i] : 0.0;
+    // a faster warp may have marked pivot c + 1 already: every warp leaves at the marked one
+    const int f = *fail;
+    if (f >= 0 && f <= c) return;
+    const double g = p > c ? bp * dv : 0.0;
+    if (w > cc) t[0] = fma(-g, x[0], t[0]);
+    if (w == cc + 1) pivot(c + 1, t[0]);
+    if (m0 + 8 < TB) t[1] = fma(-g, x[1], t[1]);
+    if (cc == 7 && w == 0 && c + 1 < TB) pivot(c + 1, t[1]);
+    if (m0 + 16 < TB) t[2] = fma(-g, x[2], t[2]);
+    if (m0 + 24 < TB) t[3] = fma(-g, x[3], t[3]);
+    if (cc == 7) {
+      sm.T[p + m0 * LDT] = p <= m0 ? t[0] : 0.0;   // this warp's column of the eight
+      t[0] = t[1];
+      t[1] = t[2];
+      t[2] = t[3];
     }
   }
   const double r = rsqrt(sm.piv[p]);
 #pragma unroll
-  for (int i = 0; i < 8; i++) sm.T[p + (w + 4 * i) * LDT] = p <= w + 4 * i ? t[i] * r : 0.0;
+  for (int i = 0; i < 4; i++) sm.T[p + (w + 8 * i) * LDT] *= r;
   if (w == 0) sm.rc[p] = r;
 }
 
@@ -232,11 +242,50 @@ __device__ void tile_update(int kp, double* C, const double* P, bool trans_p, co
   __syncthreads();
 }
 
+// C -= P^T P on and above the diagonal of the diagonal tile C (the part that is read): 528
+// elements instead of 1024, two per thread and a third for sixteen.
+__device__ void diag_update(int kp, double* C, const double* P, double* Ps) {
+  const int t = threadIdx.x;
+  for (int q = t; q < TB * TB; q += NTHR) {
+    const int lo = q & (TB - 1), hi = q >> 5;
+    Ps[lo * LDT + hi] = ld(P + at(kp, lo, hi));
+  }
+  __syncthreads();
+  // elements in the order (0,0) (0,1) (1,1) (0,2) ...: e = c (c + 1) / 2 + r
+  int rr[2], cc[2];
+  double acc[2];
+#pragma unroll
+  for (int u = 0; u < 2; u++) {
+    const int e = t + u * NTHR;
+    int c = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+    while ((c + 1) * (c + 2) / 2 <= e) c++;
+    while (c * (c + 1) / 2 > e) c--;
+    cc[u] = c;
+    rr[u] = e - c * (c + 1) / 2;
+    acc[u] = ld(C + at(kp, rr[u], cc[u]));
+  }
+#pragma unroll 8
+  for (int p = 0; p < TB; p++)
+#pragma unroll
+    for (int u = 0; u < 2; u++) acc[u] = fma(-Ps[p * LDT + rr[u]], Ps[p * LDT + cc[u]], acc[u]);
+#pragma unroll
+  for (int u = 0; u < 2; u++) C[at(kp, rr[u], cc[u])] = acc[u];
+  if (t >= NTHR - (TB * (TB + 1) / 2 - 2 * NTHR)) {   // the last sixteen: column 31, rows 16 .. 31
+    const int r = t - (NTHR - TB), c = TB - 1;
+    double s = ld(C + at(kp, r, c));
+#pragma unroll 8
+    for (int p = 0; p < TB; p++) s = fma(-Ps[p * LDT + r], Ps[p * LDT + c], s);
+    C[at(kp, r, c)] = s;
+  }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
   __shared__ TileSmem sm;
   __shared__ double Ps[TB * LDT];
   __shared__ double Qs[TB * LDT];
   const int kp = a.kp, nt = a.nt;
+  unsigned arrivals = 0;
   const int64_t n2 = (int64_t)kp * kp;
   const int64_t tid = (int64_t)blockIdx.x * NTHR + threadIdx.x, nth = (int64_t)gridDim.x * NTHR;
   // phase 0: A = upper triangle of S (identity padding), W = 0, D = diag(S)
@@ -248,7 +297,7 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
     a.W[q] = 0.0;
   }
   for (int64_t q = tid; q < kp; q += nth) a.D[q] = q < a.k ? a.S[q + q * a.lds] : 1.0;
-  if (!grid_sync(a)) return;
+  if (!grid_sync(a, &arrivals)) return;
   for (int j = 0; j < nt; j++) {
     // phase B: the diagonal tile's factor.  Block row 0 (and a one-CTA grid): every CTA
     // factors it (the same arithmetic everywhere); later block rows: CTA 0 factored it at
@@ -272,7 +321,7 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
       if (threadIdx.x < TB) sm.dg[threadIdx.x] = ld(a.D + r0 + threadIdx.x);
       if (threadIdx.x == 0) sm.fail = -1;
       __syncthreads();
-      if (threadIdx.x < 128) factor_diag4(a, j, sm);
+      factor_diag(a, j, sm);
       __syncthreads();
       if (sm.fail >= 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) a.status[0] = j * TB + sm.fail + 1;
@@ -297,7 +346,7 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
       }
       __syncthreads();
     }
-    if (!grid_sync(a)) return;
+    if (!grid_sync(a, &arrivals)) return;
     // phase C.  Item 0 is the next diagonal tile (j+1, j+1), whose only update this is: with
     // more than one CTA, CTA 0 takes it alone and then factors the tile while the other CTAs
     // work through items 1, 2, ...
@@ -313,7 +362,10 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
         while (lp * (lp + 1) / 2 > it) lp--;
         const int mp = it - lp * (lp + 1) / 2;
         const int m = j + 1 + mp, l = j + 1 + lp;
-        tile_update(kp, a.A + at(kp, m * TB, l * TB), a.A + at(kp, j * TB, m * TB), true,
+        if (m == l)
+          diag_update(kp, a.A + at(kp, m * TB, m * TB), a.A + at(kp, j * TB, m * TB), Ps);
+        else
+          tile_update(kp, a.A + at(kp, m * TB, l * TB), a.A + at(kp, j * TB, m * TB), true,
                     a.A + at(kp, j * TB, l * TB), Ps, Qs);
       } else {
         const int q = it - n_trail;
@@ -334,7 +386,7 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
       if (threadIdx.x < TB) sm.dg[threadIdx.x] = ld(a.D + r1 + threadIdx.x);
       if (threadIdx.x == 0) sm.fail = -1;
       __syncthreads();
-      if (threadIdx.x < 128) factor_diag4(a, j + 1, sm);
+      factor_diag(a, j + 1, sm);
       __syncthreads();
       if (sm.fail < 0) {
         for (int q = threadIdx.x; q < TB * TB; q += NTHR) {
@@ -346,7 +398,7 @@ __global__ void __launch_bounds__(NTHR) chol_inv_kernel(CholArgs a) {
         a.bar[2] = (unsigned)((j + 1) * TB + sm.fail + 1);
       }
     }
-    if (!grid_sync(a)) return;
+    if (!grid_sync(a, &arrivals)) return;
   }
   // output: R^-1 (upper) into out, zero below the diagonal
   const int64_t nk = (int64_t)a.k * a.k;
