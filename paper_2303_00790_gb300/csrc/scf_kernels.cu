@@ -353,7 +353,13 @@ __device__ __forceinline__ uint32_t abs_hw(double v) { return (uint32_t)__double
 // Byte offsets (in the fixed-point field) of the face neighbours of slot s: nb[2 ax + sg] +-
 // 8 k stride is the slot at distance k beyond the brick's face.  A missing brick points into
 // the zeros behind the field (kCgZeroSlots), so that the star needs no predicates; 32-bit
-// offsets from one base keep the address arithmetic out of the loads.
+// offsets from one base keep the address arithmetic out of the loads.  The base is a brick before
+// the field (cg_base), so that no offset is negative (that of a high neighbour starts below the
+// neighbour's first slot).
+template <int B>
+__device__ __forceinline__ const char* cg_base(const int2* rf) {
+  return (const char*)(rf - B * B * B);
+}
 template <int B>
 __device__ __forceinline__ void cg_faces(const int32_t* nbr, int s, uint32_t zero, uint32_t* nb) {
   constexpr int B3 = B * B * B;
@@ -362,17 +368,17 @@ __device__ __forceinline__ void cg_faces(const int32_t* nbr, int s, uint32_t zer
 #pragma unroll
   for (int f = 0; f < 6; f++) {
     const int n = __ldg(nbr + brick * 6 + f);
-    nb[f] = n >= 0 ? 8u * (uint32_t)(n * B3 + li + ((f & 1) ? -B : B) * stride[f >> 1]) : zero;
+    nb[f] = n >= 0 ? 8u * (uint32_t)((n + 1) * B3 + li + ((f & 1) ? -B : B) * stride[f >> 1]) : zero + 8u * B3;
   }
 }
 
-// 831600 h^2 Lap_h of the fixed-point field f at slot s
+// 831600 h^2 Lap_h of the fixed-point field (f: its cg_base) at slot s
 template <int B>
 __device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* nb, int nbs) {
   const int li = s & (B * B * B - 1);
   const int l[3] = {li % B, (li / B) % B, li / (B * B)};
   const int stride[3] = {1, B, B * B};
-  const uint32_t own = 8u * (uint32_t)s;
+  const uint32_t own = 8u * (uint32_t)(s + B * B * B);
   FixAcc acc = {0, 0};
   fix_mad(acc, FIX_W0, *(const int2*)(f + own));
   uint32_t face[6];
@@ -438,7 +444,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
       uint32_t nb[6];
       if (on) cg_faces<B>(c.a.nbr, sv[k], zero, nb);
 #pragma unroll
-      for (int q = 0; q < 6; q++) s_face[(q * NPT + k) * nt + tid] = on ? nb[q] : zero;
+      for (int q = 0; q < 6; q++) s_face[(q * NPT + k) * nt + tid] = on ? nb[q] : zero + 8u * (B * B * B);
       xv[k] = on ? c.x[sv[k]] : 0.0;
       rv[k] = on ? c.r[sv[k]] : 0.0;
       pv[k] = on && !c.first ? c.p[sv[k]] : 0.0;
@@ -480,11 +486,11 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
     each([&](int k, int s, double&, double& r, double& p, double& q) {
       FixAcc t;
       if constexpr (NPT > 0) {
-        t = cg_star<B>((const char*)c.rf, s, s_face + k * nt + tid, NPT * nt);
+        t = cg_star<B>(cg_base<B>(c.rf), s, s_face + k * nt + tid, NPT * nt);
       } else {
         uint32_t nb[6];
         cg_faces<B>(c.a.nbr, s, zero, nb);
-        t = cg_star<B>((const char*)c.rf, s, nb, 1);
+        t = cg_star<B>(cg_base<B>(c.rf), s, nb, 1);
       }
       const double pn = fma(beta, p, r);
       double qn = fma(sc, fix_value(t), beta * q);
