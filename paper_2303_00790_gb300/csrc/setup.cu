@@ -122,24 +122,32 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   return z;
 }
 
-__device__ __forceinline__ double normal_entry(uint64_t key, uint64_t n) {
-  const uint64_t q = n >> 1;
-  const uint64_t a = mix64(key + (2 * q + 1) * 0x9E3779B97F4A7C15ull);
-  const uint64_t b = mix64(key + (2 * q + 2) * 0x9E3779B97F4A7C15ull);
-  const double u1 = ((double)(a >> 11) + 1.0) * 0x1.0p-53;
-  const double u2 = (double)(b >> 11) * 0x1.0p-53;
-  const double r = sqrt(-2.0 * log(u1));
-  return (n & 1) ? r * sinpi(2.0 * u2) : r * cospi(2.0 * u2);
-}
-
+// One thread per pair of entries (2q, 2q + 1) of a slot's row: both share the radius, and no
+// warp evaluates a sine for one half of its lanes and a cosine for the other.  Bound by the FP64
+// pipe (log, sqrt, sinpi, cospi): 45,025 points x 100 columns in 350 us, 677 us with one thread
+// per entry.
 template <typename T>
 __global__ void random_kernel(T* X, int64_t ld, int k, const int64_t* lex, int64_t n_slots, uint64_t key) {
+  const int pairs = k / 2 + 1;   // a row starts at an even or an odd entry
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n_slots * k) return;
-  const int64_t s = idx / k;
-  const int j = (int)(idx - s * k);
+  if (idx >= n_slots * pairs) return;
+  const int64_t s = idx / pairs;
+  const int t = (int)(idx - s * pairs);
   const int64_t p = lex[s];
-  X[s * ld + j] = p < 0 ? T(0) : (T)normal_entry(key, (uint64_t)p * (uint64_t)k + (uint64_t)j);
+  const uint64_t n0 = p < 0 ? 0 : (uint64_t)p * (uint64_t)k, q = (n0 >> 1) + (uint64_t)t;
+  const int64_t j = (int64_t)(2 * q) - (int64_t)n0;   // -1 .. k
+  T v0 = T(0), v1 = T(0);
+  if (p >= 0 && j < k) {
+    const uint64_t a = mix64(key + (2 * q + 1) * 0x9E3779B97F4A7C15ull);
+    const uint64_t b = mix64(key + (2 * q + 2) * 0x9E3779B97F4A7C15ull);
+    const double u1 = ((double)(a >> 11) + 1.0) * 0x1.0p-53;
+    const double u2 = (double)(b >> 11) * 0x1.0p-53;
+    const double r = sqrt(-2.0 * log(u1));
+    v0 = (T)(r * cospi(2.0 * u2));
+    v1 = (T)(r * sinpi(2.0 * u2));
+  }
+  if (j >= 0 && j < k) X[s * ld + j] = v0;
+  if (j + 1 < k) X[s * ld + j + 1] = v1;
 }
 
 static uint64_t mix64_host(uint64_t z) {
@@ -152,8 +160,8 @@ static uint64_t mix64_host(uint64_t z) {
 }
 
 cudaError_t launch_random(const Ham& H, void* X, int64_t ld, int k, int dtype, uint64_t seed, cudaStream_t st) {
-  const int64_t n = H.grid.n_slots * k;
-  if (n == 0) return cudaSuccess;
+  const int64_t n = H.grid.n_slots * (k / 2 + 1);
+  if (H.grid.n_slots == 0 || k == 0) return cudaSuccess;
   const uint64_t key = mix64_host(seed);
   if (dtype == KSCF_F64)
     random_kernel<double><<<blocks_for(n, 256), 256, 0, st>>>((double*)X, ld, k, H.d_lex, H.grid.n_slots, key), count_launch();
