@@ -202,7 +202,21 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
           orow[r] = (p.rowmap && ir < p.rows) ? (int64_t)__ldg(p.rowmap + ir) : ir;
         }
       }
-      for (int c0 = 0; c0 < TN; c0 += 16) {
+      // the addends of the first sixteen columns; those of the next sixteen are loaded before
+      // this block's are used (narrow outputs are bound by their latency)
+      const int jj = lane & 15, rh = lane >> 4;
+      const int64_t ir0 = (int64_t)mt * TM + q * 32 + rh;
+      float add[16], nadd[16];
+      auto addends = [&](int c0, float* d) {
+        const int j = nt * TN + c0 + jj;
+#pragma unroll
+        for (int r = 0; r < 16; r++)
+          d[r] = p.addsrc && j < p.n && ir0 + 2 * r < p.rows ? p.addsrc[orow[r] * p.ldadd + j] : 0.0f;
+      };
+      addends(0, add);
+      const int nc = min(TN, p.n - nt * TN);   // columns of this tile
+      for (int c0 = 0; c0 < nc; c0 += 16) {
+        if (c0 + 16 < nc) addends(c0 + 16, nadd);
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + b * TN + c0, v);
         // transpose the 32 x 16 block through shared memory: each store instruction then
@@ -210,27 +224,19 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
 #pragma unroll
         for (int c = 0; c < 16; c++) tr[lane * 17 + c] = v[c];
         __syncwarp();
-        const int jj = lane & 15, rh = lane >> 4;
         const int j = nt * TN + c0 + jj;
         if (j < p.n) {
-          const int64_t ir0 = (int64_t)mt * TM + q * 32 + rh;
-          float add[16];
-          // the sixteen addends are loaded before any store (out may alias addsrc; each
-          // element is read and written by this lane only), so their latencies overlap
+          // out may alias addsrc: each element is read and written by this lane only
 #pragma unroll
           for (int r = 0; r < 16; r++) {
-            const int64_t ir = ir0 + 2 * r;
-            add[r] = (p.addsrc && ir < p.rows) ? p.addsrc[orow[r] * p.ldadd + j] : 0.0f;
-          }
-#pragma unroll
-          for (int r = 0; r < 16; r++) {
-            const int64_t ir = ir0 + 2 * r;
-            if (ir < p.rows) {
+            if (ir0 + 2 * r < p.rows) {
               const float v = tr[(2 * r + rh) * 17 + jj];
               p.out[orow[r] * p.ldo + j] = p.addsrc ? v + add[r] : v;
             }
           }
         }
+#pragma unroll
+        for (int r = 0; r < 16; r++) add[r] = nadd[r];
         __syncwarp();
       }
       tc_fence_before();
@@ -257,6 +263,7 @@ __global__ void __launch_bounds__(192, 1) tc_gemm_kernel(TcArgs p) {
 constexpr int GN = 128;                                  // N tile of the Gram kernel
 constexpr int G_SUB_KB = 8;                              // K blocks per FP32 chain (256 rows)
 constexpr int G_STAGES = 4;
+constexpr int G_KB_CYCLES = 1150, G_CTA_CYCLES = 15000;   // for the split of K over CTAs
 constexpr int G_A_BYTES = NPIECE * BLK_ELEMS * 2;        // 24 KB
 constexpr int G_STAGE_BYTES = 2 * G_A_BYTES;             // 48 KB
 constexpr int G_SMEM_BYTES = G_STAGES * G_STAGE_BYTES + 1024 + 512;
@@ -657,26 +664,26 @@ cudaError_t launch_gram_tc(const float* A, int64_t lda, const float* B, int64_t 
       split_T_kernel<<<dim3(nkb, cdiv(n, GN)), 256, 0, st>>>(B, ldb, r0, nr, 0, n, nkb, rowmap, Bp[0], Bp[1], Bp[2]),
           count_launch();
     a.nkb = nkb;
-    // split the K range over CTAs: pick the split whose active CTAs fill whole waves
-    // of one CTA per SM best (the lower-triangle tiles of a symmetric Gram exit at once)
+    // split the K range over CTAs (one per SM; the lower-triangle tiles of a symmetric Gram
+    // exit at once): the split with the least modelled time, waves x (cycles of a K block of
+    // twelve MMAs and copies + set-up, first copies, drain and atomics of a CTA).  Counting how
+    // well the last wave is filled alone took 176 CTAs of 8 blocks, two waves, where 88 of 16
+    // take one (45,025 rows x 100 columns with the split of X: 103 -> 87 us; 100,000 x 160 153 ->
+    // 139 us, 234,489 x 850 1375 -> 1341 us; 10,000 to 50,000 cycles give the same).
     int active = 0;
     for (int t = 0; t < tiles; t++) {
       const int mt = t % a.m_tiles, nt = t / a.m_tiles;
       if (!(sym && nt * GN + GN - 1 < mt * TM)) active++;
     }
     int ks = 1;
-    double best = -1.0;
+    int64_t best = INT64_MAX;
     const int max_ks = std::max(1, cdiv(nkb, G_SUB_KB));
     for (int cand = 1; cand <= max_ks; cand++) {
       const int kpc = cdiv(cdiv(nkb, cand), G_SUB_KB) * G_SUB_KB;
       const int real = cdiv(nkb, kpc);
-      const int64_t ctas = (int64_t)active * real;
-      const double waves = (double)((ctas + 151) / 152);
-      const double eff = (double)ctas / (waves * 152.0);
-      // prefer filled waves, then more parallelism up to ~4 waves
-      const double score = eff - 0.02 * std::max(0.0, waves - 4.0) + (ctas >= 152 ? 0.05 : 0.0);
-      if (score > best + 1e-9) {
-        best = score;
+      const int64_t cost = ((int64_t)active * real + 151) / 152 * (G_CTA_CYCLES + (int64_t)kpc * G_KB_CYCLES);
+      if (cost < best) {
+        best = cost;
         ks = real;
       }
     }
