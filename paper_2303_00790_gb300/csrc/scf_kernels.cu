@@ -14,6 +14,7 @@
 #include <algorithm>
 
 #include "fixlap.cuh"
+#include "fp64.cuh"
 #include "kscf_internal.h"
 #include "scf_internal.h"
 
@@ -270,7 +271,8 @@ struct CgArgs {
   LapArgs a;
   const int32_t* live;      // domain slots
   int64_t n_live;
-  double lap_unit;          // -1 / (831600 h^2)
+  double lap_unit;          // -FIX_SUM_UNIT / (831600 h^2)
+  int has_shift;            // a.shift is not zero
   double *x, *r, *p, *q;
   int2* rf;                 // r in fixed point, zero in padding slots
   const double* rr_in;      // partial sums of r.r at entry
@@ -291,8 +293,8 @@ struct CgArgs {
 
 // Grid barrier as in the eigensolver's tridiagonalisation: release arrivals on a monotonic
 // counter, acquire polls, bounded by spin_limit clock cycles.
+// Called after a CTA barrier that follows the other threads' stores.
 __device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
-  __syncthreads();
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.bar) : "memory");
     int ok = 1;
@@ -314,29 +316,25 @@ __device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
   return *s_ok != 0;
 }
 
-// CTA sum of v and maximum of m into *sum and *mx (global, thread 0).  The first four warps,
-// one per SM sub-partition, add the other warps' values, so that the FP64 adds (64 cycles
-// per warp) number 9 in a row instead of 5 in every warp and 16 more.  sh: kCgThreads, zero
-// beyond the CTA's threads (at least 128).
-__device__ __forceinline__ void cg_reduce(double v, uint32_t m, double* sh, double* sh4, uint32_t* shm, double* sum,
+// CTA sum of v and maximum of m into *sum and *mx (global, thread 0): two levels of warp sums.
+// red, shm: kCgThreads / 32.
+__device__ __forceinline__ void cg_reduce(double v, uint32_t m, double* red, uint32_t* shm, double* sum,
                                           uint32_t* mx) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  sh[tid] = v;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  v = warp_sum(v);
   m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) shm[warp] = m;
-  __syncthreads();
-  if (warp < 4) {
-    double s = (sh[tid] + sh[tid + 128]) + (sh[tid + 256] + sh[tid + 384]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) sh4[warp] = s;
+  if (lane == 0) {
+    red[warp] = v;
+    shm[warp] = m;
   }
   __syncthreads();
-  if (tid == 0) {
-    *sum = (sh4[0] + sh4[1]) + (sh4[2] + sh4[3]);
-    uint32_t t = shm[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) t = max(t, shm[w]);
-    *mx = t;
+  if (warp == 0) {
+    const double s = warp_sum(lane < nw ? red[lane] : 0.0);
+    const uint32_t t = __reduce_max_sync(0xffffffffu, lane < nw ? shm[lane] : 0u);
+    if (lane == 0) {
+      *sum = s;
+      *mx = t;
+    }
   }
 }
 
@@ -345,23 +343,29 @@ __device__ __forceinline__ double cg_collect(const double* part, const uint32_t*
   const int lane = threadIdx.x & 31;
   double s = 0.0;
   uint32_t m = 0;
-  for (int b0 = lane; b0 < P; b0 += 160) {
+  for (int b0 = 0; b0 < P; b0 += 160) {
     double v[5];
     uint32_t u[5];
 #pragma unroll
     for (int q = 0; q < 5; q++) {
-      const int b = b0 + 32 * q;
+      const int b = b0 + 32 * q + lane;
       v[q] = b < P ? __ldcg(part + b) : 0.0;
       u[q] = b < P ? __ldcg(mx + b) : 0u;
     }
-    s += ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+    const double t = ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
+    s = b0 == 0 ? t : s + t;
 #pragma unroll
     for (int q = 0; q < 5; q++) m = max(m, u[q]);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   *m_out = __reduce_max_sync(0xffffffffu, m);
-  return s;
+  return warp_sum(s);
+}
+
+// v 2^k (exact) for normal v, in integer instructions where the result is normal
+__device__ __forceinline__ double scale_pow2(double v, int k) {
+  const long long b = __double_as_longlong(v);
+  const int e = ((int)(b >> 52) & 0x7ff) + k;
+  return e >= 1 && e <= 2046 ? __longlong_as_double(b + ((long long)k << 52)) : scalbn(v, k);
 }
 
 // A double at least every double whose high word (sign cleared) is hw
@@ -420,7 +424,7 @@ __device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* 
 template <int B, int NPT>
 __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
   extern __shared__ uint32_t s_face[];   // NPT > 0: [6][NPT][threads] face neighbours of the points
-  __shared__ double sh[kCgThreads], sh4[4];
+  __shared__ double sh[kCgThreads / 32];
   __shared__ uint32_t shm[kCgThreads / 32];
   __shared__ double s_val[2];
   __shared__ uint32_t s_max;
@@ -433,7 +437,6 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
   uint32_t* max_q = c.hmax;
   uint32_t* max_r = c.hmax + P;
   unsigned target = 0;
-  for (int t = tid; t < kCgThreads; t += nt) sh[t] = 0.0;
   const uint32_t zero = 8u * (uint32_t)(c.a.n + kCgZeroSlots / 2);
   constexpr int NR = NPT > 0 ? NPT : 1;
   int sv[NR];
@@ -475,7 +478,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
   uint32_t mr = 0;
   each([&](int, int, double&, double& r, double&, double&) { mr = max(mr, abs_hw(r)); });
   __syncthreads();
-  cg_reduce(0.0, mr, sh, sh4, shm, part_pq + cta, max_r + cta);
+  cg_reduce(0.0, mr, sh, shm, part_pq + cta, max_r + cta);
   if (!cg_barrier(c, target += P, &s_ok)) return;
   if (warp == 0) {
     const double rr0 = warp_sum_partials(c.rr_in, c.n_rr), bb0 = warp_sum_partials(c.part_bb, c.n_bb);
@@ -493,12 +496,17 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
   mr = s_max;
   int e = fix_exp(mr);
   each([&](int, int s, double&, double& r, double&, double&) { c.rf[s] = fix_from(r, e); });
+  __syncthreads();
   if (!cg_barrier(c, target += P, &s_ok)) return;
+  const long long tol_bits = __double_as_longlong(c.rtol2 * bb);
   int it = 0;
   for (; it < c.max_iters; it++) {
-    if (rr < c.rtol2 * bb || !(rr <= 1.7976931348623157e308)) break;
+    // rr < rtol^2 b.b or not finite; rr >= 0, so the bits compare like the values (FP64
+    // comparisons and products in every warp, here and in sc, took 64 cycles each of its pipe)
+    const long long rr_bits = __double_as_longlong(rr);
+    if (rr_bits < tol_bits || rr_bits >= 0x7ff0000000000000LL) break;
     // q = A r + beta q, p = r + beta p, p.q
-    const double sc = c.lap_unit * FIX_SUM_UNIT * fix_unit(e);
+    const double sc = scale_pow2(c.lap_unit, e - 1022 - FIX_BITS);
     double acc = 0.0;
     uint32_t mq = 0;
     each([&](int k, int s, double&, double& r, double& p, double& q) {
@@ -512,13 +520,13 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
       }
       const double pn = fma(beta, p, r);
       double qn = fma(sc, fix_value(t), beta * q);
-      if (c.a.shift != 0.0) qn = fma(c.a.shift, r, qn);
+      if (c.has_shift) qn = fma(c.a.shift, r, qn);
       p = pn;
       q = qn;
       acc = fma(pn, qn, acc);
       mq = max(mq, abs_hw(qn));
     });
-    cg_reduce(acc, mq, sh, sh4, shm, part_pq + cta, max_q + cta);
+    cg_reduce(acc, mq, sh, shm, part_pq + cta, max_q + cta);
     if (!cg_barrier(c, target += P, &s_ok)) return;
     if (warp == 0) {
       uint32_t m;
@@ -544,7 +552,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
       acc = fma(rn, rn, acc);
       mr = max(mr, abs_hw(rn));
     });
-    cg_reduce(acc, mr, sh, sh4, shm, part_rr + cta, max_r + cta);
+    cg_reduce(acc, mr, sh, shm, part_rr + cta, max_r + cta);
     if (!cg_barrier(c, target += P, &s_ok)) return;
     if (warp == 0) {
       uint32_t m;
@@ -637,7 +645,8 @@ cudaError_t launch_cg(const Ham& H, double shift, const CgWork& w, double rtol, 
   c.a = lap_args(H, shift);
   c.live = H.d_live;
   c.n_live = H.n_live;
-  c.lap_unit = -1.0 / (FIX_DEN * H.grid.h * H.grid.h);
+  c.lap_unit = -1.0 / (FIX_DEN * H.grid.h * H.grid.h) * FIX_SUM_UNIT;
+  c.has_shift = shift != 0.0 ? 1 : 0;
   c.x = x;
   c.r = w.r;
   c.p = w.p;
