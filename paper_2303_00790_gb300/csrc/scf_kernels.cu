@@ -293,10 +293,13 @@ struct CgArgs {
 
 // Grid barrier as in the eigensolver's tridiagonalisation: release arrivals on a monotonic
 // counter, acquire polls, bounded by spin_limit clock cycles.
-// Called after a CTA barrier that follows the other threads' stores.
-__device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
+// cg_arrive is called after a CTA barrier that follows the other threads' stores; work that no
+// other CTA reads can stand between it and cg_wait.
+__device__ __forceinline__ void cg_arrive(const CgArgs& c) {
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.bar) : "memory");
+}
+__device__ bool cg_wait(const CgArgs& c, unsigned target, int* s_ok) {
   if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.bar) : "memory");
     int ok = 1;
     const long long t0 = clock64();
     for (unsigned tries = 1;; tries++) {
@@ -314,6 +317,10 @@ __device__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
   }
   __syncthreads();
   return *s_ok != 0;
+}
+__device__ __forceinline__ bool cg_barrier(const CgArgs& c, unsigned target, int* s_ok) {
+  cg_arrive(c);
+  return cg_wait(c, target, s_ok);
 }
 
 // CTA sum of v and maximum of m into *sum and *mx (global, thread 0): two levels of warp sums.
@@ -541,19 +548,20 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
     __syncthreads();
     const double alpha = s_val[0];
     e = fix_exp(s_max);
-    // x += alpha p, r -= alpha q, r.r
+    // r -= alpha q, r.r; x += alpha p while the CTA waits for the others
     acc = 0.0;
     mr = 0;
-    each([&](int, int s, double& x, double& r, double& p, double& q) {
+    each([&](int, int s, double&, double& r, double&, double& q) {
       const double rn = fma(-alpha, q, r);
-      x = fma(alpha, p, x);
       r = rn;
       c.rf[s] = fix_from(rn, e);
       acc = fma(rn, rn, acc);
       mr = max(mr, abs_hw(rn));
     });
     cg_reduce(acc, mr, sh, shm, part_rr + cta, max_r + cta);
-    if (!cg_barrier(c, target += P, &s_ok)) return;
+    cg_arrive(c);
+    each([&](int, int, double& x, double&, double& p, double&) { x = fma(alpha, p, x); });
+    if (!cg_wait(c, target += P, &s_ok)) return;
     if (warp == 0) {
       uint32_t m;
       const double t = cg_collect(part_rr, max_r, P, &m);
