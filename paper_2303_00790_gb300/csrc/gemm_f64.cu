@@ -22,10 +22,12 @@
 // A NaN, an Inf or magnitudes outside 2^+-500 in an operand set a device flag: the kernels here
 // then do nothing and the CUDA-core kernels, launched behind the same flag, do the work.
 //
-// What bounds it: the MMA's operand reads.  A 128 x 64 x 16 MMA reads 6 KB from shared memory
-// and takes ~70 cycles (87 B per cycle) where the tensor core needs 32; more or finer pipeline
-// stages changed nothing.  The drain of 8192 x 8 accumulators every 128 terms (16 % of the time)
-// is not overlapped, because the eight accumulators of 64 columns fill tensor memory.
+// What bounds it: shared memory.  A 128 x 64 x 16 MMA takes 48 cycles with its operands resident
+// (6 KB of them at 128 bytes per cycle; 64 and 128 cycles for N = 128 and 256, with or without
+// swizzle) and ~70 here, where the copies add 1.3 KB per MMA and the chains wait for their
+// drain; the tensor core would need 32.  More or finer pipeline stages changed nothing.  The
+// drain of 8192 x 8 accumulators every 128 terms (16 % of the time) is not overlapped, because
+// the eight accumulators of 64 columns fill tensor memory.
 // Measured at 234,489 rows x 850 columns: Gram 6.8 ms and triangular rotation 8.6 ms (~1.0
 // PFLOP/s of bf16 products) plus 3.4 ms for maxima and digits; the CUDA-core FP64 kernels took
 // ~450 and ~480 ms.  Errors against exact sums, relative to |a||b|, rms: Gram 45,025 x 100 4e-19
