@@ -10,6 +10,8 @@
 //     grid-wide barrier; then every CTA forms w = p - (tau/2)(p^T v) v, row j+1 of the
 //     updated matrix (published by its owner during the pass) and the next Householder
 //     vector from it, redundantly, so that each step costs a single barrier.
+//     Matrices of at most 160 rows run in one cluster of eight CTAs that exchange p and the
+//     row through distributed shared memory.
 //  2. Tridiagonal divide and conquer (Cuppen 1981) with the deflation of Dongarra &
 //     Sorensen (1987) and the eigenvector formula of Gu & Eisenstat (1995).  The
 //     recursion tree is balanced (node t of depth d covers [t n / 2^d, (t+1) n / 2^d))
@@ -191,6 +193,24 @@ __device__ bool tri_barrier(const TriArgs& a, unsigned target, int* s_ok) {
   return *s_ok != 0;
 }
 
+// Small matrices: one cluster of eight CTAs, p and the published row written straight into
+// every CTA's shared memory, the cluster's hardware barrier instead of the grid's (the trips
+// through L2 are 3,800 of a step's 8,500 cycles).  Up to TRI_CLUSTER_N rows the eight SMs'
+// FP64 pipes are enough: the whole solver takes 860 instead of 960 us at n = 100 and 1280 instead of
+// 1350 at 160, but 1740 instead of 1670 at 200.
+constexpr int TRI_CLUSTER = 8, TRI_CLUSTER_N = 160;
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p = v at the same place of CTA `rank`'s shared memory
+__device__ __forceinline__ void store_to_cta(double* p, int rank, double v) {
+  asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f64 [a], %2;\n}" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(p)),
+               "r"(rank), "d"(v)
+               : "memory");
+}
+
 // Scalars of the Householder reflector of x = r[s .. n-1] (Golub & Van Loan, Sec. 5.1.2,
 // without the normalisation v_0 = 1): with |x|^2 = alpha^2 + sigma, beta = -sign(alpha)|x|,
 // v = x - beta e_1 (so v_0 = alpha - beta = sign(alpha)(|alpha| + |x|), v_l = x_l after it)
@@ -246,9 +266,11 @@ __device__ __forceinline__ void reflector_scalars(double alpha, double sigma, do
 // p and the row as tagged 16-byte words that every CTA polls, without a barrier, was slower (152
 // CTAs read 27 KB a step from lines being written: 13.0 ms instead of 11.2 for the whole solver
 // at 850).
-template <bool SMEM>
+template <bool SMEM, bool CLUSTER = false>
 __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
-  constexpr int VT = NT - 32, VE = 4;
+  static_assert(SMEM || !CLUSTER, "a cluster keeps its rows in shared memory");
+  constexpr int VT = NT - 32, VE = CLUSTER ? 1 : 4;   // elements per thread (a cluster has n <= VT)
+  constexpr int UQ = CLUSTER ? TRI_CLUSTER_N / 32 : 8;   // columns per lane in flight
   extern __shared__ __align__(16) double smd[];
   __shared__ double red[NW];
   __shared__ double sc[4], s_k[2];
@@ -261,7 +283,8 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
   double* vp = smd + n;
   double* wp = smd + 2 * n;
   double* rw = !SMEM && a.rwg ? a.rwg + (int64_t)cta * n : smd + 3 * n;
-  double* rows = smd + 4 * n;   // SMEM only (then rw is in shared memory as well)
+  double* xbuf = smd + 4 * n;   // CLUSTER: p and the published row, for even and odd steps
+  double* rows = smd + (CLUSTER ? 8 : 4) * n;   // SMEM only (then rw is in shared memory as well)
   const int nown = cta < n ? (n - cta + P - 1) / P : 0;
   if (n == 1) {
     if (cta == 0 && threadIdx.x == 0) {
@@ -271,6 +294,7 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     }
     return;
   }
+  if (CLUSTER) cluster_sync();   // the other CTAs' shared memory may be written from here on
   if (SMEM) {
     for (int r = 0; r < nown; r++) {
       const double* src = a.A + (int64_t)(cta + r * P) * a.lda;
@@ -310,8 +334,8 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     if (r0 < nown && cta + r0 * P <= j) r0++;
     if (++wcta == P) wcta = 0;
     const int par = j & 1;
-    double* pb = a.pbuf + (int64_t)par * n;
-    double* rb = a.rowbuf + (int64_t)par * n;
+    double* pb = CLUSTER ? xbuf + par * 2 * n : a.pbuf + (int64_t)par * n;
+    double* rb = CLUSTER ? pb + n : a.rowbuf + (int64_t)par * n;
     // pass over the owned rows i > j: A^(j) = A^(j-1) - v w^T - w v^T, p_i = tau_j A^(j)_i. v_j
     double dotp = 0.0;
     const bool upd = !SMEM && j >= 1;   // shared-memory rows were updated in the last step
@@ -323,11 +347,11 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       double acc0 = 0.0, acc1 = 0.0;
       // whole warps branch, lanes beyond n multiply zeros: a branch that splits a warp costs
       // ~50 cycles, nearly one FP64 operation
-      for (int lb = j + 1; lb < n; lb += 8 * 32) {
+      for (int lb = j + 1; lb < n; lb += UQ * 32) {
         const int l = lb + lane;
-        double x[8], v[8];
+        double x[UQ], v[UQ];
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
+        for (int q = 0; q < UQ; q++) {
           x[q] = v[q] = 0.0;
           if (l + 32 * q < n) {
             x[q] = row[l + 32 * q];
@@ -335,7 +359,7 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
           }
         }
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
+        for (int q = 0; q < UQ; q++) {
           if (lb + 32 * q < n) {
             const int ll = l + 32 * q;
             double y = x[q];
@@ -343,25 +367,38 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
               y = fma(-vpi, wp[ll], fma(-wpi, vp[ll], y));
               row[ll] = y;
             }
-            if (pub && ll < n) rb[ll] = y;
+            if (pub && ll < n) {
+              if (CLUSTER) {
+#pragma unroll
+                for (int c = 0; c < TRI_CLUSTER; c++) store_to_cta(rb + ll, c, y);
+              } else {
+                rb[ll] = y;
+              }
+            }
             if (q & 1) acc1 = fma(y, v[q], acc1);
             else acc0 = fma(y, v[q], acc0);
           }
         }
       }
       const double pi = warp_sum(acc0 + acc1) * tj;
-      if (lane == 0) {
+      if (CLUSTER) {
+        if (lane < TRI_CLUSTER) store_to_cta(pb + i, lane, pi);
+      } else if (lane == 0) {
         pb[i] = pi;
         dotp = fma(pi, vc[i], dotp);
       }
     }
-    if (lane == 0) red[warp] = dotp;
-    __syncthreads();
-    if (warp == 0) {
-      const double s = warp_sum(lane < NW ? red[lane] : 0.0);
-      if (lane == 0) a.dotbuf[par * P + cta] = s;
+    if (CLUSTER) {
+      cluster_sync();
+    } else {
+      if (lane == 0) red[warp] = dotp;
+      __syncthreads();
+      if (warp == 0) {
+        const double s = warp_sum(lane < NW ? red[lane] : 0.0);
+        if (lane == 0) a.dotbuf[par * P + cta] = s;
+      }
+      if (!tri_barrier(a, (unsigned)P * (unsigned)(j + 1), &s_ok)) return;
     }
-    if (!tri_barrier(a, (unsigned)P * (unsigned)(j + 1), &s_ok)) return;
     // every CTA: K = tau/2 p.v, w_j = p - K v_j, row j+1 of A^(j+1), next reflector.
     // The row r + 2 K v_1 v - v_1 p - p_1 v is K's multiple of v added to what is known
     // before K.  Warp 0 sums K, the others have the vectors (the first VE VT elements in
@@ -369,14 +406,14 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
     const int l0 = j + 1 + (int)threadIdx.x - 32;
     double pv[VE], yv[VE], vv[VE];
     auto load = [&](int l) {
-      const double v1 = vc[j + 1], p1 = __ldcg(pb + j + 1);
+      const double v1 = vc[j + 1], p1 = CLUSTER ? pb[j + 1] : __ldcg(pb + j + 1);
 #pragma unroll
       for (int q = 0; q < VE; q++) {
         const int ll = l + q * VT;
         pv[q] = yv[q] = vv[q] = 0.0;
         if (ll < n) {
-          pv[q] = __ldcg(pb + ll);
-          yv[q] = __ldcg(rb + ll);
+          pv[q] = CLUSTER ? pb[ll] : __ldcg(pb + ll);
+          yv[q] = CLUSTER ? rb[ll] : __ldcg(rb + ll);
           vv[q] = vc[ll];
         }
       }
@@ -387,17 +424,40 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       }
     };
     if (warp == 0) {
-      double part[MAX_P / 32];
-#pragma unroll
-      for (int c = 0; c < MAX_P / 32; c++) {
-        part[c] = 0.0;
-        if (c * 32 < P && c * 32 + lane < P) part[c] = __ldcg(a.dotbuf + par * P + c * 32 + lane);
-      }
       const double ht = 0.5 * tj, tv = tj * vc[j + 1];
-      double s = part[0];
-      if (P > 32) s += part[1];
-      if (P > 64) s += part[2] + part[3];
-      if (P > 128) s += (part[4] + part[5]) + (part[6] + part[7]);
+      double s;
+      if constexpr (CLUSTER) {   // n <= TRI_CLUSTER_N: all of p is here
+        double x[UQ], v[UQ], s1 = 0.0;
+        s = 0.0;
+#pragma unroll
+        for (int q = 0; q < UQ; q++) {
+          const int l = j + 1 + 32 * q + lane;
+          x[q] = v[q] = 0.0;
+          if (l < n) {
+            x[q] = pb[l];
+            v[q] = vc[l];
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < UQ; q++) {
+          if (j + 1 + 32 * q < n) {   // warp-uniform
+            if (q & 1) s1 = fma(x[q], v[q], s1);
+            else s = fma(x[q], v[q], s);
+          }
+        }
+        s += s1;
+      } else {
+        double part[MAX_P / 32];
+#pragma unroll
+        for (int c = 0; c < MAX_P / 32; c++) {
+          part[c] = 0.0;
+          if (c * 32 < P && c * 32 + lane < P) part[c] = __ldcg(a.dotbuf + par * P + c * 32 + lane);
+        }
+        s = part[0];
+        if (P > 32) s += part[1];
+        if (P > 64) s += part[2] + part[3];
+        if (P > 128) s += (part[4] + part[5]) + (part[6] + part[7]);
+      }
       s = warp_sum(s);
       const double K = ht * s, c2 = tv * s;
       if (lane == 0) {
@@ -461,22 +521,22 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       } else if (SMEM && (warp & 3) != 0) {
         // meanwhile the warps of the other three SM sub-partitions (whose FP64 pipes the
         // scalar chain does not use) update the owned rows i >= j+2 to A^(j+1) over the
-        // columns l >= j+2, in items of one row x 256 columns
+        // columns l >= j+2, in items of one row x 32 UQ columns
         const int u = (warp >> 2) * 3 + (warp & 3) - 1;
         const int rs = r0 < nown && cta + r0 * P == j + 1 ? r0 + 1 : r0;
-        const int nch = (n - (j + 2) + 255) / 256;
+        const int nch = CLUSTER ? 1 : (n - (j + 2) + UQ * 32 - 1) / (UQ * 32);
         const int items = (nown - rs) * nch;
         for (int it = u; it < items; it += NW - NW / 4) {
           const int r = rs + it / nch;
           const int i = cta + r * P;
           double* row = rows + (int64_t)r * n;
           const double vi = vc[i], wi = wp[i];
-          const int lb = j + 2 + (it % nch) * 256;
-          double x[8];
+          const int lb = j + 2 + (it % nch) * (UQ * 32);
+          double x[UQ];
 #pragma unroll
-          for (int q = 0; q < 8; q++) x[q] = lb + lane + 32 * q < n ? row[lb + lane + 32 * q] : 0.0;
+          for (int q = 0; q < UQ; q++) x[q] = lb + lane + 32 * q < n ? row[lb + lane + 32 * q] : 0.0;
 #pragma unroll
-          for (int q = 0; q < 8; q++) {
+          for (int q = 0; q < UQ; q++) {
             if (lb + 32 * q < n) {   // warp-uniform
               const int ll = lb + 32 * q + lane, lc = min(ll, n - 1);
               const double y = fma(-vi, wp[lc], fma(-wi, vc[lc], x[q]));
@@ -505,6 +565,7 @@ __global__ void __launch_bounds__(NT, 1) tridiag_kernel(TriArgs a) {
       a.tau[n - 1] = 0.0;
     }
   }
+  if (CLUSTER) cluster_sync();   // no CTA ends while another may still write its shared memory
 }
 
 // ------------------------------------------------------- divide and conquer ----
@@ -1436,8 +1497,11 @@ cudaError_t launch_sym_eig(double* A, int64_t lda, int n, double* w, void* work,
   t.status = info;
   t.spin_limit = spin_limit;
   t.leave_cta = leave_cta;
+  // (the self-test of the bounded barrier needs the grid's)
+  const bool cluster = n <= TRI_CLUSTER_N && leave_cta < 0;
+  if (cluster) t.P = TRI_CLUSTER;
   const int R = (n + t.P - 1) / t.P;
-  size_t vec_bytes = (size_t)4 * n * 8;
+  size_t vec_bytes = (size_t)(cluster ? 8 : 4) * n * 8;
   if (vec_bytes > SMEM_CAP) {
     vec_bytes = (size_t)3 * n * 8;
     t.rwg = (double*)P_(L_RWG);
@@ -1445,17 +1509,27 @@ cudaError_t launch_sym_eig(double* A, int64_t lda, int n, double* w, void* work,
   const size_t rows_bytes = (size_t)R * n * 8;
   const bool smem_rows = vec_bytes + rows_bytes <= SMEM_CAP;
   const size_t tri_smem = vec_bytes + (smem_rows ? rows_bytes : 0);
+  const void* tri = cluster     ? (const void*)tridiag_kernel<true, true>
+                    : smem_rows ? (const void*)tridiag_kernel<true>
+                                : (const void*)tridiag_kernel<false>;
+  if ((e = cudaFuncSetAttribute(tri, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem)) != cudaSuccess)
+    return e;
   void* targs[] = {&t};
-  if (smem_rows) {
-    if ((e = cudaFuncSetAttribute(tridiag_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tri_smem)) !=
-        cudaSuccess)
-      return e;
-    e = cudaLaunchCooperativeKernel((void*)tridiag_kernel<true>, dim3(t.P), dim3(NT), targs, tri_smem, st);
+  if (cluster) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = TRI_CLUSTER;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(TRI_CLUSTER);
+    cfg.blockDim = dim3(NT);
+    cfg.dynamicSmemBytes = tri_smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelExC(&cfg, tri, targs);
   } else {
-    if ((e = cudaFuncSetAttribute(tridiag_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tri_smem)) != cudaSuccess)
-      return e;
-    e = cudaLaunchCooperativeKernel((void*)tridiag_kernel<false>, dim3(t.P), dim3(NT), targs, tri_smem, st);
+    e = cudaLaunchCooperativeKernel(tri, dim3(t.P), dim3(NT), targs, tri_smem, st);
   }
   count_launch();
   if (e != cudaSuccess) return e;

@@ -1,7 +1,8 @@
 """Eigensolver at the sizes where the tridiagonalisation's paths change, against the residual and
-orthogonality of the eigenpairs.  n = 2 .. 7: one or two CTAs; 153, 305, 609: around one more row
-per CTA; 1023 .. 1026: the registers' first 1024 elements; 1800, 2000: rows in shared and in global
-memory; 7100: the row work vectors in global memory.
+orthogonality of the eigenpairs.  n = 2 .. 9: a cluster with CTAs that own no row or one; 159 .. 161:
+the last cluster and the first grid; 305, 609: around one more row per CTA; 1023 .. 1026: more
+elements than the registers hold; 1800, 2000: rows in shared and in global memory; 7100: the row
+work vectors in global memory.
 
 Bar: |A Z - Z w| and |Z^T Z - I| are O(n u) max|A| for a backward-stable solver; with a constant of
 16 that is 16 n 2^-53, and 64 u below n = 4 (|A| <= 1 here, so its norm is at most n)."""
@@ -21,7 +22,7 @@ def kscf():
     return mod
 
 
-@pytest.mark.parametrize("n", [2, 3, 4, 5, 6, 7, 153, 305, 609, 1023, 1024, 1025, 1026, 1800, 2000, 7100])
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 6, 7, 8, 9, 33, 64, 159, 160, 161, 305, 609, 1023, 1024, 1025, 1026, 1800, 2000, 7100])
 def test_eigenpairs(kscf, n):
     g = torch.Generator(device="cuda").manual_seed(n)
     B = torch.rand((n, n), dtype=torch.float64, device="cuda", generator=g) * 2 - 1
