@@ -391,26 +391,51 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
   }
 }
 
-// float to double with integer instructions (an FP64 conversion costs as much as the addition
-// that follows it: 64 cycles per warp)
-__device__ __forceinline__ double widen(float f) {
-  const uint32_t b = __float_as_uint(f), e = (b >> 23) & 0xff;
-  if (e == 0 || e == 255) return (double)f;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+// Sum of RB floats as an FP64 number, formed in integers: the values are aligned
+// to the largest exponent with 57 bits (cut below 2^-57 of the largest, where FP64 additions
+// round at 2^-53) and one conversion rounds the sum.  NaN and Inf are added in FP64.
+constexpr int RB = 20;
+__device__ __forceinline__ double sum_floats(const float (&f)[RB]) {
+  int em = 1;
+#pragma unroll
+  for (int u = 0; u < RB; u++) em = max(em, (__float_as_int(f[u]) >> 23) & 255);
+  if (em == 255) {
+    double s = 0.0;
+#pragma unroll
+    for (int u = 0; u < RB; u++) s += (double)f[u];
+    return s;
+  }
+  long long m = 0;
+#pragma unroll
+  for (int u = 0; u < RB; u++) {
+    const int b = __float_as_int(f[u]), e = (b >> 23) & 255;
+    const long long x = ((long long)((b & 0x7fffff) | (e ? 0x800000 : 0)) << 33) >> min(em - max(e, 1), 63);
+    m += b < 0 ? -x : x;
+  }
+  return (double)m * __hiloint2double((em - 127 - 23 - 33 + 1023) << 20, 0);
 }
 
 // grad[q] = sum_b part[b][q] (FP64, fixed order); loss = sum_b part[b][NPAR] / n.  A block adds 32
-// values, each in eight interleaved chains of blocks that meet in shared memory: one chain of
-// 152 FP64 conversions and additions per value on 82 blocks took 27 us, this takes 17 us with
-// cold caches (12.7 MB of partials).
+// values, each in eight chains of rows that meet in shared memory.  A chain's loads are in
+// flight together and its sum is formed in integers: the 152 FP64 additions per value alone took
+// 5 us of the FP64 pipe (one chain on 82 blocks 27 us, eight chains 17 us, this 7.4 us with cold
+// caches, 12.7 MB of partials).
 __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict__ part, int nb, int64_t n,
                                                          float* __restrict__ grad, double* __restrict__ loss) {
   __shared__ double red[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = blockIdx.x * 32 + lane;
   double s = 0.0;
   if (q <= NPAR) {
-#pragma unroll 4
-    for (int b = w; b < nb; b += 8) s += widen(__ldg(part + (int64_t)b * (NPAR + 1) + q));
+    for (int b0 = w; b0 < nb; b0 += 8 * RB) {
+      float f[RB];
+#pragma unroll
+      for (int u = 0; u < RB; u++) {
+        const int b = b0 + 8 * u;
+        f[u] = b < nb ? __ldg(part + (int64_t)b * (NPAR + 1) + q) : 0.0f;
+      }
+      const double t = sum_floats(f);
+      s = b0 == w ? t : s + t;
+    }
   }
   red[w][lane] = s;
   __syncthreads();
