@@ -13,19 +13,19 @@ namespace kscf {
 // 320.  The sum is therefore formed in integers: every value is aligned to the largest
 // exponent of the warp as a 58-bit integer (cut below 2^-57 of the largest value, where each
 // addition of the tree rounds at 2^-53), the integers are summed exactly as three 26-bit parts
-// by integer reductions, and the total is rounded to a double once.  Values near or beyond the
-// end of the range (Inf and NaN among them) take the tree.  Subnormal values count as zero.
+// by integer reductions, and the total is rounded to a double once.  Warps whose largest value
+// is near the ends of the range (Inf, NaN and subnormal sums among them) take the tree.
 __device__ __forceinline__ double warp_sum(double v) {
   const long long b = __double_as_longlong(v);
   const int e = (int)(b >> 52) & 0x7ff;
   const int em = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if (em >= 0x7f8) {
+  if ((unsigned)(em - 64) >= 0x7f8u - 64u) {
+    if (!__any_sync(0xffffffffu, (b << 1) != 0)) return 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
   }
-  if (em == 0) return 0.0;
-  long long m = e ? ((b & 0xfffffffffffffLL) | (1LL << 52)) << 5 : 0;
+  long long m = e ? ((b & 0xfffffffffffffLL) | (1LL << 52)) << 5 : 0;   // (subnormal: cut)
   m >>= min(em - e, 63);
   if (b < 0) m = -m;
   const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x3ffffffu);
@@ -37,8 +37,7 @@ __device__ __forceinline__ double warp_sum(double v) {
   unsigned long long u = s < 0 ? -(unsigned long long)s : (unsigned long long)s;
   const int z = __clzll((long long)u);
   u <<= z;
-  const int ex = em + 6 - z;
-  if (ex <= 0) return 0.0;
+  const int ex = em + 6 - z;   // > 0: z <= 63
   const long long mag = ((long long)(ex - 1) << 52) + (long long)((u >> 11) + (u >> 10 & 1));
   return __longlong_as_double(mag | (s & (1LL << 63)));
 }

@@ -258,13 +258,14 @@ __global__ void __launch_bounds__(kScfThreads) cg_init_kernel(LapArgs a, double*
 // (q = A p by the recurrence of Chronopoulos & Gear 1989, so that the only neighbour values
 // read are those of r, which are ready at the barrier of r.r.)  A r reads r as 58-bit fixed
 // point (fixlap.cuh), whose exponent comes from max|r| and max|q| of the reductions before.
-// What bounds an iteration: the barriers (~1.5 us each with their skew), the FP64 chains of
-// the two reductions (only one warp of a CTA adds the other CTAs' partial sums) and 10 FP64
-// instructions per point (64 cycles per warp each).  Up to 4 points per thread the vectors
-// stay in registers; larger grids (NPT = 0) keep them in global memory.  Three launches per
-// iteration with the star in FP64 and every warp adding the 304 partials two or three times
-// took 89 us at 234,489 points and 67 us at 45,025; this kernel takes 15.6 us and 9.1 us (Hartree
-// solve of the 2.2 nm cluster, 368 iterations: 32.7 -> 5.75 ms).
+// What bounds an iteration is latency: at 45,025 points (one per thread; cycles) the star takes
+// 1,500, the CTA's sums 2 x 950, the barriers 2 x 2,500, the partial sums from L2 2 x 1,500, the
+// divisions 1,400, the update 500; at 234,489 points the star 11,500 (loads, and 5 of the 10
+// FP64 instructions per point at 64 cycles per warp) and the update 2,700.  Up to 4 points per
+// thread the vectors stay in registers; larger grids (NPT = 0) keep them in global memory.  Three
+// launches per iteration with the star in FP64 and every warp adding the 304 partials two or
+// three times took 89 us at 234,489 points and 67 us at 45,025; this kernel takes 14.0 us and
+// 7.1 us (Hartree solve of the 2.2 nm cluster, 368 iterations: 32.7 -> 5.18 ms).
 constexpr int kCgThreads = 512;   // most threads of a CTA
 
 struct CgArgs {
