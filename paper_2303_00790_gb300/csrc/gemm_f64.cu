@@ -28,8 +28,8 @@
 // drain; the tensor core would need 32.  More or finer pipeline stages changed nothing.  The
 // drain of 8192 x 8 accumulators every 128 terms (16 % of the time) is not overlapped, because
 // the eight accumulators of 64 columns fill tensor memory.
-// Measured at 234,489 rows x 850 columns: Gram 6.8 ms and triangular rotation 8.6 ms (~1.0
-// PFLOP/s of bf16 products) plus 3.4 ms for maxima and digits; the CUDA-core FP64 kernels took
+// Measured at 234,489 rows x 850 columns: Gram 8.1 ms and triangular rotation 8.6 ms (~0.9
+// PFLOP/s of bf16 products) plus 2.0 ms for maxima and digits; the CUDA-core FP64 kernels took
 // ~450 and ~480 ms.  Errors against exact sums, relative to |a||b|, rms: Gram 45,025 x 100 4e-19
 // (FP64 kernel 3e-18), rotation 30,000 x 850 x 850 relative 9e-17 (1e-15), with column norms over
 // eight decades 2.4e-16 (3.2e-16).
@@ -206,20 +206,24 @@ __global__ void __launch_bounds__(256) digits_T_kernel(const double* __restrict_
   }
 }
 
-// Rotation A operand: MN = rows, K = columns.  One warp per row, a lane per 8 columns; columns
-// are taken relative to their maximum (cmax), the row's largest relative exponent is its unit
-// (rexp, <= 0; a row of zeros gets -4096).  Rows nr .. of the last block are zero.
+// Rotation A operand: MN = rows, K = columns; columns are taken relative to their maximum
+// (cmax), the row's largest relative exponent is its unit (rexp, <= 0; a row of zeros gets
+// -4096).  Rows nr .. of the last block are zero.  Eight rows per CTA: a warp per row finds the
+// units; then a lane has 8 columns of one of the eight rows, so that eight lanes store the 128
+// bytes of a core matrix.  HBM bound (8 B read, 14 B written per value); a warp per row for the
+// digits too, storing 16 bytes of every line, and zero tests in FP64 (64 cycles each) took
+// 2.11 ms at 234,489 x 850, this takes 1.00 ms.
 __global__ void __launch_bounds__(256) digits_N_kernel(const double* __restrict__ X, int64_t ld, int64_t nr, int nc,
                                                        int nkb, const int32_t* __restrict__ rowmap,
                                                        const uint32_t* __restrict__ cmax, const int* __restrict__ flag,
                                                        __nv_bfloat16* __restrict__ D, int* __restrict__ rexp) {
+  __shared__ int s_unit[8];
   if (*flag) return;
-  const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const bool live = r < nr;
-  const double* row = X + (live ? (rowmap ? (int64_t)rowmap[r] : r) : 0) * ld;
+  const int64_t r0 = (int64_t)blockIdx.x * 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = (ld & 1) == 0 && ((uintptr_t)X & 15) == 0;
-  auto load8 = [&](int c, double* v) {
+  // eight values of row r from column c on (zeros outside)
+  auto load8 = [&](const double* row, bool live, int c, double* v) {
     if (live && vec && c + 8 <= nc) {
 #pragma unroll
       for (int u = 0; u < 4; u++) {
@@ -232,24 +236,37 @@ __global__ void __launch_bounds__(256) digits_N_kernel(const double* __restrict_
       for (int u = 0; u < 8; u++) v[u] = live && c + u < nc ? row[c + u] : 0.0;
     }
   };
+  auto row_of = [&](int64_t r) { return X + (r < nr ? (rowmap ? (int64_t)rowmap[r] : r) : 0) * ld; };
   auto rel = [&](double v, int c) { return bexp(v) - (c < nc ? (int)(cmax[c] >> 20) : 0); };
-  int m = -4096;
-  for (int c = lane * 8; c < nc; c += 256) {
-    double v[8];
-    load8(c, v);
+  auto nonzero = [](double v) { return (__double_as_longlong(v) << 1) != 0; };
+  {
+    const int64_t r = r0 + warp;
+    const double* row = row_of(r);
+    int m = -4096;
+    for (int c = lane * 8; c < nc; c += 256) {
+      double v[8];
+      load8(row, r < nr, c, v);
 #pragma unroll
-    for (int u = 0; u < 8; u++)
-      if (v[u] != 0.0) m = max(m, rel(v[u], c + u));
+      for (int u = 0; u < 8; u++)
+        if (nonzero(v[u])) m = max(m, rel(v[u], c + u));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) {
+      rexp[r] = m;
+      s_unit[warp] = m;
+    }
   }
-  m = __reduce_max_sync(0xffffffffu, m);
-  if (lane == 0) rexp[r] = m;
-  const int64_t mb = r >> 7;
-  for (int c = lane * 8; c < nkb * F_TK; c += 256) {
+  __syncthreads();
+  const int64_t r = r0 + (lane & 7);
+  const double* row = row_of(r);
+  const int m = s_unit[lane & 7];
+  const int64_t mb = r0 >> 7;
+  for (int c = (warp * 4 + (lane >> 3)) * 8; c < nkb * F_TK; c += 256) {
     double v[8];
-    load8(c, v);
+    load8(row, r < nr, c, v);
     long long x[8];
 #pragma unroll
-    for (int u = 0; u < 8; u++) x[u] = v[u] != 0.0 ? shifted(v[u], rel(v[u], c + u) - m + 2) : 0;
+    for (int u = 0; u < 8; u++) x[u] = nonzero(v[u]) ? shifted(v[u], rel(v[u], c + u) - m + 2) : 0;
     store_digits(x, D + blk_off(mb, nkb, c / F_TK) + tile_off((int)(r & 127), c % F_TK));
   }
 }
