@@ -102,15 +102,21 @@ __device__ void load_weights(const float* __restrict__ P, float* sm) {
   }
 }
 
-// Standardised input tile: rows p0 .. p0 + TP - 1 (rows from n on are zero).
-template <bool BF16>
+// Tiles of at most TP points, or of SMALL where no block has more (n <= 64 per block: up to 9,728
+// points): the products run over whole tiles of TE points, so a tile of 112 for 64 points
+// wastes 40 % of them (4,000 points: gradient and Adam step 115 -> 97 us).
+constexpr int SMALL = 64;
+__host__ __device__ constexpr int rows_of(int te) { return (te + 31) / 32; }   // per thread
+
+// Standardised input tile: rows p0 .. p0 + TE - 1 (rows from n on are zero).
+template <bool BF16, int TE>
 __device__ void load_tile(const float* __restrict__ D, const float* __restrict__ mu, const float* __restrict__ inv_sd,
                           int64_t n, int64_t p0, float* sm) {
   if (aligned16(D) && aligned16(mu) && aligned16(inv_sd)) {
     const int i = 4 * (threadIdx.x % (NIN / 4));   // NT is a multiple of NIN / 4
     const float4 m = __ldg((const float4*)(mu + i)), s = __ldg((const float4*)(inv_sd + i));
 #pragma unroll
-    for (int e = threadIdx.x; e < TP * NIN / 4; e += NT) {
+    for (int e = threadIdx.x; e < TE * NIN / 4; e += NT) {
       const int p = e / (NIN / 4);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p0 + p < n) {
@@ -121,7 +127,7 @@ __device__ void load_tile(const float* __restrict__ D, const float* __restrict__
     }
     return;
   }
-  for (int e = threadIdx.x; e < TP * NIN; e += NT) {
+  for (int e = threadIdx.x; e < TE * NIN; e += NT) {
     const int p = e / NIN, i = e % NIN;
     const int64_t row = p0 + p;
     float v = 0.0f;
@@ -130,24 +136,25 @@ __device__ void load_tile(const float* __restrict__ D, const float* __restrict__
   }
 }
 
-__device__ __forceinline__ int tile_row(int pr, int r) { return min(pr + 32 * r, TP - 1); }
+template <int TE>
+__device__ __forceinline__ int tile_row(int pr, int r) { return min(pr + 32 * r, TE - 1); }
 
 // acc[r][c] += sum_k A[pr + 32 r][k] W[k][col(c)] over k < K, col(c) = 4 hc + c, 64 + 4 hc + c - 4;
 // rows past the tile are clamped to its last one and not stored
-template <int K>
+template <int K, int TE>
 __device__ __forceinline__ void layer_product(const float* A, int as, const float* W, int ws, int pr, int hc,
-                                              float (&acc)[4][8]) {
+                                              float (&acc)[rows_of(TE)][8]) {
 #pragma unroll 2
   for (int k = 0; k < K; k += 4) {
-    float4 a4[4];
+    float4 a4[rows_of(TE)];
 #pragma unroll
-    for (int r = 0; r < 4; r++) a4[r] = ld4(A + tile_row(pr, r) * as + k);
+    for (int r = 0; r < rows_of(TE); r++) a4[r] = ld4(A + tile_row<TE>(pr, r) * as + k);
 #pragma unroll
     for (int u = 0; u < 4; u++) {
       const float4 w0 = ld4(W + (k + u) * ws + 4 * hc), w1 = ld4(W + (k + u) * ws + 64 + 4 * hc);
       const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
-      for (int r = 0; r < 4; r++) {
+      for (int r = 0; r < rows_of(TE); r++) {
         const float av = u == 0 ? a4[r].x : u == 1 ? a4[r].y : u == 2 ? a4[r].z : a4[r].w;
 #pragma unroll
         for (int c = 0; c < 8; c++) acc[r][c] = fmaf(av, wv[c], acc[r][c]);
@@ -157,22 +164,22 @@ __device__ __forceinline__ void layer_product(const float* A, int as, const floa
 }
 
 // h1, h2 and y of the tile in shared memory
-template <bool BF16>
+template <bool BF16, int TE>
 __device__ void forward_tile(float* sm, float b3) {
   const int t = threadIdx.x, pr = t >> 4, hc = t & 15;
-  float acc[4][8];
+  float acc[rows_of(TE)][8];
   auto start = [&](int bias) {
     const float4 b0 = ld4(sm + bias + 4 * hc), b1 = ld4(sm + bias + 64 + 4 * hc);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
+    for (int r = 0; r < rows_of(TE); r++) {
       acc[r][0] = b0.x, acc[r][1] = b0.y, acc[r][2] = b0.z, acc[r][3] = b0.w;
       acc[r][4] = b1.x, acc[r][5] = b1.y, acc[r][6] = b1.z, acc[r][7] = b1.w;
     }
   };
   auto finish = [&](int dst) {
 #pragma unroll
-    for (int r = 0; r < 4; r++)
-      if (pr + 32 * r < TP)
+    for (int r = 0; r < rows_of(TE); r++)
+      if (pr + 32 * r < TE)
 #pragma unroll
         for (int h = 0; h < 2; h++)
           *(float4*)(sm + dst + (pr + 32 * r) * HS + 64 * h + 4 * hc) =
@@ -180,18 +187,18 @@ __device__ void forward_tile(float* sm, float b3) {
                           q<BF16>(tanhf(acc[r][4 * h + 2])), q<BF16>(tanhf(acc[r][4 * h + 3])));
   };
   start(S_B1);
-  layer_product<NIN>(sm + S_X, XS, sm + S_W1, NH, pr, hc, acc);
+  layer_product<NIN, TE>(sm + S_X, XS, sm + S_W1, NH, pr, hc, acc);
   finish(S_H1);
   __syncthreads();
   start(S_B2);
-  layer_product<NH>(sm + S_H1, HS, sm + S_W2, HS, pr, hc, acc);
+  layer_product<NH, TE>(sm + S_H1, HS, sm + S_W2, HS, pr, hc, acc);
   finish(S_H2);
   __syncthreads();
-  // output: warp w handles points 7w .. 7w+6
+  // output: warp w handles points w TE / 16 .. + TE / 16 - 1
   const int warp = t >> 5, lane = t & 31;
 #pragma unroll
-  for (int pp = 0; pp < TP / (NT / 32); pp++) {
-    const int p = warp * (TP / (NT / 32)) + pp;
+  for (int pp = 0; pp < TE / (NT / 32); pp++) {
+    const int p = warp * (TE / (NT / 32)) + pp;
     float s = 0.0f;
 #pragma unroll
     for (int c = 0; c < 4; c++) s = fmaf(sm[S_H2 + p * HS + lane + 32 * c], sm[S_W3 + lane + 32 * c], s);
@@ -201,7 +208,7 @@ __device__ void forward_tile(float* sm, float b3) {
   __syncthreads();
 }
 
-template <bool BF16>
+template <bool BF16, int TE>
 __global__ void __launch_bounds__(NT, 1) mlp_forward_kernel(const float* __restrict__ P, const float* __restrict__ mu,
                                                            const float* __restrict__ inv_sd,
                                                            const float* __restrict__ D, int64_t n,
@@ -211,17 +218,18 @@ __global__ void __launch_bounds__(NT, 1) mlp_forward_kernel(const float* __restr
   const float b3 = P[OB3];
   // the block's share of the points
   const int64_t per = (n + gridDim.x - 1) / gridDim.x, r1 = min(n, (blockIdx.x + 1) * per);
-  for (int64_t r0 = blockIdx.x * per; r0 < r1; r0 += TP) {
+  for (int64_t r0 = blockIdx.x * per; r0 < r1; r0 += TE) {
     __syncthreads();
-    load_tile<BF16>(D, mu, inv_sd, r1, r0, sm);
+    load_tile<BF16, TE>(D, mu, inv_sd, r1, r0, sm);
     __syncthreads();
-    forward_tile<BF16>(sm, b3);
-    for (int p = threadIdx.x; p < TP; p += NT)
+    forward_tile<BF16, TE>(sm, b3);
+    for (int p = threadIdx.x; p < TE; p += NT)
       if (r0 + p < r1) y[r0 + p] = sm[S_Y + p];
   }
 }
 
 // Loss and gradient: every block handles its share of the points and writes part[block * (NPAR + 1) + q] (q < NPAR: gradient, q = NPAR: sum of (y - t)^2).
+template <int TE>
 __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict__ P, const float* __restrict__ mu,
                                                         const float* __restrict__ inv_sd,
                                                         const float* __restrict__ D, const float* __restrict__ tgt,
@@ -244,20 +252,20 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
 #pragma unroll
     for (int c = 0; c < 2; c++) gW1[a][c] = 0.0f;
   // column sums over the thread's quarter of the tile
-  const int sj = t & (NH - 1), s0 = (t >> 7) * (TP / 4);
+  const int sj = t & (NH - 1), s0 = (t >> 7) * (TE / 4);
   float* sacc = sm + S_ACC + (t >> 7) * 3 * NH;
   float loss = 0.0f, gb3 = 0.0f;
   const float scale = 2.0f / (float)n;
   const int64_t per = (n + gridDim.x - 1) / gridDim.x, row1 = min(n, (blockIdx.x + 1) * per);
-  for (int64_t row0 = blockIdx.x * per; row0 < row1; row0 += TP) {
-    const int np = (int)min((int64_t)TP, row1 - row0);   // points of this tile
+  for (int64_t row0 = blockIdx.x * per; row0 < row1; row0 += TE) {
+    const int np = (int)min((int64_t)TE, row1 - row0);   // points of this tile
     __syncthreads();
-    load_tile<false>(D, mu, inv_sd, row1, row0, sm);
-    for (int p = t; p < TP; p += NT) sm[S_T + p] = p < np ? tgt[row0 + p] : 0.0f;
+    load_tile<false, TE>(D, mu, inv_sd, row1, row0, sm);
+    for (int p = t; p < TE; p += NT) sm[S_T + p] = p < np ? tgt[row0 + p] : 0.0f;
     __syncthreads();
-    forward_tile<false>(sm, b3);
+    forward_tile<false, TE>(sm, b3);
     // dy = 2 (y - t) / n for the points of the tile, 0 past n
-    if (t < TP) {
+    if (t < TE) {
       const float r = t < np ? sm[S_Y + t] - sm[S_T + t] : 0.0f;
       loss += r * r;
       sm[S_Y + t] = scale * r;
@@ -267,17 +275,17 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
     {
       float s = 0.0f;
 #pragma unroll 8
-      for (int p = s0; p < s0 + TP / 4; p++) s = fmaf(sm[S_Y + p], sm[S_H2 + p * HS + sj], s);
+      for (int p = s0; p < s0 + TE / 4; p++) s = fmaf(sm[S_Y + p], sm[S_H2 + p * HS + sj], s);
       sacc[2 * NH + sj] += s;
     }
     if (t == 0) {
       float s = 0.0f;
-      for (int p = 0; p < TP; p++) s += sm[S_Y + p];
+      for (int p = 0; p < TE; p++) s += sm[S_Y + p];
       gb3 += s;
     }
     __syncthreads();
     // g2 = dy w3 (1 - h2^2), in place over h2
-    for (int e = t; e < TP * NH / 4; e += NT) {
+    for (int e = t; e < TE * NH / 4; e += NT) {
       const int p = e >> 5, j = 4 * (e & 31);
       float4 h = ld4(sm + S_H2 + p * HS + j);
       const float4 w = ld4(sm + S_W3 + j);
@@ -293,7 +301,7 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
     {
       float s = 0.0f;
 #pragma unroll 8
-      for (int p = s0; p < s0 + TP / 4; p++) s += sm[S_H2 + p * HS + sj];
+      for (int p = s0; p < s0 + TE / 4; p++) s += sm[S_H2 + p * HS + sj];
       sacc[NH + sj] += s;
     }
 #pragma unroll 2
@@ -309,31 +317,31 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
     __syncthreads();
     // g1[p][i] = (sum_j g2[p][j] W2[i][j]) (1 - h1[p][i]^2), in place over h1; units hc + 16 c
     {
-      float acc[4][8];
+      float acc[rows_of(TE)][8];
 #pragma unroll
-      for (int r = 0; r < 4; r++)
+      for (int r = 0; r < rows_of(TE); r++)
 #pragma unroll
         for (int c = 0; c < 8; c++) acc[r][c] = 0.0f;
 #pragma unroll 2
       for (int j = 0; j < NH; j += 4) {
-        float4 g4[4];
+        float4 g4[rows_of(TE)];
 #pragma unroll
-        for (int r = 0; r < 4; r++) g4[r] = ld4(sm + S_H2 + tile_row(pr, r) * HS + j);
+        for (int r = 0; r < rows_of(TE); r++) g4[r] = ld4(sm + S_H2 + tile_row<TE>(pr, r) * HS + j);
 #pragma unroll
         for (int c = 0; c < 8; c++) {
           const float4 w = ld4(sm + S_W2 + (hc + 16 * c) * HS + j);
 #pragma unroll
-          for (int r = 0; r < 4; r++)
+          for (int r = 0; r < rows_of(TE); r++)
             acc[r][c] = fmaf(g4[r].w, w.w, fmaf(g4[r].z, w.z, fmaf(g4[r].y, w.y, fmaf(g4[r].x, w.x, acc[r][c]))));
         }
       }
       __syncthreads();
 #pragma unroll
-      for (int r = 0; r < 4; r++)
+      for (int r = 0; r < rows_of(TE); r++)
 #pragma unroll
         for (int c = 0; c < 8; c++) {
           const int p = pr + 32 * r, i = hc + 16 * c;
-          if (p >= TP) continue;
+          if (p >= TE) continue;
           const float h = sm[S_H1 + p * HS + i];
           sm[S_H1 + p * HS + i] = acc[r][c] * (1.0f - h * h);
         }
@@ -343,7 +351,7 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
     {
       float s = 0.0f;
 #pragma unroll 8
-      for (int p = s0; p < s0 + TP / 4; p++) s += sm[S_H1 + p * HS + sj];
+      for (int p = s0; p < s0 + TE / 4; p++) s += sm[S_H1 + p * HS + sj];
       sacc[sj] += s;
     }
 #pragma unroll 4
@@ -378,7 +386,7 @@ __global__ void __launch_bounds__(NT, 1) mlp_grad_kernel(const float* __restrict
     out[OW3 + t] = quarters(2 * NH);
   }
   if (t == 0) out[OB3] = gb3;
-  // loss: threads < TP hold their points' squared residuals
+  // loss: threads < TE hold their points' squared residuals
   __shared__ float sl[NT / 32];
   float l = loss;
   for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -517,15 +525,18 @@ unsigned mlp_grid(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 63) / 64, sms));   // at least 64 points each
 }
 
+// no block of nb has more than SMALL points
+bool small_tiles(int64_t n, unsigned nb) { return (n + nb - 1) / nb <= SMALL; }
+
 cudaError_t set_smem_attrs() {
   static bool done = false;
   if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(mlp_forward_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kMlpSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_forward_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
+  const void* ks[] = {(const void*)mlp_forward_kernel<false, TP>, (const void*)mlp_forward_kernel<false, SMALL>,
+                      (const void*)mlp_forward_kernel<true, TP>,  (const void*)mlp_forward_kernel<true, SMALL>,
+                      (const void*)mlp_grad_kernel<TP>,           (const void*)mlp_grad_kernel<SMALL>};
+  cudaError_t e = cudaSuccess;
+  for (const void* k : ks)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem);
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -661,10 +672,11 @@ extern "C" int kscf_mlp_forward(const float* params, const float* mu, const floa
   if (n == 0) return KSCF_OK;
   KSCF_CUDA_TRY(set_smem_attrs());
   cudaStream_t st = (cudaStream_t)stream;
-  if (precision == KSCF_MLP_FP32)
-    mlp_forward_kernel<false><<<mlp_grid(n), NT, kMlpSmem, st>>>(params, mu, inv_sd, D, n, y);
-  else
-    mlp_forward_kernel<true><<<mlp_grid(n), NT, kMlpSmem, st>>>(params, mu, inv_sd, D, n, y);
+  const unsigned nb = mlp_grid(n);
+  const bool small = small_tiles(n, nb);
+  auto k = precision == KSCF_MLP_FP32 ? (small ? mlp_forward_kernel<false, SMALL> : mlp_forward_kernel<false, TP>)
+                                      : (small ? mlp_forward_kernel<true, SMALL> : mlp_forward_kernel<true, TP>);
+  k<<<nb, NT, kMlpSmem, st>>>(params, mu, inv_sd, D, n, y);
   count_launch();
   KSCF_CUDA_TRY(cudaGetLastError());
   return KSCF_OK;
@@ -694,7 +706,8 @@ extern "C" int kscf_mlp_loss_grad(const float* params, const float* mu, const fl
   }
   KSCF_CUDA_TRY(set_smem_attrs());
   cudaStream_t st = (cudaStream_t)stream;
-  mlp_grad_kernel<<<nb, NT, kMlpSmem, st>>>(params, mu, inv_sd, D, t, n, (float*)work);
+  auto k = small_tiles(n, nb) ? mlp_grad_kernel<SMALL> : mlp_grad_kernel<TP>;
+  k<<<nb, NT, kMlpSmem, st>>>(params, mu, inv_sd, D, t, n, (float*)work);
   count_launch();
   KSCF_CUDA_TRY(cudaGetLastError());
   mlp_reduce_kernel<<<(NPAR + 1 + 31) / 32, 256, 0, st>>>((const float*)work, (int)nb, n, grad, loss);
