@@ -123,8 +123,10 @@ __device__ __noinline__ double star64(const Step64& a, const double* in, int64_t
   return acc;
 }
 
-// SMEM_KB: the brick has at most KSCF_BRICK_ATOMS atoms with projectors, whose coefficients
-// are staged in shared memory with the first S_ENT entries
+// SMEM_KB: the bricks have at most KSCF_BRICK_ATOMS atoms with projectors (so that 16 bits hold
+// the number of an entry inside its brick), whose coefficients are staged in shared memory with
+// the first S_ENT entries
+static_assert(KSCF_BRICK_ATOMS * 512 < 65536, "entry numbers of a brick in 16 bits");
 // CM: `in` is chunk-major (ld_in = S_NV)
 template <bool SMEM_KB, bool CM>
 __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
   double* kbc = (double*)(smb + S_KBC);        // [atom][l][4]
   double* echi = (double*)(smb + S_CHI);       // [entry][4]
   uint32_t* ew = (uint32_t*)(smb + S_EW);
-  uint16_t* kbp = (uint16_t*)(smb + S_KBP);    // [513]: first entry of each point
+  uint16_t* kbp = (uint16_t*)(smb + S_KBP);    // [513]: first entry of each point (SMEM_KB)
   __shared__ int s_max[S_NV];
   int cell, chunk;
   {
@@ -163,9 +165,9 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
       if (nb[f] >= 0) e = max(e, __ldg(a.emax_in + (int64_t)nb[f] * a.wq + col));
   }
   const int64_t e0 = __ldg(a.kb_ptr + b0), e1 = __ldg(a.kb_ptr + b0 + 512);
-  for (int t = tid; t <= 512; t += S_THR) kbp[t] = (uint16_t)(__ldg(a.kb_ptr + b0 + t) - e0);
   for (int t = tid; t < 512; t += S_THR) vs[t] = __ldg(a.V + b0 + t);
   if (SMEM_KB) {
+    for (int t = tid; t <= 512; t += S_THR) kbp[t] = (uint16_t)(__ldg(a.kb_ptr + b0 + t) - e0);
     const int nat = __ldg(a.bnat + cell);
     for (int t = tid; t < nat * 4 * S_NV; t += S_THR) {
       const int at = __ldg(a.batoms + (int64_t)cell * KSCF_BRICK_ATOMS + t / (4 * S_NV)), l = (t / S_NV) & 3;
@@ -270,9 +272,9 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
       t = ku * (double)((s.hi << (FIX_LO - S_DROP)) + (s.lo >> S_DROP));
     }
     t = fma(vs[r], yv[z], t);
-    for (int i = kbp[r], i1 = kbp[r + 1]; i < i1; i++) {
-      const int64_t qe = e0 + i;
-      if (SMEM_KB) {
+    if (SMEM_KB) {
+      for (int i = kbp[r], i1 = kbp[r + 1]; i < i1; i++) {
+        const int64_t qe = e0 + i;
         uint32_t word;
         double2 c0, c1;
         if (i < S_ENT) {
@@ -289,7 +291,9 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
         t = fma(c0.y, cf[S_NV], t);
         t = fma(c1.x, cf[2 * S_NV], t);
         t = fma(c1.y, cf[3 * S_NV], t);
-      } else {
+      }
+    } else {   // any number of entries in the brick
+      for (int64_t qe = __ldg(a.kb_ptr + b0 + r), q1 = __ldg(a.kb_ptr + b0 + r + 1); qe < q1; qe++) {
         const double* cf = a.coef + (int64_t)__ldg(a.kb_atom + qe) * 4 * a.cld + col;
         const double* ch = a.kb_chi + 4 * qe;
         t = fma(ch[0], cf[0], t);
