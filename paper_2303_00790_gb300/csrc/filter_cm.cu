@@ -152,7 +152,8 @@ constexpr int LDG_CORE = 0, LDG_ACC = 32768, LDG_KBC = 65536, LDG_EW = LDG_KBC +
 // (their points are padding and never stored).  The nonlocal gather of the z pass reads
 // the projection coefficients of the cell's KB atoms and the cell's entries from shared
 // memory, staged at the start together with the core (SMEM_KB; otherwise from global
-// memory).  B: brick edge (8 or 16), which sets the slot steps inside a cell.
+// memory, through the 64-bit entry pointers: 16 bits number the entries of a cell with at most
+// KSCF_BRICK_ATOMS atoms only).  B: brick edge (8 or 16), which sets the slot steps inside a cell.
 template <bool SMEM_KB, int B>
 __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t* __restrict__ lines,
                                                         const uint8_t* __restrict__ nlines,
@@ -168,7 +169,7 @@ __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t*
   uint32_t* ew = (uint32_t*)(smw + LDG_EW);
   float4* echi = (float4*)(smw + LDG_ECHI);
   const float4* prev4 = (const float4*)(smw + LDG_PREV);   // [512][4]: Y_{j-2} rows of this cell
-  uint16_t* kbp = (uint16_t*)(smw + LDG_KBP);              // [513]: first entry of each point, from e0
+  uint16_t* kbp = (uint16_t*)(smw + LDG_KBP);              // [513]: first entry of each point, from e0 (SMEM_KB)
   auto sl = [](int x, int y, int z) { return (z * 8 + y) * 8 + (x ^ (y & 1)); };
   int c, cell;
   if (!cta_item(a, &c, &cell)) return;
@@ -208,9 +209,9 @@ __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t*
     }
   }
   const int64_t e0 = __ldg(a.kb_ptr + k0), e1 = __ldg(a.kb_ptr + k0 + 512);
-  const int ne = (int)(e1 - e0);
-  for (int t = tid; t <= 512; t += 256) kbp[t] = (uint16_t)(__ldg(a.kb_ptr + k0 + t) - e0);
   if (SMEM_KB) {
+    const int ne = (int)(e1 - e0);
+    for (int t = tid; t <= 512; t += 256) kbp[t] = (uint16_t)(__ldg(a.kb_ptr + k0 + t) - e0);
     const int nat = __ldg(bnat + cell);
     for (int t = tid; t < nat * 16; t += 256) {
       const int at = __ldg(batoms + (int64_t)cell * KSCF_BRICK_ATOMS + (t >> 4));
@@ -315,11 +316,17 @@ __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t*
         // nonlocal term of this point: sum over its KB entries (cell order) of
         // chi_l(e) * coef(atom(e), l), accumulated in registers
         const int sloc = z * 64 + lz;
-        for (int i = kbp[sloc], i1 = kbp[sloc + 1]; i < i1; i++) {
-          const int64_t qe = e0 + i;
-          float4 ch;
-          float4 cv[4];
-          if (SMEM_KB) {
+        auto add = [&](float4 ch, const float4 (&cv)[4]) {
+          hy = f4_fma(f2(ch.x), cv[0], hy);
+          hy = f4_fma(f2(ch.y), cv[1], hy);
+          hy = f4_fma(f2(ch.z), cv[2], hy);
+          hy = f4_fma(f2(ch.w), cv[3], hy);
+        };
+        if (SMEM_KB) {
+          for (int i = kbp[sloc], i1 = kbp[sloc + 1]; i < i1; i++) {
+            const int64_t qe = e0 + i;
+            float4 ch;
+            float4 cv[4];
             uint32_t word;
             if (i < LDG_ENT) {
               word = ew[i];
@@ -331,16 +338,16 @@ __global__ void __launch_bounds__(256, 2) cm_step_ldg16(CmArgs a, const uint8_t*
             const float4* cf = kbc + (word >> 16) * 16 + vp;
 #pragma unroll
             for (int l = 0; l < 4; l++) cv[l] = cf[4 * l];
-          } else {
-            ch = __ldg((const float4*)(a.kb_chi + 4 * qe));
+            add(ch, cv);
+          }
+        } else {   // any number of entries in the cell
+          for (int64_t qe = __ldg(a.kb_ptr + k0 + sloc), q1 = __ldg(a.kb_ptr + k0 + sloc + 1); qe < q1; qe++) {
+            float4 cv[4];
             const float* g = a.coef + (int64_t)__ldg(a.kb_atom + qe) * 4 * a.cld + c * 16 + vl;
 #pragma unroll
             for (int l = 0; l < 4; l++) cv[l] = ld4(g + l * a.cld);
+            add(__ldg((const float4*)(a.kb_chi + 4 * qe)), cv);
           }
-          hy = f4_fma(f2(ch.x), cv[0], hy);
-          hy = f4_fma(f2(ch.y), cv[1], hy);
-          hy = f4_fma(f2(ch.z), cv[2], hy);
-          hy = f4_fma(f2(ch.w), cv[3], hy);
         }
         float4 r = f4_mul(alpha, f4_fma(negc, yc, hy));
         if (prevp) {

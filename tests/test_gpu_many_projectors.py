@@ -84,3 +84,20 @@ def test_fp64_star_kernel(kscf, n_atoms, degree):
         ref = filter_reference(kscf, both[16], P, degree, 1.0, 80.0, -2.0)
     got = kscf.kscf_slots_to_points(ham, Y, torch.empty_like(P))
     assert (got - ref).abs().max() <= 1e-11 * ref.abs().max()
+
+
+@pytest.mark.parametrize("brick", [8, 16])
+@pytest.mark.parametrize("n_atoms", [40, 200])
+def test_fp32_filter_kernel(kscf, n_atoms, brick):
+    """FP32 against the FP64 reference: the 842 roundings of a step, u = 2^-24, bound nothing useful
+    when they all add up; as a random walk they give sqrt(842) * 60 u = 1.0e-4 of max|y|, three times
+    over the three steps."""
+    both = systems(kscf, n_atoms)
+    n, k, degree = both[8][0].info["n_points"], 20, 3
+    P = torch.tensor(np.random.default_rng(k).standard_normal((n, k)), device="cuda")
+    ham = both[brick][1]
+    X = in_slots(kscf, ham, P.float())
+    kscf.kscf_chebyshev_filter(ham, X, degree, 1.0, 80.0, -2.0)
+    got = kscf.kscf_slots_to_points(ham, X, torch.empty_like(P, dtype=torch.float32)).double()
+    ref = filter_reference(kscf, both[16], P, degree, 1.0, 80.0, -2.0)
+    assert (got - ref).abs().max() <= 3e-4 * ref.abs().max()
