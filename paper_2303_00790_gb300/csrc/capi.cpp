@@ -278,7 +278,8 @@ int rotate_inplace(const Ham& H, void* X, int64_t ld, int k, int dtype, int mode
     const int* only_if = nullptr;
     if (gw.rot64)
       KSCF_CUDA_TRY(launch_rotate_f64tc((const double*)Xr, ld, (const double*)Qm, k, nr, k, k, upper, (double*)Xr, ld,
-                                        gw.buf, gw.bytes, map, gw.gram64, r0 > 0, &only_if, st));
+                                        gw.buf, gw.bytes, map, gw.gram64 || r0 > 0 ? 0 : rows, r0 > 0, &only_if,
+                                        st));
     KSCF_CUDA_TRY(launch_rotate_native(Xr, ld, Qm, k, nr, k, k, dtype, panel, k, st, map, only_if));
     KSCF_CUDA_TRY(launch_copy_cols(panel, k, Xr, ld, nr, k, dtype, st, map, only_if));
   }
@@ -869,10 +870,14 @@ extern "C" int kscf_rotate(const void* A, int64_t lda, const double* Q, int64_t 
   // native: convert Q into the work buffer (column-major, ld = kin), then rotate
   double* Qc = (double*)work;
   if (dtype == KSCF_F64 && ldq == kin) {
+    // on the tensor cores in row panels, when the buffer holds one
     const int* only_if = nullptr;
-    if (rotate_f64tc_wanted(rows, kin, kout) && work_bytes >= rotate_f64tc_work_bytes(rows, kin, kout))
-      KSCF_CUDA_TRY(launch_rotate_f64tc((const double*)A, lda, Q, ldq, rows, kin, kout, false, (double*)out, ldo, work,
-                                        work_bytes, nullptr, false, false, &only_if, st));
+    const int64_t pr = rotate_f64tc_panel(rows, kin);
+    if (rotate_f64tc_wanted(rows, kin, kout) && work_bytes >= rotate_f64tc_work_bytes(pr, kin, kout))
+      for (int64_t r0 = 0; r0 < rows; r0 += pr)
+        KSCF_CUDA_TRY(launch_rotate_f64tc((const double*)A + r0 * lda, lda, Q, ldq, std::min(pr, rows - r0), kin, kout,
+                                          false, (double*)out + r0 * ldo, ldo, work, work_bytes, nullptr,
+                                          r0 > 0 ? 0 : rows, r0 > 0, &only_if, st));
     KSCF_CUDA_TRY(launch_rotate_native(A, lda, Q, ldq, rows, kin, kout, dtype, out, ldo, st, nullptr, only_if));
     return KSCF_OK;
   }
@@ -897,7 +902,8 @@ extern "C" int kscf_gemm_workspace_size(int op, int64_t rows, int m, int n, int 
     *bytes = op == 0 ? 256 : kscf_align256((size_t)m * n * esize(dtype));
   if (mode == KSCF_GEMM_NATIVE && dtype == KSCF_F64) {
     if (op == 0 && gram_f64tc_wanted(rows)) *bytes = std::max(*bytes, gram_f64tc_work_bytes(rows, m, n));
-    if (op != 0 && rotate_f64tc_wanted(rows, m, n)) *bytes = std::max(*bytes, rotate_f64tc_work_bytes(rows, m, n));
+    if (op != 0 && rotate_f64tc_wanted(rows, m, n))
+      *bytes = std::max(*bytes, rotate_f64tc_work_bytes(rotate_f64tc_panel(rows, m), m, n));
   }
   return KSCF_OK;
 }

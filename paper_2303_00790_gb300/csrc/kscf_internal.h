@@ -212,6 +212,7 @@ bool rotate_f64tc_wanted(int64_t rows, int kin, int kout);
 size_t gram_f64tc_work_bytes(int64_t rows, int m, int n);
 bool gram_f64tc_fits(int64_t rows, int m, int n, bool same, size_t bytes);
 size_t rotate_f64tc_work_bytes(int64_t rows, int kin, int kout);
+int64_t rotate_f64tc_panel(int64_t rows, int kin);   // rows per panel that bound a rotation's work buffer
 // C (zeroed here) = scale * A^T B over the (mapped) rows; symmetric: A^T B is known to be symmetric (upper tiles,
 // mirrored).  Operands that hold a NaN, an Inf or extreme magnitudes go through launch_gram_native.
 cudaError_t launch_gram_f64tc(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t rows, int m, int n,
@@ -219,11 +220,12 @@ cudaError_t launch_gram_f64tc(const double* A, int64_t lda, const double* B, int
                               const int32_t* rowmap, cudaStream_t st);
 // out = A Q (out may be A; rows of both through rowmap).  *flag_out: device word set when Q or A hold a NaN, an
 // Inf or extreme magnitudes; out is then untouched and the caller's general path runs behind only_if.
-// upper: Q is upper triangular.  reuse_max: the work buffer still holds the column maxima that a Gram with the same
-// A (all rows) left there; reuse_q: and Q's digits from the previous row panel.
+// upper: Q is upper triangular.  max_rows: the columns' maxima are taken over that many rows of A, all panels' rows
+// for the first panel of a product; 0: the work buffer still holds them, from a Gram with the same A or from the
+// first panel.  reuse_q: it also holds Q's digits, from the first panel.
 cudaError_t launch_rotate_f64tc(const double* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin,
                                 int kout, bool upper, double* out, int64_t ldo, void* work, size_t work_bytes,
-                                const int32_t* rowmap, bool reuse_max, bool reuse_q, const int** flag_out,
+                                const int32_t* rowmap, int64_t max_rows, bool reuse_q, const int** flag_out,
                                 cudaStream_t st);
 cudaError_t f64tc_status(bool reset, unsigned int* status);
 cudaError_t launch_symmetrize(double* C, int k, int64_t ldc, cudaStream_t st);
