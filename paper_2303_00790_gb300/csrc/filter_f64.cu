@@ -6,21 +6,33 @@
 //
 // The GB300 issues one FP64 warp instruction per 64 cycles and SM sub-partition, so the star is
 // evaluated in integers (fixlap.cuh's weights): a CTA takes one brick and four vectors,
-// converts the brick and its six halos once into 57-bit fixed point in two limbs (in units of
-// the largest value of the vector in the brick and its neighbours, whose exponents every step
-// writes for the next one, emax), and then every thread evaluates the 37-point sums of eight
-// points from shared memory: 36 loads at register + constant addresses, six additions of 32
-// bits per limb and distance, seven 32 x 32 -> 64 products per limb.  The sums are exact; FP64 is
-// left for their conversion, the potential, the recurrence and the nonlocal term.
-// What bounds it: the FP64 pipe is 43 % busy (10.5 instructions per point and vector, 4.5 of them
-// the nonlocal term with its divergence), the rest is the load and conversion phase of 5.5 values per
-// point that two CTAs per SM hide half.  One degree step of 234,489 points x 850 vectors: 7.4 ms
-// (gather 1.1 ms beside it) against 23.5 ms of the FP64 star; whole 12-step filter 295 -> 101 ms.
-// Also built: the 13-point sums as three line passes over register windows as in the FP32
-// filter, three CTAs per SM (6.4 ms, but a less accurate order of the last operations), and 512
-// threads with half the planes each (7.9 ms).  Error after 10 steps against extended precision:
-// 1.6-2.4e-16 per column, FP64 star 2.4-3.3e-16.
-// A vector with a NaN, an Inf or values below 2^-895 in the brick or its neighbours takes the
+// converts the brick and its six halos once into 60-bit fixed point (in units of 2^-60 of 2^E, the
+// power of two above the largest value of the vector in the brick and its neighbours, whose exponents
+// every step writes for the next one, emax), and then every thread evaluates the 37-point sums of eight
+// points from shared memory: 36 loads at register + constant addresses, five 64-bit additions per
+// distance, fourteen 32 x 32 -> 64 products.  The sums are exact; FP64 is left for their
+// conversion, the potential, the recurrence and the nonlocal term.
+//
+// Accuracy: no point's star is less accurate than in FP64, also where its neighbourhood lies far below
+// 2^E.  A point whose own and next values are below S_STEEP gets its star apart (steep_points): the FP64
+// star when a CTA has few of them, else from a second pass in a window 29 bits lower (a sum modulo
+// 2^60, which the first pass's leading bits complete), and the FP64 star below 2^-36 of 2^E.  Measured
+// against quadruple precision, error / (2^-53 sum |w v|) over fields exp(-r/2) .. exp(-4 r),
+// Gaussians, waves and noise: rms 0.06-0.77 (FP64 star 0.22-0.94), largest 0.8-5.4 (0.9-5.4); filters of 8 to
+// 12 steps with the recurrence's scalars as given: 1.3e-16 of a column's norm (FP64 star, whose
+// seven weights are rounded, 6.0e-16 to 8.8e-16; the scalars' own rounding moves a result by 1e-15).
+//
+// What bounds it: the FP64 pipe (10.5 instructions per point and vector, 4.5 of them the nonlocal term
+// with its divergence) is busy 40 % of the time, the rest is the load and conversion phase of 5.5
+// values per point that two CTAs per SM hide half.  One degree step of 234,489 points x 850 vectors:
+// 8.4 ms (gather 1.1 ms beside it) against 23.5 ms of the FP64 star; whole 12-step filter 295 -> 114 ms.
+// Two limbs of 29 bits and no second look at small values took 102 ms, 105 ms 60 bits alone; a value of 1e-3
+// of 2^E then had 47 bits, orbitals exp(-r) lost three digits in their tails.  Orbitals exp(-r/2), exp(-r)
+// and exp(-2 r) about 200 centres (most CTAs make the second pass): 40, 59, 63 ms, FP64 star 70.
+// Also built: the small values' stars one by one by the warp that meets them (120 to 137 ms: code that few
+// warps run is fetched when it runs, and it shared the hot loop's registers), the 13-point sums as three
+// line passes over register windows as in the FP32 filter, and 512 threads with half the planes each.
+// A vector with a NaN, an Inf or nothing above 2^-767 in the brick or its neighbours takes the
 // FP64 star, as do 16^3 bricks (cheb_step_generic).
 #include <cuda_runtime.h>
 
@@ -36,9 +48,17 @@ namespace kscf {
 
 namespace {
 
-constexpr int S_BITS = 57;                       // |value| < 2^E -> |fixed| <= 2^57, unit 2^(E - 57)
-constexpr int S_MULT = 64;                       // largest multiple of the integer weights
-constexpr int S_DROP = 25;                       // low bits of the sum not kept (2^-62 of the largest sum)
+constexpr int S_BITS = 60;                       // |value| < 2^E -> |fixed| <= 2^60, unit 2^(E - 60)
+constexpr int S_MULT = 56;                       // largest multiple of the integer weights, and twice the smallest
+// Low bits of the sum that its conversion leaves out: the largest sum (21.2 2^E, 2^89.9 units) keeps 63 bits
+constexpr int S_DROP = 27;
+constexpr int S_FINE = 29;                       // the second window lies this many bits lower
+// 5 |v| at the point + |v| at its six neighbours, 1/1.7 of what these put into sum |w v|, below
+// which the sum is too coarse: 2^-6 of 2^E, in upper words (2^28 for 2^E).  The sum is off by at most
+// 13.5 2^-60 2^E (cut values 10.6, S_DROP 2.9), so by 4 2^-53 sum |w v| at this line, where the FP64 star has
+// 39 roundings; measured there 1.2 to 1.9, FP64 1.5 to 3.9.  (Twice the line: 0.4 to 1.6, 3 ms slower.)
+constexpr uint32_t S_STEEP = 1u << 22;
+constexpr int S_FEW = 192;                       // points of a CTA up to which they are taken one by one
 constexpr int S_NV = 4;                          // vectors per CTA
 constexpr int S_ENT = 256;                       // KB entries staged in shared memory
 constexpr int S_THR = 256;                       // threads: 64 points of a plane x S_NV
@@ -49,7 +69,7 @@ constexpr int P_XL = 64, P_XH = 112, P_YL = 160, P_YH = 208, P_PLANE = 256, P_ZL
               P_ALL = P_ZH + 6 * 64;
 constexpr int S_FIX = 0, S_V = S_FIX + P_ALL * S_NV * 8, S_KBC = S_V + 512 * 8,
               S_CHI = S_KBC + KSCF_BRICK_ATOMS * 4 * S_NV * 8, S_EW = S_CHI + S_ENT * 32, S_KBP = S_EW + S_ENT * 4,
-              S_SMEM = S_KBP + 514 * 2;
+              S_LEFT = S_KBP + 514 * 2, S_SMEM = S_LEFT + 4 + S_FEW * 2;
 
 // element (chunk c of S_NV columns, slot s, v) of a block at p[c * cs + s * ld + v]
 struct Step64 {
@@ -63,7 +83,8 @@ struct Step64 {
   int w, nchunk, wq;    // columns, chunks of S_NV, row length of emax
   double alpha, beta, c;
   int wt[7];            // integer weights: m 831600 (3 w_0, w_1 .. w_6)
-  double ku;            // -2^S_DROP / (2 h^2 831600 m)
+  uint32_t wabs[7];     // their magnitudes
+  double ku;            // -1 / (2 h^2 831600 m)
   const double* coef;
   int64_t cld;
   const double* V;
@@ -84,20 +105,18 @@ __device__ __forceinline__ uint32_t abs_hw(double v) { return (uint32_t)__double
 // biased exponent of a maximum's high word; 0 only for zero
 __device__ __forceinline__ int hw_exp(uint32_t hw) { return max((int)(hw >> 20), hw ? 1 : 0); }
 
-// value -> floor(value 2^(S_BITS - E)) (negative values: one's complement) as limbs hi 2^29 + lo,
-// lo in [0, 2^29) stored less 2^28 so that six of them add up in 32 bits.  That constant, and the
-// mean of what is cut off, drop out of the star: its weights add up to zero.  e: the biased
+// value -> floor(value 2^(S_BITS - E)) (negative values: one's complement).  What is cut off has
+// the same mean everywhere and drops out of the star: its weights add up to zero.  e: the biased
 // exponent with E = e - 1022.
-__device__ __forceinline__ int2 fix57(double v, int e) {
+__device__ __forceinline__ long long fix60(double v, int e) {
   const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
   const int n = min(e - (int)((h >> 20) & 0x7ff), 63);
   const uint32_t mh = (h & 0xfffffu) | 0x100000u;
-  unsigned long long t = (((unsigned long long)mh << 32) | l) << (S_BITS - 53);
-  t >>= n;
-  const unsigned long long x = t ^ (unsigned long long)((long long)(int)h >> 31);
-  return make_int2((int)(uint32_t)(x >> FIX_LO), (int)((uint32_t)x & ((1u << FIX_LO) - 1)) - (1 << (FIX_LO - 1)));
+  const unsigned long long t = ((((unsigned long long)mh << 32) | l) << (S_BITS - 53)) >> n;
+  return (long long)(t ^ (unsigned long long)((long long)(int)h >> 31));
 }
-
+// the magnitude of a fixed-point value's upper word
+__device__ __forceinline__ uint32_t abs_up(long long x) { return (uint32_t)abs((int)(x >> 32)); }
 // the FP64 star at slot s of one column (bricks with non-finite or tiny values)
 __device__ __noinline__ double star64(const Step64& a, const double* in, int64_t ld, int64_t s) {
   const int64_t brick = s >> 9;
@@ -123,15 +142,211 @@ __device__ __noinline__ double star64(const Step64& a, const double* in, int64_t
   return acc;
 }
 
+// the same window of 60 bits, S_FINE bits lower: modulo 2^60
+__device__ __forceinline__ long long fix60_low(double v, int e) {
+  const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
+  const int n = e - (int)((h >> 20) & 0x7ff) - S_FINE;
+  const unsigned long long m = (((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32) | l) << (S_BITS - 53);
+  const unsigned long long t = (n < 0 ? m << -n : m >> min(n, 63)) ^ (unsigned long long)((long long)(int)h >> 31);
+  return (long long)(t << (64 - S_BITS)) >> (64 - S_BITS);
+}
+// a sum in units of 2^(E - S_BITS - S_FINE), |sum| < 2^119: its leading 63 bits; ku: the value
+// of a unit of 2^(E - S_BITS)
+__device__ __forceinline__ double sum_value(__int128 sum, double ku) {
+  if (sum == 0) return 0.0;
+  const unsigned __int128 m = sum < 0 ? -(unsigned __int128)sum : (unsigned __int128)sum;
+  const unsigned long long mh = (unsigned long long)(m >> 64);
+  const int z = mh ? __clzll((long long)mh) : 64 + __clzll((long long)(unsigned long long)m);
+  const double r = (double)(long long)((unsigned long long)((m << z) >> 64) >> 1);   // in [2^62, 2^63]
+  const double scale = __longlong_as_double(__double_as_longlong(ku) + ((long long)(65 - z - S_FINE) << 52));
+  return sum < 0 ? -(r * scale) : r * scale;
+}
+
+// The FP64 star by eight lanes, one for each arm and one for the point itself; all lanes of the
+// warp call it
+__device__ __forceinline__ double star64_lanes(const Step64& a, const double* in, int64_t ld, int64_t s) {
+  const int f = threadIdx.x & 7;
+  double t = 0.0;
+  if (f < 6) {
+    const int li = (int)(s & 511), sh = 3 * (f >> 1), l = (li >> sh) & 7, room = (f & 1) ? 7 - l : l;
+    const int st = (f & 1) ? 1 << sh : -(1 << sh), nb = __ldg(a.nbr + (s >> 9) * 6 + f);
+    const int64_t out = (int64_t)nb * 512 + li - 8 * st;
+    double v[6];
+#pragma unroll
+    for (int k = 1; k <= 6; k++)
+      v[k - 1] = k <= room ? __ldg(in + (s + k * st) * ld) : nb >= 0 ? __ldg(in + (out + k * st) * ld) : 0.0;
+#pragma unroll
+    for (int k = 6; k >= 1; k--) t = fma(a.st[k], v[k - 1], t);
+  } else if (f == 6) {
+    t = 3.0 * a.st[0] * __ldg(in + s * ld);
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
+// the star's constant times 2^(e - 1022 - S_BITS)
+__device__ __forceinline__ double unit_value(const Step64& a, int e) {
+  return a.ku * __hiloint2double((e - 1022 - S_BITS + 1023) << 20, 0);
+}
+
+// The thread's vector of the brick from slot b0 and of its halos to fixed point: N rows 64 rows
+// apart from row r0, to N points dstep apart
+template <typename F>
+__device__ __forceinline__ void stage_brick(long long* fx, const double* inc, int64_t ld, int64_t b0, const int (&nb)[6],
+                                            bool on, int e, F fix) {
+  const int v = threadIdx.x & 3, p = threadIdx.x >> 2, px = p & 7, py = p >> 3;
+  auto stage = [&](auto n_c, bool use, int64_t r0, int dst, int dstep) {
+    constexpr int N = decltype(n_c)::value;
+    const double* src = inc + r0 * ld;
+    double h[N];
+#pragma unroll
+    for (int q = 0; q < N; q++) h[q] = use ? __ldg(src + q * 64 * ld) : 0.0;
+#pragma unroll
+    for (int q = 0; q < N; q++) fx[(dst + q * dstep) * S_NV + v] = fix(h[q], e);
+  };
+  using I8 = std::integral_constant<int, 8>;
+  using I6 = std::integral_constant<int, 6>;
+  stage(I8(), on, b0 + p, p, P_PLANE);
+  // x halos: px < 6 of every line; y halos: rows py < 6; planes z = 0..7
+  if (px < 6) {
+    stage(I8(), on && nb[0] >= 0, (int64_t)nb[0] * 512 + py * 8 + 2 + px, P_XL + py * 6 + px, P_PLANE);
+    stage(I8(), on && nb[1] >= 0, (int64_t)nb[1] * 512 + p, P_XH + py * 6 + px, P_PLANE);
+  }
+  if (py < 6) {
+    stage(I8(), on && nb[2] >= 0, (int64_t)nb[2] * 512 + (2 + py) * 8 + px, P_YL + p, P_PLANE);
+    stage(I8(), on && nb[3] >= 0, (int64_t)nb[3] * 512 + p, P_YH + p, P_PLANE);
+  }
+  stage(I6(), on && nb[4] >= 0, (int64_t)nb[4] * 512 + 128 + p, P_ZL + p, 64);
+  stage(I6(), on && nb[5] >= 0, (int64_t)nb[5] * 512 + p, P_ZH + p, 64);
+}
+
+// Byte offsets of the thread's point of plane 0 and of its neighbours along x and y (plane z is
+// P_PLANE points further)
+struct Arms {
+  uint32_t me, x[12], y[12];
+};
+__device__ __forceinline__ Arms arms() {
+  const int v = threadIdx.x & 3, p = threadIdx.x >> 2, px = p & 7, py = p >> 3;
+  auto off = [&](int pt) { return (uint32_t)(pt * S_NV + v) * 8u; };
+  Arms n;
+  n.me = off(p);
+#pragma unroll
+  for (int k = 1; k <= 6; k++) {
+    n.x[2 * k - 2] = off(px >= k ? p - k : P_XL + py * 6 + px - k + 6);
+    n.x[2 * k - 1] = off(px + k < 8 ? p + k : P_XH + py * 6 + px + k - 8);
+    n.y[2 * k - 2] = off(py >= k ? p - 8 * k : P_YL + (py - k + 6) * 8 + px);
+    n.y[2 * k - 1] = off(py + k < 8 ? p + 8 * k : P_YH + (py + k - 8) * 8 + px);
+  }
+  return n;
+}
+// The star at the thread's point of plane z: hi 2^32 + lo, from the upper words with the signed
+// weights and the lower words with their magnitudes in a positive (k odd) and a negative sum, one
+// 32 x 32 -> 64 product each.  Returns what stands at the point and next to it (S_STEEP).
+__device__ __forceinline__ uint32_t star60(const Step64& a, const long long* fx, const Arms& n, int z, long long& hi,
+                                           long long& lo) {
+  auto at = [&](uint32_t o, int imm) { return *(const long long*)((const char*)fx + o + imm); };
+  constexpr int PL = P_PLANE * S_NV * 8;   // bytes of a plane
+  auto zoff = [](int zz) {                 // plane zz, possibly in the z halos
+    return zz < 0 ? (P_ZL + (zz + 6) * 64) * S_NV * 8 : zz > 7 ? (P_ZH + (zz - 8) * 64) * S_NV * 8 : zz * PL;
+  };
+  const long long x0 = at(n.me, z * PL);
+  hi = (long long)a.wt[0] * (int)(x0 >> 32);
+  unsigned long long neg = (unsigned long long)a.wabs[0] * (uint32_t)x0, pos = 0;
+  uint32_t size = 0;
+#pragma unroll
+  for (int k = 1; k <= 6; k++) {
+    const long long xa = at(n.x[2 * k - 2], z * PL), xb = at(n.x[2 * k - 1], z * PL), ya = at(n.y[2 * k - 2], z * PL),
+                    yb = at(n.y[2 * k - 1], z * PL), za = at(n.me, zoff(z - k)), zb = at(n.me, zoff(z + k));
+    const long long x = (xa + xb + ya) + (yb + za + zb);
+    hi += (long long)a.wt[k] * (int)(x >> 32);
+    if (k & 1) pos += (unsigned long long)a.wabs[k] * (uint32_t)x;
+    else neg += (unsigned long long)a.wabs[k] * (uint32_t)x;
+    if (k == 1)
+      size = 5u * abs_up(x0) + (abs_up(xa) + abs_up(xb) + abs_up(ya)) + (abs_up(yb) + abs_up(za) + abs_up(zb));
+  }
+  lo = (long long)(pos - neg);
+  return size;
+}
+// the sum in units of 2^S_DROP, rounded
+__device__ __forceinline__ long long leading(long long hi, long long lo) {
+  return (hi << (32 - S_DROP)) + ((lo + (1ll << (S_DROP - 1))) >> S_DROP);
+}
+
+// Adds alpha times the star where the first pass left it out (`left`: planes of the thread's
+// point).  Called by all threads; apart from the kernel, whose registers it does not share.
+//   Few points: the FP64 star, four points a warp at a time.
+//   More: the whole brick once more in the window S_FINE bits lower, which gives the sum modulo
+// 2^60; the leading bits of the first pass, off by less than 2^58.2, give the rest.  Where that is
+// too coarse as well, the FP64 star.
+template <bool CM>
+__device__ __noinline__ void steep_points(const Step64& a, uint8_t* smb, int cell, int chunk, int e, uint32_t left,
+                                          int* s_max) {
+  long long* fx = (long long*)(smb + S_FIX);
+  int* count = (int*)(smb + S_LEFT);
+  uint16_t* list = (uint16_t*)(count + 1);   // point * S_NV + vector
+  const int64_t ld = CM ? S_NV : a.ld_in, b0 = (int64_t)cell * 512;
+  const int tid = threadIdx.x, v = tid & 3, p = tid >> 2;
+  const double* in = a.in + (int64_t)chunk * a.cs_in;
+  auto add = [&](int r, int vec, double t) {
+    double* o = a.out + (int64_t)chunk * a.cs_out + vec + (b0 + r) * a.ld_out;
+    t = fma(a.alpha, t, *o);
+    *o = t;
+    if (a.flag && abs_hw(t) >= 0x7ff00000u) atomicOr(a.flag, 1u);
+    if (a.emax_out) atomicMax(&s_max[vec], hw_exp(abs_hw(t)));
+  };
+#pragma unroll 1
+  for (uint32_t m = left; m; m &= m - 1) {
+    const int i = atomicAdd(count, 1);
+    if (i < S_FEW) list[i] = (uint16_t)(((__ffs(m) - 1) * 64 + p) * S_NV + v);
+  }
+  __syncthreads();
+  const int n = *count;
+  if (n <= S_FEW) {
+    for (int i0 = tid / 32 * 4; i0 < n; i0 += S_THR / 8) {
+      const int i = i0 + (tid & 31) / 8, item = list[min(i, n - 1)], vec = item & (S_NV - 1), r = item / S_NV;
+      const double t = star64_lanes(a, in + vec, ld, b0 + r);
+      if ((tid & 7) == 0 && i < n) add(r, vec, t);
+    }
+    return;
+  }
+  const Arms at = arms();
+  long long lead[8], hi, lo;
+#pragma unroll 1
+  for (uint32_t m = left; m; m &= m - 1) {
+    const int z = __ffs(m) - 1;
+    star60(a, fx, at, z, hi, lo);
+    lead[z] = leading(hi, lo);
+  }
+  __syncthreads();
+  int nb[6];
+#pragma unroll
+  for (int f = 0; f < 6; f++) nb[f] = __ldg(a.nbr + (int64_t)cell * 6 + f);
+  stage_brick(fx, in + v, ld, b0, nb, chunk * S_NV + v < a.w, e, [](double h, int ex) { return fix60_low(h, ex); });
+  __syncthreads();
+#pragma unroll 1
+  for (; left; left &= left - 1) {
+    const int z = __ffs(left) - 1;
+    double t;
+    if (star60(a, fx, at, z, hi, lo) < S_STEEP) {
+      t = star64(a, in + v, ld, b0 + z * 64 + p);
+    } else {
+      const __int128 low = ((__int128)hi << 32) + lo, rest = ((__int128)lead[z] << (S_DROP + S_FINE)) - low;
+      t = sum_value(low + ((rest + ((__int128)1 << (S_BITS - 1))) >> S_BITS << S_BITS), unit_value(a, e));
+    }
+    add(z * 64 + p, v, t);
+  }
+}
+
 // SMEM_KB: the bricks have at most KSCF_BRICK_ATOMS atoms with projectors (so that 16 bits hold
 // the number of an entry inside its brick), whose coefficients are staged in shared memory with
 // the first S_ENT entries
 static_assert(KSCF_BRICK_ATOMS * 512 < 65536, "entry numbers of a brick in 16 bits");
 // CM: `in` is chunk-major (ld_in = S_NV)
 template <bool SMEM_KB, bool CM>
-__global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
+__global__ void __launch_bounds__(S_THR, 2) step64_kernel(const __grid_constant__ Step64 a) {
   extern __shared__ __align__(16) uint8_t smb[];
-  int2* fx = (int2*)(smb + S_FIX);             // [point][4]
+  long long* fx = (long long*)(smb + S_FIX);   // [point][4]
   double* vs = (double*)(smb + S_V);           // [512]: V
   double* kbc = (double*)(smb + S_KBC);        // [atom][l][4]
   double* echi = (double*)(smb + S_CHI);       // [entry][4]
@@ -147,11 +362,11 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
   }
   const int64_t ld = CM ? S_NV : a.ld_in;
   const int tid = threadIdx.x, v = tid & 3, p = tid >> 2;   // p: the thread's point of every plane
-  const int px = p & 7, py = p >> 3;
   const int col = chunk * S_NV + v;
   const bool on = col < a.w;
   const int64_t b0 = (int64_t)cell * 512;
   if (tid < S_NV) s_max[tid] = 0;
+  if (tid == 0) *(int*)(smb + S_LEFT) = 0;
   int nb[6];
 #pragma unroll
   for (int f = 0; f < 6; f++) nb[f] = __ldg(a.nbr + (int64_t)cell * 6 + f);
@@ -181,37 +396,15 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
       *(double2*)(echi + 4 * t + 2) = __ldg((const double2*)(a.kb_chi + 4 * (e0 + t)) + 1);
     }
   }
-  const bool slow = __syncthreads_or(e >= 2046 || (e > 0 && e < 128));
   // a vector of zeros (some may be -0, one unit below): its star is zero
-  const double ku = e == 0 ? 0.0 : a.ku * fix_unit(e);
-  if (e == 0) e = 1023;
-  // ---- values to fixed point (S_BITS = FIX_BITS): N rows `step` rows apart from row r0, to N
-  // points dstep apart ----
-  if (!slow) {
-    auto stage = [&](auto n_c, bool use, int64_t r0, int dst, int dstep) {
-      constexpr int N = decltype(n_c)::value;
-      const double* src = inc + r0 * ld;
-      double h[N];
-#pragma unroll
-      for (int q = 0; q < N; q++) h[q] = use ? __ldg(src + q * 64 * ld) : 0.0;
-#pragma unroll
-      for (int q = 0; q < N; q++) fx[(dst + q * dstep) * S_NV + v] = fix57(h[q], e);
-    };
-    using I8 = std::integral_constant<int, 8>;
-    using I6 = std::integral_constant<int, 6>;
-    stage(I8(), on, b0 + p, p, P_PLANE);
-    // x halos: px < 6 of every line; y halos: rows py < 6; planes z = 0..7
-    if (px < 6) {
-      stage(I8(), on && nb[0] >= 0, (int64_t)nb[0] * 512 + py * 8 + 2 + px, P_XL + py * 6 + px, P_PLANE);
-      stage(I8(), on && nb[1] >= 0, (int64_t)nb[1] * 512 + p, P_XH + py * 6 + px, P_PLANE);
-    }
-    if (py < 6) {
-      stage(I8(), on && nb[2] >= 0, (int64_t)nb[2] * 512 + (2 + py) * 8 + px, P_YL + p, P_PLANE);
-      stage(I8(), on && nb[3] >= 0, (int64_t)nb[3] * 512 + p, P_YH + p, P_PLANE);
-    }
-    stage(I6(), on && nb[4] >= 0, (int64_t)nb[4] * 512 + 128 + p, P_ZL + p, 64);
-    stage(I6(), on && nb[5] >= 0, (int64_t)nb[5] * 512 + p, P_ZH + p, 64);
-  }
+  const bool zero = e == 0;
+  // the value of a unit of the sum (used when not slow); the FP64 star also where it is not well
+  // inside the normal numbers
+  const double ku = unit_value(a, e);
+  const bool slow = __syncthreads_or(!zero && (e >= 2046 || e < 256 || (int)(abs_hw(ku) >> 20) < 200));
+  if (zero) e = 1023;
+  const double ku_d = zero ? 0.0 : ku * (double)(1 << S_DROP);
+  if (!slow) stage_brick(fx, inc, ld, b0, nb, on, e, [](double h, int ex) { return fix60(h, ex); });
   // ---- the point's own value, prev and mask of all planes, before the first store (plain loads
   // of prev: it may be the output) ----
   double yv[8], pv[8];
@@ -228,22 +421,11 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
       pv[z] = use && a.prev ? prevc[z * 64 * a.ld_prev] : 0.0;
     }
   }
-  // neighbour points of plane 0 along x and y (byte offsets; plane z is P_PLANE points further)
-  uint32_t xo[12], yo[12];
-  auto off = [&](int pt) { return (uint32_t)(pt * S_NV + v) * 8u; };
-#pragma unroll
-  for (int k = 1; k <= 6; k++) {
-    xo[2 * k - 2] = off(px >= k ? p - k : P_XL + py * 6 + px - k + 6);
-    xo[2 * k - 1] = off(px + k < 8 ? p + k : P_XH + py * 6 + px + k - 8);
-    yo[2 * k - 2] = off(py >= k ? p - 8 * k : P_YL + (py - k + 6) * 8 + px);
-    yo[2 * k - 1] = off(py + k < 8 ? p + 8 * k : P_YH + (py + k - 8) * 8 + px);
-  }
-  const uint32_t me = off(p);
+  const Arms at = arms();
   __syncthreads();   // the fixed-point values, V and the KB tables are visible
-  uint32_t mx = 0;
+  uint32_t mx = 0, left = 0;   // left: planes of points that steep_points adds the star to
   double* outc = a.out + (int64_t)chunk * a.cs_out + v + (b0 + p) * a.ld_out;
-  const char* fb = (const char*)fx;
-  constexpr int PL = P_PLANE * S_NV * 8;   // bytes of a plane
+  const uint32_t limit = zero ? 0u : S_STEEP;
 #pragma unroll
   for (int z = 0; z < 8; z++) {
     if (!((live >> z) & 1u)) {
@@ -252,24 +434,17 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
     }
     const int r = z * 64 + p;
     double t;
+    bool steep = false;
     if (slow) {
       t = star64(a, inc, ld, b0 + r);
     } else {
-      auto at = [&](uint32_t o, int imm) { return *(const int2*)(fb + o + imm); };
-      // plane zz, possibly in the z halos (compile time)
-      auto zoff = [](int zz) {
-        return zz < 0 ? (P_ZL + (zz + 6) * 64) * S_NV * 8 : zz > 7 ? (P_ZH + (zz - 8) * 64) * S_NV * 8 : zz * PL;
-      };
-      FixAcc s = {0, 0};
-      fix_mad(s, a.wt[0], at(me, z * PL));
-#pragma unroll
-      for (int k = 1; k <= 6; k++) {
-        const int2 xa = at(xo[2 * k - 2], z * PL), xb = at(xo[2 * k - 1], z * PL), ya = at(yo[2 * k - 2], z * PL),
-                   yb = at(yo[2 * k - 1], z * PL), za = at(me, zoff(z - k)), zb = at(me, zoff(z + k));
-        fix_mad(s, a.wt[k], make_int2((xa.x + xb.x + ya.x) + (yb.x + za.x + zb.x),
-                                      (xa.y + xb.y + ya.y) + (yb.y + za.y + zb.y)));
+      long long hi, lo;
+      steep = star60(a, fx, at, z, hi, lo) < limit;
+      t = ku_d * (double)leading(hi, lo);
+      if (steep) {   // without its star for now
+        t = 0.0;
+        left |= 1u << z;
       }
-      t = ku * (double)((s.hi << (FIX_LO - S_DROP)) + (s.lo >> S_DROP));
     }
     t = fma(vs[r], yv[z], t);
     if (SMEM_KB) {
@@ -304,8 +479,9 @@ __global__ void __launch_bounds__(S_THR, 2) step64_kernel(Step64 a) {
     }
     t = fma(a.beta, pv[z], a.alpha * fma(-a.c, yv[z], t));
     outc[z * 64 * a.ld_out] = t;
-    mx = max(mx, abs_hw(t));
+    mx = max(mx, steep ? 0u : abs_hw(t));
   }
+  if (__syncthreads_or(left != 0)) steep_points<CM>(a, smb, cell, chunk, e, left, s_max);
   if (a.flag && mx >= 0x7ff00000u) atomicOr(a.flag, 1u);
   if (a.emax_out) {
     // lanes of the same vector are 4 apart
@@ -376,12 +552,13 @@ constexpr int kFixW[6] = {1425600, -222750, 44000, -7425, 864, -50};
 
 // The star's one floating-point constant is -1 / (2 h^2 831600 m); its rounding error would be a
 // systematic relative error of the kinetic energy in every step.  The weights may be taken any
-// m <= S_MULT times: the m whose constant is closest to a double.
+// S_MULT/2 < m <= S_MULT times: the m whose constant is closest to a double (a smaller m has
+// the error of twice its value).
 int weight_multiple(double h, double* ku) {
   const double hh = h * h, hl = std::fma(h, h, -hh);   // h^2 = hh + hl exactly
-  int best = 1;
+  int best = S_MULT;
   double err = 1.0;
-  for (int m = 1; m <= S_MULT; m++) {
+  for (int m = S_MULT / 2 + 1; m <= S_MULT; m++) {
     const double d = 2.0 * FIX_DEN * m, p = d * hh, pl = std::fma(d, hh, -p) + d * hl, u = 1.0 / p;
     const double q = u * p, r = std::fabs(((1.0 - q) - std::fma(u, p, -q)) - u * pl);   // |1 - u d h^2|
     if (r < err) {
@@ -398,8 +575,8 @@ int weight_multiple(double h, double* ku) {
 bool step64_available(const Ham& H) { return H.grid.B == 8 && H.n_cells == H.grid.n_bricks && H.n_cells > 0; }
 
 // A single application also needs the exponents' pass: measured, us, this path | FP64 star:
-// 4,169 points x 8 60 | 49, x 32 64 | 64, 45,025 x 1 79 | 66, x 4 80 | 87, x 32 129 | 222,
-// 97,569 x 1 90 | 82, x 4 91 | 119
+// 4,169 points x 8 39 | 29, x 32 43 | 43, 8,925 x 16 40 | 44, 45,025 x 1 50 | 37, x 2 50 | 44, x 4 50 | 50 (three
+// launches of 12 us and more each), 97,569 x 1 54 | 46
 bool step64_wanted(const Ham& H, int w) { return step64_available(H) && (double)H.grid.n_points * w >= 1.5e5; }
 
 size_t step64_emax_bytes(const Ham& H, int w) { return kscf_align256((size_t)H.grid.n_bricks * emax_ld(w) * 4); }
@@ -454,9 +631,9 @@ cudaError_t launch_step64(const Ham& H, const double* in, int64_t ld_in, const d
   a.beta = beta;
   a.c = c;
   const int m = weight_multiple(H.grid.h, &a.ku);
-  a.ku *= (double)(1 << S_DROP);
   a.wt[0] = m * FIX_W0;
   for (int k = 1; k <= 6; k++) a.wt[k] = m * kFixW[k - 1];
+  for (int k = 0; k <= 6; k++) a.wabs[k] = (uint32_t)std::abs(a.wt[k]);
   a.coef = coef;
   a.cld = cld;
   a.V = H.d_v64;
