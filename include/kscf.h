@@ -230,11 +230,11 @@ int kscf_hamiltonian_apply_noalloc(const kscf_ham* ham, void* Y, int64_t ld_y, v
  * (0 = all k); the result does not depend on block.  F32 on bricks of 8^3 or 16^3: each
  * block runs as two halves of whole 16-column chunks, the second on a stream the call
  * creates and releases; both halves are ordered after the work already on `stream`, and
- * the work enqueued on `stream` after the call waits for both.  F64 on bricks of 8^3: the
- * 37-point star of every point is an exact sum of integers (or the FP64 star, where the values
- * around a point are too far below the largest of the brick and its neighbours); it is within
- * 24 units of 2^-53 of sum |w y| over the star's own points, like an FP64 star.  The same
- * holds for kscf_hamiltonian_apply from 1.5e5 values (points times columns) on. */
+ * the work enqueued on `stream` after the call waits for both.  F64 on bricks of 8^3: from
+ * some 5e4 values (points times columns) on, the 37-point star of every point is an exact sum
+ * of integers (or the FP64 star, where the values around a point are too far below the largest
+ * of the brick and its neighbours); it is within 24 units of 2^-53 of sum |w y| over the star's
+ * own points, like an FP64 star.  The same holds for kscf_hamiltonian_apply from 1.5e5 on. */
 int kscf_chebyshev_filter(const kscf_ham* ham, void* X, int64_t ld, int k, int degree,
                           double a, double b, double a0, int dtype, int block,
                           void* work, size_t work_bytes, void* stream);

@@ -569,6 +569,7 @@ extern "C" int kscf_chebyshev_filter(const kscf_ham* ham, void* X, int64_t ld, i
   void* buf = cv.take((size_t)H.grid.n_slots * wpad * es);
   void* coef = cv.take((size_t)std::max(H.n_kb, 1) * 4 * wpad * es);
   KSCF_CUDA_TRY(launch_zero_rows(H, X, ld, k, dtype, st));
+  int ws = 0;   // columns per part of the FP64 step in fixed point, 0: the FP64 star
   if (dtype == KSCF_F64 && step64_available(H)) {
     // the buffer of one slot-major copy holds two chunk-major copies of about half the columns
     // and their exponents; the last step writes into the caller's block
@@ -578,10 +579,12 @@ extern "C" int kscf_chebyshev_filter(const kscf_ham* ham, void* X, int64_t ld, i
       const int n4 = (n + 3) / 4 * 4;
       return 2 * kscf_align256((size_t)H.grid.n_slots * n4 * 8) + 2 * step64_emax_bytes(H, n4);
     };
-    int ws = half;
+    ws = half;
     while (ws > 4 && need(ws) > room) ws -= 4;
     const int parts = (w + ws - 1) / ws;
-    ws = ((w + parts - 1) / parts + 3) / 4 * 4;   // even parts
+    ws = step64_filter_wanted(H, w, parts) ? ((w + parts - 1) / parts + 3) / 4 * 4 : 0;   // even parts
+  }
+  if (ws > 0) {
     Carver cb(buf);
     double* A = (double*)cb.take((size_t)H.grid.n_slots * ws * 8);
     double* B = (double*)cb.take((size_t)H.grid.n_slots * ws * 8);

@@ -579,6 +579,16 @@ bool step64_available(const Ham& H) { return H.grid.B == 8 && H.n_cells == H.gri
 // launches of 12 us and more each), 97,569 x 1 54 | 46
 bool step64_wanted(const Ham& H, int w) { return step64_available(H) && (double)H.grid.n_points * w >= 1.5e5; }
 
+// A filter's block goes through in `parts`, one after the other, each with a gather and a step per
+// degree that a small grid does not fill.  Measured, us per degree: this path 31 for every part + 4e-5 for
+// every value (points x columns), the FP64 star 25 + 1.1e-4.  Whole filters of 10 degrees, this path | FP64
+// star: 4,169 points x 8 (1 part) 323 | 260, x 32 (3) 963 | 404, x 100 (2) 841 | 717; 8,925 x 8 (1) 327 | 324, x 48
+// (2) 755 | 709; 17,557 x 8 (1) 329 | 419, x 24 (2) 730 | 723, x 36 (2) 815 | 961, x 32 (3) 1043 | 858, x 64 (3)
+// 1299 | 1491; 33,401 x 1 (1) 344 | 302, x 28 (3) 1175 | 1317; 45,025 x 128 (3) 3453 | 7094
+bool step64_filter_wanted(const Ham& H, int w, int parts) {
+  return step64_available(H) && 30.0 * parts - 26.0 < 7.5e-5 * (double)H.grid.n_points * w;
+}
+
 size_t step64_emax_bytes(const Ham& H, int w) { return kscf_align256((size_t)H.grid.n_bricks * emax_ld(w) * 4); }
 
 cudaError_t launch_emax64(const Ham& H, const double* X, int64_t ld, int w, int* emax, cudaStream_t st) {

@@ -126,6 +126,7 @@ cudaError_t launch_cheb_step(const Ham& H, const void* in, int64_t ld_in, const 
 // ---- FP64 step on 8^3 bricks in fixed point (filter_f64.cu) ----
 bool step64_available(const Ham& H);
 bool step64_wanted(const Ham& H, int w);   // for a single application to w columns
+bool step64_filter_wanted(const Ham& H, int w, int parts);   // for a filter of w columns in so many parts
 // emax tables (exponents per brick and vector) of w columns
 size_t step64_emax_bytes(const Ham& H, int w);
 cudaError_t launch_emax64(const Ham& H, const double* X, int64_t ld, int w, int* emax, cudaStream_t st);
