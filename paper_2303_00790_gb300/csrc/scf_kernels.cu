@@ -13,6 +13,7 @@
 
 #include <algorithm>
 
+#include "cg_offsets.cuh"
 #include "fixlap.cuh"
 #include "fp64.cuh"
 #include "kscf_internal.h"
@@ -380,38 +381,32 @@ __device__ __forceinline__ double scale_pow2(double v, int k) {
 __device__ __forceinline__ double hw_bound(uint32_t hw) { return __hiloint2double((int)min(hw + 1, 0x7ff00000u), 0); }
 __device__ __forceinline__ uint32_t abs_hw(double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; }
 
-// Byte offsets (in the fixed-point field) of the face neighbours of slot s: nb[2 ax + sg] +-
-// 8 k stride is the slot at distance k beyond the brick's face.  A missing brick points into
-// the zeros behind the field (kCgZeroSlots), so that the star needs no predicates; 32-bit
-// offsets from one base keep the address arithmetic out of the loads.  The base is a brick before
-// the field (cg_base), so that no offset is negative (that of a high neighbour starts below the
-// neighbour's first slot).
+// The fixed-point field's base for the offsets of cg_offsets.cuh
 template <int B>
 __device__ __forceinline__ const char* cg_base(const int2* rf) {
   return (const char*)(rf - B * B * B);
 }
-template <int B>
-__device__ __forceinline__ void cg_faces(const int32_t* nbr, int s, uint32_t zero, uint32_t* nb) {
+// Face neighbours of slot s: nb[2 ax + sg] +- 8 k stride is the slot at distance k beyond the
+// brick's face; a missing brick points into the zeros behind the field (kCgZeroSlots), so that
+// the star needs no predicates.
+template <int B, typename O>
+__device__ __forceinline__ void cg_faces(const int32_t* nbr, int s, O zero, O* nb) {
   constexpr int B3 = B * B * B;
   const int brick = s / B3, li = s - brick * B3;
-  const int stride[3] = {1, B, B * B};
 #pragma unroll
-  for (int f = 0; f < 6; f++) {
-    const int n = __ldg(nbr + brick * 6 + f);
-    nb[f] = n >= 0 ? 8u * (uint32_t)((n + 1) * B3 + li + ((f & 1) ? -B : B) * stride[f >> 1]) : zero + 8u * B3;
-  }
+  for (int f = 0; f < 6; f++) nb[f] = cg_face<O, B>(__ldg(nbr + (int64_t)brick * 6 + f), li, f, zero);
 }
 
 // 831600 h^2 Lap_h of the fixed-point field (f: its cg_base) at slot s
-template <int B>
-__device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* nb, int nbs) {
+template <int B, typename O>
+__device__ __forceinline__ FixAcc cg_star(const char* f, int s, const O* nb, int nbs) {
   const int li = s & (B * B * B - 1);
   const int l[3] = {li % B, (li / B) % B, li / (B * B)};
   const int stride[3] = {1, B, B * B};
-  const uint32_t own = 8u * (uint32_t)(s + B * B * B);
+  const O own = cg_own<O, B>(s);
   FixAcc acc = {0, 0};
   fix_mad(acc, FIX_W0, *(const int2*)(f + own));
-  uint32_t face[6];
+  O face[6];
 #pragma unroll
   for (int q = 0; q < 6; q++) face[q] = nb[q * nbs];
 #pragma unroll
@@ -419,7 +414,7 @@ __device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* 
     int2 v[6];
 #pragma unroll
     for (int ax = 0; ax < 3; ax++) {
-      const uint32_t lo = l[ax] >= k ? own : face[2 * ax], hi = l[ax] + k < B ? own : face[2 * ax + 1];
+      const O lo = l[ax] >= k ? own : face[2 * ax], hi = l[ax] + k < B ? own : face[2 * ax + 1];
       v[2 * ax] = *(const int2*)(f + (size_t)lo - 8 * k * stride[ax]);
       v[2 * ax + 1] = *(const int2*)(f + (size_t)hi + 8 * k * stride[ax]);
     }
@@ -429,8 +424,10 @@ __device__ __forceinline__ FixAcc cg_star(const char* f, int s, const uint32_t* 
   return acc;
 }
 
-template <int B, int NPT>
+// O: type of the offsets into the field
+template <int B, int NPT, typename O = uint32_t>
 __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
+  static_assert(NPT == 0 || sizeof(O) == 4, "the vectors of a large field are not in registers");
   extern __shared__ uint32_t s_face[];   // NPT > 0: [6][NPT][threads] face neighbours of the points
   __shared__ double sh[kCgThreads / 32];
   __shared__ uint32_t shm[kCgThreads / 32];
@@ -445,7 +442,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
   uint32_t* max_q = c.hmax;
   uint32_t* max_r = c.hmax + P;
   unsigned target = 0;
-  const uint32_t zero = 8u * (uint32_t)(c.a.n + kCgZeroSlots / 2);
+  const O zero = cg_zero<O>(c.a.n, kCgZeroSlots);
   constexpr int NR = NPT > 0 ? NPT : 1;
   int sv[NR];
   double xv[NR], rv[NR], pv[NR], qv[NR];
@@ -470,10 +467,10 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
       const int64_t i = i0 + tid + (int64_t)k * nt;
       const bool on = i < i1;
       sv[k] = on ? c.live[i] : (int)(zero / 8);
-      uint32_t nb[6];
+      O nb[6];
       if (on) cg_faces<B>(c.a.nbr, sv[k], zero, nb);
 #pragma unroll
-      for (int q = 0; q < 6; q++) s_face[(q * NPT + k) * nt + tid] = on ? nb[q] : zero + 8u * (B * B * B);
+      for (int q = 0; q < 6; q++) s_face[(q * NPT + k) * nt + tid] = on ? nb[q] : zero + 8 * (B * B * B);
       xv[k] = on ? c.x[sv[k]] : 0.0;
       rv[k] = on ? c.r[sv[k]] : 0.0;
       pv[k] = on && !c.first ? c.p[sv[k]] : 0.0;
@@ -522,7 +519,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) cg_kernel(CgArgs c) {
       if constexpr (NPT > 0) {
         t = cg_star<B>(cg_base<B>(c.rf), s, s_face + k * nt + tid, NPT * nt);
       } else {
-        uint32_t nb[6];
+        O nb[6];
         cg_faces<B>(c.a.nbr, s, zero, nb);
         t = cg_star<B>(cg_base<B>(c.rf), s, nb, 1);
       }
@@ -603,10 +600,12 @@ static cudaError_t cg_launch(CgArgs& c, int P, cudaStream_t st) {
   int nt = npt <= 4 ? (int)(((per + npt - 1) / npt + 31) / 32 * 32) : kCgThreads;
   nt = std::max(nt, 128);
   const int smem = npt <= 4 ? 6 * npt * nt * (int)sizeof(int) : 0;
+  const bool wide = cg_wide(c.a.n, kCgZeroSlots, B);
   const void* k = npt == 1   ? (const void*)cg_kernel<B, 1>
                   : npt == 2 ? (const void*)cg_kernel<B, 2>
                   : npt == 3 ? (const void*)cg_kernel<B, 3>
                   : npt == 4 ? (const void*)cg_kernel<B, 4>
+                  : wide     ? (const void*)cg_kernel<B, 0, uint64_t>
                              : (const void*)cg_kernel<B, 0>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
