@@ -319,7 +319,8 @@ int kscf_random_subspace(const kscf_ham* ham, void* X, int64_t ld, int k, int dt
  *   native mode out must not overlap A.
  * Work buffers: kscf_gemm_workspace_size(op = 0 gram / 1 rotate, rows, m|kin, n|kout,
  * dtype, mode, &bytes).  In the native mode a Gram needs none and a rotation kin * kout
- * elements; FP64 products use the rest of the reported size for the tensor cores. */
+ * elements; FP64 products use the rest of the reported size for the tensor cores (about 1 GiB
+ * of digits at a time, whatever the rows, and 14 bytes for each element of Q). */
 int kscf_gram(const void* A, int64_t lda, const void* B, int64_t ldb, int64_t rows, int m, int n, int dtype,
               int mode, double scale, double* C, int64_t ldc, void* work, size_t work_bytes, void* stream);
 int kscf_rotate(const void* A, int64_t lda, const double* Q, int64_t ldq, int64_t rows, int kin, int kout,

@@ -20,7 +20,7 @@
 // runs at ~1 TFLOP/s (2 k^3 / 3 flop in total: 0.41 ms at k = 850), but the chain through the
 // block rows is longer: 5,400 cycles to load the tiles, 19,000 for the triangular solve, 12,000
 // for the next diagonal tile's update, 49,000 for its 32 pivots and 2,200 per grid barrier (it
-// was 110,000 together with 61,000 for the pivots and 5,400 per barrier: k = 850 1.42 -> 1.11 ms).
+// was 110,000 together with 61,000 for the pivots and 5,400 per barrier: k = 850 1.42 -> 1.15 ms).
 //
 // A pivot counts as failed when it is not above tau_c = S_cc * max((c + 8) u64, floor_rel)
 // (or is not finite): (c + 8) u64 S_cc is the rounding level of a Cholesky pivot, so an

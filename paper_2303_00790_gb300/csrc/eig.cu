@@ -16,9 +16,9 @@
 //     Sorensen (1987) and the eigenvector formula of Gu & Eisenstat (1995).  The
 //     recursion tree is balanced (node t of depth d covers [t n / 2^d, (t+1) n / 2^d))
 //     with leaves of one row; every depth is a batch of independent merges.  Each
-//     secular-equation root is solved by one warp with a two-pole rational model of
-//     the secular function (the "middle way" of R.-C. Li, 1994) safeguarded by
-//     bisection; roots are kept as an offset from their nearer pole.  The merged
+//     secular-equation root is solved by one warp (four lanes in merges of at most 32 rows)
+//     with a two-pole rational model of the secular function (the "middle way" of R.-C. Li,
+//     1994) safeguarded by bisection; roots are kept as an offset from their nearer pole.  The merged
 //     eigenvectors are diag(Q1, Q2) M, two FP64 GEMMs per merge.
 //  3. Back-transformation Z = Q_H Z_T, column-parallel: each CTA holds a few columns of
 //     Z_T in shared memory and applies the reflectors from the last to the first.
@@ -27,8 +27,10 @@
 // dependent operation to the next, 111 with a shuffle between them), so every stage is written
 // to keep all four FP64 pipes busy and to keep the dependent chains (reductions, square roots,
 // reciprocals) short: reciprocals and reciprocal square roots start from an FP32 seed, and sums
-// over a warp are formed in integers.  All waits
-// are bounded; a wait that gives up sets a status word that the host reports.
+// over a warp are formed in integers.  The grid's
+// barrier waits are bounded; a wait that gives up sets a status word that the host reports.  The
+// cluster variant waits on the hardware's cluster barrier, which has no limit and needs none: its
+// eight CTAs are scheduled together and all reach every barrier.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -18,7 +18,7 @@
 // star when a CTA has few of them, else from a second pass in a window 29 bits lower (a sum modulo
 // 2^60, which the first pass's leading bits complete), and the FP64 star below 2^-36 of 2^E.  Measured
 // against quadruple precision, error / (2^-53 sum |w v|) over fields exp(-r/2) .. exp(-4 r),
-// Gaussians, waves and noise: rms 0.06-0.77 (FP64 star 0.22-0.94), largest 0.8-5.4 (0.9-5.4); filters of 8 to
+// Gaussians, waves and noise: rms 0.06-0.77 (FP64 star 0.22-0.94), largest 0.9-5.4 (0.9-5.4); filters of 8 to
 // 12 steps with the recurrence's scalars as given: 1.3e-16 of a column's norm (FP64 star, whose
 // seven weights are rounded, 6.0e-16 to 8.8e-16; the scalars' own rounding moves a result by 1e-15).
 //

@@ -628,9 +628,10 @@ cudaError_t col_max(const double* X, int64_t ld, int64_t rows, int nc, const int
 
 }  // namespace
 
-// Where the lines lie (measured, us, this path | CUDA-core kernels): Gram 4,169 rows x 8 columns
-// 44 | 899, 45,025 x 16 90 | 1087, 234,489 x 2 282 | 2078 -- everywhere, since the CUDA-core
-// kernel walks at least 1024 rows in one FP64 chain; shorter ones stay there.  Rotation 45,025
+// Where the lines lie (measured, us, this path | CUDA-core kernels): Gram 128 rows x 1 column 43 | 141,
+// 128 x 100 53 | 144, 512 x 8 44 | 546, 4,169 x 8 44 | 899, 45,025 x 16 90 | 1087, 234,489 x 2 282 | 2078
+// -- everywhere, since the CUDA-core kernel walks up to 1024 rows in one FP64 chain; less than a tile of
+// 128 rows stays there (100 rows: 122).  Rotation 45,025
 // rows x 16 107 | 88, x 24 116 | 168, 4,169 x 32 61 | 41, x 100 69 | 127, 234,489 x 8 362 | 405.
 bool gram_f64tc_wanted(int64_t rows) { return rows >= 128 && rows <= F_ROWS_MAX; }
 bool rotate_f64tc_wanted(int64_t rows, int kin, int kout) {
