@@ -227,7 +227,8 @@ int kscf_hamiltonian_apply_noalloc(const kscf_ham* ham, void* Y, int64_t ld_y, v
  *   Y_j = (2 sigma_j/e)(H Y_{j-1} - c Y_{j-1}) - sigma_{j-1} sigma_j Y_{j-2},
  *   sigma_j = 1/(tau - sigma_{j-1}),  j = 2..m;   X <- Y_m.
  * Requires a0 < a < b, degree >= 1.  Columns are processed `block` at a time
- * (0 = all k); the result does not depend on block.  F32 on bricks of 8^3 or 16^3: each
+ * (0 = all k); the result depends on block by rounding only (the order of the projections'
+ * sums and, in F64, the way the star is evaluated are chosen by the width).  F32 on bricks of 8^3 or 16^3: each
  * block runs as two halves of whole 16-column chunks, the second on a stream the call
  * creates and releases; both halves are ordered after the work already on `stream`, and
  * the work enqueued on `stream` after the call waits for both.  F64 on bricks of 8^3: from
