@@ -228,10 +228,10 @@ int kscf_hamiltonian_apply_noalloc(const kscf_ham* ham, void* Y, int64_t ld_y, v
  *   sigma_j = 1/(tau - sigma_{j-1}),  j = 2..m;   X <- Y_m.
  * Requires a0 < a < b, degree >= 1.  Columns are processed `block` at a time
  * (0 = all k); the result depends on block by rounding only (the order of the projections'
- * sums and, in F64, the way the star is evaluated are chosen by the width).  F32 on bricks of 8^3 or 16^3: each
- * block runs as two halves of whole 16-column chunks, the second on a stream the call
- * creates and releases; both halves are ordered after the work already on `stream`, and
- * the work enqueued on `stream` after the call waits for both.  F64 on bricks of 8^3: from
+ * sums and, in F64, the way the star is evaluated are chosen by the width).  F32 on bricks
+ * of 8^3 or 16^3: each block runs as two halves of whole 16-column chunks, the second on a
+ * stream the call creates and releases; both halves are ordered after the work already on
+ * `stream`, and the work enqueued on `stream` after the call waits for both.  F64 on bricks of 8^3: from
  * some 5e4 values (points times columns) on, the 37-point star of every point is an exact sum
  * of integers (or the FP64 star, where the values around a point are too far below the largest
  * of the brick and its neighbours); it is within 24 units of 2^-53 of sum |w y| over the star's
