@@ -27,8 +27,10 @@
 // values per point that two CTAs per SM hide half.  One degree step of 234,489 points x 850 vectors:
 // 8.4 ms (gather 1.1 ms beside it) against 23.5 ms of the FP64 star; whole 12-step filter 295 -> 114 ms.
 // Two limbs of 29 bits and no second look at small values took 102 ms, 105 ms 60 bits alone; a value of 1e-3
-// of 2^E then had 47 bits, orbitals exp(-r) lost three digits in their tails.  Orbitals exp(-r/2), exp(-r)
-// and exp(-2 r) about 200 centres (most CTAs make the second pass): 40, 59, 63 ms, FP64 star 70.
+// of 2^E then had 47 bits, orbitals exp(-r) lost three digits in their tails.  What the small values'
+// stars cost depends on the block: the orbitals of a self-consistent run, whose tails fill the shell
+// outside the cluster, take 145 ms (with 64 or 512 for S_FEW 153 and 143); 200 orbitals exp(-r/2), exp(-r)
+// or exp(-2 r) about as many centres, where most CTAs make the second pass, 40, 59 and 63 ms, FP64 star 70.
 // Also built: the small values' stars one by one by the warp that meets them (120 to 137 ms: code that few
 // warps run is fetched when it runs, and it shared the hot loop's registers), the 13-point sums as three
 // line passes over register windows as in the FP32 filter, and 512 threads with half the planes each.
